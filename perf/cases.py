@@ -66,7 +66,7 @@ def listed():
         _case("batch64_fp8_10m", n_ads=10_000_000, dtype="fp8e4m3", fields=32, vocab=15,
               zipf=1.0, pairs=128, k=2000, batch=64),
         # a full serving wave: K and targeting bitmap per request
-        _case("wave128_bf16_5m", n_ads=5_000_000, dtype="bf16", fields=32, pairs=128, k=1000,
+        _case("wave128_bf16_5m", n_ads=5_000_000, dtype="bf16", fields=32, pairs=128, k=2000,
               batch=128, mixed_k=True, filter=True),
         # the periodic rebuild of the index, up to the first scores it gives
         _case("build_fp32_2m", op="build", n_ads=2_000_000),
