@@ -1,17 +1,28 @@
 // Index construction (Algorithm 1, Sec. 3.4) on the GPU.
 //
-// Step 1 (Block Grouping): every (k, v) pair becomes the 64-bit word
-// k << 32 | v, so sorting the words orders them by (k, h = v >> 8, l = v & 255);
-// dropping repeated words turns each run of equal (k, h) into the set B[k, h].
+// Step 1 (Block Grouping): every (k, v) pair becomes the word (h, k, l) with
+// h = v >> 8 and l = v & 255, packed into as few bits as the key space and
+// the inventory need; sorting the words puts each set B[k, h] in one run, and
+// all runs of one window h = 256 consecutive ads side by side (repeated words
+// are dropped, when there are any).
 // Step 2 (Logarithmic Categorization): a run of n ads is one block of group
 // g = ceil(log2 n), padded with zero bytes to 2^g slots.
 // Step 3 (Storage Layout): per group, header[g] (h of each block) and
 // values[g] (the low bytes) in (k, h) order, and keys[g], the row pointer
 // giving each key's first block (keys[g][k] = group-g blocks with key < k).
 //
+// The words are sorted window-major because two of the three layouts the
+// queries read follow the windows: one CTA per window finds its blocks and
+// counts them (k_windows<false>), the counts are scanned, and a second walk
+// (k_windows<true>) writes the window-major view; the key-major arrays then
+// come from a stable sort of the blocks, half as many as the words, by
+// (g, k) alone.  Measured, 2 M ads with 16 keys each (32 M pairs, 15 M
+// blocks): 2.7 ms of device time for all of it, against 8.0 ms when
+// the words were sorted key-major by 7 three-kernel passes and the blocks
+// again by 8 passes into the window order.
+//
 // The radix sort, the duplicate removal and the prefix sums are this
-// library's own device primitives (ebr_prims.cuh); the grouping and storage
-// steps are the kernels below.
+// library's own device primitives (ebr_prims.cuh).
 
 #include <cstring>
 #include <vector>
@@ -26,149 +37,266 @@ int launch_quantize_rows_fp8(const float *x, uint64_t n, uint32_t d, uint8_t *q,
 
 namespace {
 
-__global__ void k_pack(const uint32_t *__restrict__ key, const uint32_t *__restrict__ ad,
-                       uint64_t nnz, uint32_t n_keys, uint32_t n_ads,
-                       uint64_t *__restrict__ out, uint32_t *__restrict__ flags) {
-  uint32_t bad = 0;
-  for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < nnz;
-       i += (uint64_t)gridDim.x * blockDim.x) {
-    uint32_t k = key[i], a = ad[i];
-    if (k >= n_keys) { bad |= DEVERR_BAD_BUILD_KEY; k = 0; }
-    if (a >= n_ads) { bad |= DEVERR_BAD_AD; a = 0; }
-    out[i] = ((uint64_t)k << 32) | a;
+// The (h, k, l) word of pair i (see above); kb: bits of a key.  Out-of-range
+// keys and ads are flagged and read as 0.
+struct PairLoad {
+  const uint32_t *key, *ad;
+  uint32_t n_keys, n_ads;
+  int kb;
+  uint32_t *flags;
+  __device__ __forceinline__ uint64_t operator()(uint64_t i) const {
+    uint32_t k = __ldg(key + i), a = __ldg(ad + i);
+    if (k >= n_keys || a >= n_ads) {
+      atomicOr(flags, (k >= n_keys ? DEVERR_BAD_BUILD_KEY : 0u) |
+                          (a >= n_ads ? DEVERR_BAD_AD : 0u));
+      k = k >= n_keys ? 0u : k;
+      a = a >= n_ads ? 0u : a;
+    }
+    return ((uint64_t)(a >> 8) << (kb + 8)) | ((uint64_t)k << 8) | (a & 255u);
   }
-  if (bad) atomicOr(flags, bad);
-}
+};
 
-// keys per ad over the distinct (key, ad) pairs, and their maximum
-__global__ void k_keys_per_ad(const uint64_t *__restrict__ x, uint32_t m, uint32_t *__restrict__ cnt) {
-  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < m; i += gridDim.x * blockDim.x)
-    atomicAdd(&cnt[(uint32_t)x[i]], 1u);
-}
-__global__ void k_u32_to_u16(const uint32_t *__restrict__ v, uint32_t n, uint16_t *__restrict__ out) {
-  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
-    out[i] = (uint16_t)v[i];
-}
-__global__ void k_max_u32(const uint32_t *__restrict__ v, uint32_t n, unsigned int *__restrict__ out) {
-  uint32_t mx = 0;
-  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
-    mx = max(mx, v[i]);
-  atomicMax(out, mx);
-}
-
-// bs[i] = 1 where a new (k, h) run starts in the sorted, duplicate-free words.
-__global__ void k_block_flags(const uint64_t *__restrict__ x, uint32_t m,
-                              uint32_t *__restrict__ bs) {
-  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < m; i += gridDim.x * blockDim.x)
-    bs[i] = (i == 0 || (x[i] >> 8) != (x[i - 1] >> 8)) ? 1u : 0u;
-}
-
-// start[b] = first word of block b; start[nb] = m.
-__global__ void k_block_start(const uint32_t *__restrict__ bs, const uint32_t *__restrict__ bid,
-                              uint32_t m, uint32_t *__restrict__ start) {
+// win_start[h] = first word of window h (n_win + 1 entries) of the sorted
+// words, and the number of words equal to the one before them.
+__global__ void k_window_starts(const uint64_t *__restrict__ x, uint32_t m, int wshift,
+                                uint32_t n_win, uint32_t *__restrict__ win_start,
+                                uint32_t *__restrict__ n_dup) {
+  uint32_t dup = 0;
   for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < m; i += gridDim.x * blockDim.x) {
-    if (bs[i]) start[bid[i] - 1] = i;
-    if (i == m - 1) start[bid[i]] = m;
+    const uint64_t a = __ldg(x + i);
+    const uint32_t h = (uint32_t)(a >> wshift);
+    uint32_t from = 0;
+    if (i) {
+      const uint64_t p = __ldg(x + i - 1);
+      dup += p == a ? 1u : 0u;
+      from = (uint32_t)(p >> wshift) + 1u;
+    }
+    for (uint32_t w = from; w <= h; w++) win_start[w] = i;
+    if (i == m - 1)
+      for (uint32_t w = h + 1; w <= n_win; w++) win_start[w] = m;
   }
+  dup = __reduce_add_sync(0xffffffffu, dup);
+  if ((threadIdx.x & 31) == 0 && dup) atomicAdd(n_dup, dup);
 }
 
 __device__ __forceinline__ uint32_t ceil_log2(uint32_t n) {
   return n <= 1 ? 0u : 32u - __clz(n - 1);
 }
 
-// Per block: group, and counts per (group, key) and per group.
-__global__ void k_block_info(const uint64_t *__restrict__ x, const uint32_t *__restrict__ start,
-                             uint32_t nb, uint32_t n_keys, uint8_t *__restrict__ grp,
-                             uint32_t *__restrict__ key_cnt /* [9][n_keys+1] */,
-                             unsigned long long *__restrict__ gcount) {
-  __shared__ unsigned int s_cnt[kGroups];
-  if (threadIdx.x < kGroups) s_cnt[threadIdx.x] = 0;
-  __syncthreads();
-  for (uint32_t b = blockIdx.x * blockDim.x + threadIdx.x; b < nb; b += gridDim.x * blockDim.x) {
-    uint32_t n = start[b + 1] - start[b];
-    uint32_t g = ceil_log2(n);
-    uint32_t k = (uint32_t)(x[start[b]] >> 32);
-    grp[b] = (uint8_t)g;
-    atomicAdd(&key_cnt[(uint64_t)g * (n_keys + 1) + k], 1u);
-    atomicAdd(&s_cnt[g], 1u);
-  }
-  __syncthreads();
-  if (threadIdx.x < kGroups && s_cnt[threadIdx.x])
-    atomicAdd(&gcount[threadIdx.x], (unsigned long long)s_cnt[threadIdx.x]);
-}
+constexpr int kWinThreads = 256, kWinWarps = kWinThreads / 32;
+constexpr uint32_t kWinChunk = 4096;  // words walked at a time; a block has at most 256
+constexpr uint32_t kWinRows = kWinChunk / kWinThreads;
 
-__global__ void k_iota(uint32_t *__restrict__ p, uint32_t n) {
-  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
-    p[i] = i;
-}
-
-struct EmitArgs {
-  uint32_t *header[kGroups];
-  uint8_t *values[kGroups];
-  unsigned long long gstart[kGroups + 1];
+struct WinArgs {
+  const uint64_t *x;            // sorted distinct words
+  const uint32_t *win_start;    // [n_win + 1]
+  const uint32_t *n_dup;        // repeated words found (then nothing is walked)
+  uint32_t n_win, n_ads;
+  int kb;
+  // counts (first walk)
+  uint32_t *gcnt;               // [9][n_win + 1] blocks of each group and window
+  uint16_t *ad_nkeys;           // [n_ads]
+  uint32_t *max_keys;           // most keys of one ad
+  // layout (second walk)
+  const uint32_t *win_ptr[kGroups];
+  uint32_t gstart[kGroups + 1];  // blocks of the groups before g
+  uint32_t *wkey[kGroups];
+  uint8_t *wvals[kGroups];
+  uint32_t *bh;                 // [blocks] window of each block, in (g, h, k) order
+  void *skey;                   // [blocks] (g, k) of each block, in that order
+  uint32_t *sval;               // [blocks] its place in that order
 };
 
-// Blocks sorted (stably) by group: position p - gstart[g] is the block's rank
-// inside its group, which preserves the (k, h) order.
-__global__ void k_emit(const uint64_t *__restrict__ x, const uint32_t *__restrict__ start,
-                       const uint32_t *__restrict__ perm, const uint8_t *__restrict__ grp_sorted,
-                       uint32_t nb, EmitArgs args) {
-  for (uint32_t p = blockIdx.x * blockDim.x + threadIdx.x; p < nb; p += gridDim.x * blockDim.x) {
-    uint32_t b = perm[p];
-    uint32_t g = grp_sorted[p];
-    uint64_t rank = p - args.gstart[g];
-    uint32_t s0 = start[b], n = start[b + 1] - s0;
-    args.header[g][rank] = (uint32_t)((x[s0] >> 8) & 0xFFFFFFu);
-    uint8_t *dst = args.values[g] + (rank << g);
-    for (uint32_t s = 0; s < n; s++) dst[s] = (uint8_t)(x[s0 + s] & 255u);
+// One CTA walks one window's words, kWinChunk at a time.  EMIT = false: blocks
+// per group and keys per ad.  EMIT = true: the window's part of the
+// window-major view, and the sort records of its blocks.  Bound by the read
+// of the words (EMIT = false) and by the byte stores of the values (true).
+// K: type of a sort record, (g << kb) | k.
+template <bool EMIT, typename K>
+__global__ void __launch_bounds__(kWinThreads) k_windows(const __grid_constant__ WinArgs a) {
+  __shared__ uint32_t s_mask[kWinChunk / 32 + 9];   // block heads of the chunk and 288 words on
+  __shared__ uint32_t s_adcnt[256];
+  __shared__ uint32_t s_g[kWinWarps][16];           // blocks per group: warp counts, then prefixes
+  __shared__ uint32_t s_run[16];                    // blocks of each group in the chunks before
+  __shared__ uint32_t s_blk[EMIT ? kWinChunk : 1];  // at a head: group << 16 | rank in its warp
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  if (*a.n_dup) return;  // blocks are sets; the caller drops the repeated words first
+  for (uint32_t w = blockIdx.x; w < a.n_win; w += gridDim.x) {
+    const uint32_t b0 = a.win_start[w], b1 = a.win_start[w + 1];
+    s_adcnt[tid] = 0;
+    if (tid < 16) s_run[tid] = 0;
+    uint32_t c0 = b0;
+    while (c0 < b1) {
+      __syncthreads();
+      if (tid < 16)
+        for (int q = 0; q < kWinWarps; q++) s_g[q][tid] = 0;
+      // head bits of words [c0, c0 + chunk + 288); the end counts as a head
+      for (uint32_t i = tid; i < kWinChunk + 288u; i += kWinThreads) {
+        const uint32_t p = c0 + i;
+        bool head = p == b1;
+        if (p < b1) head = i == 0 || (__ldg(a.x + p) >> 8) != (__ldg(a.x + p - 1) >> 8);
+        const uint32_t m = __ballot_sync(0xffffffffu, head);
+        if (lane == 0) s_mask[i >> 5] = m;
+      }
+      __syncthreads();
+      // the chunk ends at the window's end, or at its last head so that no
+      // block is cut (words beyond it are walked in the next chunk)
+      uint32_t end = b1 - c0;
+      if (end > kWinChunk) {
+        end = kWinChunk;
+        while (!((s_mask[end >> 5] >> (end & 31u)) & 1u)) end--;
+      }
+      // a warp owns kWinRows rows of 32 consecutive words
+      const uint32_t r0 = warp * 32 * kWinRows + lane;
+#pragma unroll 4
+      for (uint32_t r = 0; r < kWinRows; r++) {
+        const uint32_t i = r0 + 32 * r;
+        const bool in = i < end;
+        const bool head = in && ((s_mask[i >> 5] >> lane) & 1u);
+        uint32_t g = 15u;
+        if (head) {  // next head: the block's length
+          uint32_t wd = i >> 5;
+          uint32_t m = s_mask[wd] & (0xFFFFFFFEu << lane);
+          while (!m) m = s_mask[++wd];
+          g = ceil_log2((wd << 5) + __ffs(m) - 1u - i);
+        }
+        const uint32_t peers = __match_any_sync(0xffffffffu, g);
+        const int leader = __ffs(peers) - 1;
+        uint32_t old = 0;
+        if (lane == leader && g < 15u) {
+          old = s_g[warp][g];
+          s_g[warp][g] = old + __popc(peers);
+        }
+        __syncwarp();
+        if (EMIT) {
+          old = __shfl_sync(0xffffffffu, old, leader);
+          if (head) s_blk[i] = (g << 16) | (old + __popc(peers & ((1u << lane) - 1u)));
+        } else if (in) {
+          atomicAdd(&s_adcnt[(uint32_t)__ldg(a.x + c0 + i) & 255u], 1u);
+        }
+      }
+      __syncthreads();
+      if (tid < kGroups) {  // exclusive over the warps, from the chunks before
+        uint32_t acc = s_run[tid];
+        for (int q = 0; q < kWinWarps; q++) {
+          const uint32_t c = s_g[q][tid];
+          s_g[q][tid] = acc;
+          acc += c;
+        }
+        s_run[tid] = acc;
+      }
+      __syncthreads();
+      if (EMIT) {
+#pragma unroll 4
+        for (uint32_t r = 0; r < kWinRows; r++) {
+          const uint32_t i = r0 + 32 * r;
+          if (i >= end) continue;
+          const uint64_t word = __ldg(a.x + c0 + i);
+          // this word's block starts at the last head at or before it
+          uint32_t wd = i >> 5;
+          uint32_t m = s_mask[wd] & (0xFFFFFFFFu >> (31 - lane));
+          while (!m) m = s_mask[--wd];
+          const uint32_t hp = (wd << 5) + 31u - __clz(m);
+          const uint32_t e = s_blk[hp], g = e >> 16;
+          const uint32_t rank =
+              a.win_ptr[g][w] + s_g[hp / (32 * kWinRows)][g] + (e & 0xFFFFu);
+          a.wvals[g][((uint64_t)rank << g) + (i - hp)] = (uint8_t)word;
+          if (hp == i) {
+            const uint32_t key = (uint32_t)((word >> 8) & ((1ull << a.kb) - 1ull));
+            const uint32_t q = a.gstart[g] + rank;
+            a.wkey[g][rank] = key;
+            a.bh[q] = w;
+            reinterpret_cast<K *>(a.skey)[q] = ((K)g << a.kb) | (K)key;
+            a.sval[q] = q;
+          }
+        }
+      }
+      c0 += end;
+    }
+    if (!EMIT) {
+      __syncthreads();
+      if (tid < kGroups) a.gcnt[(uint64_t)tid * (a.n_win + 1) + w] = s_run[tid];
+      const uint32_t ad = w * 256u + tid, c = s_adcnt[tid];
+      if (ad < a.n_ads) a.ad_nkeys[ad] = (uint16_t)c;
+      const uint32_t mx = __reduce_max_sync(0xffffffffu, c);
+      if (lane == 0 && mx) atomicMax(a.max_keys, mx);
+    }
+    __syncthreads();
   }
 }
 
-// Window-major view of the same blocks: sort key (g, h, k) per block, with the
-// block's position in the group-sorted order as payload.
-__global__ void k_wm_keys(const uint64_t *__restrict__ x, const uint32_t *__restrict__ start,
-                          const uint32_t *__restrict__ perm, const uint8_t *__restrict__ grp_sorted,
-                          uint32_t nb, uint64_t *__restrict__ skey, uint32_t *__restrict__ sval) {
+// win_ptr[g][h] (per group) from the scan over all groups' counts, and the
+// totals per group (gc, 9 words).
+__global__ void k_win_ptrs(const uint32_t *__restrict__ scan, uint32_t n_win,
+                           uint32_t *__restrict__ win_ptr, uint32_t *__restrict__ gc) {
+  const uint32_t g = blockIdx.y;
+  const uint64_t row = (uint64_t)g * (n_win + 1);
+  const uint32_t base = scan[row];
+  for (uint32_t h = blockIdx.x * blockDim.x + threadIdx.x; h <= n_win;
+       h += gridDim.x * blockDim.x) {
+    const uint32_t v = scan[row + h] - base;
+    win_ptr[row + h] = v;
+    if (h == n_win) gc[g] = v;
+  }
+}
+
+struct KeyArgs {
+  const uint32_t *bh;
+  const uint8_t *wvals[kGroups];
+  uint32_t *header[kGroups];
+  uint8_t *values[kGroups];
+  uint32_t gstart[kGroups + 1];
+  int kb;
+};
+
+// p-th block in (g, k, h) order: its header and its 2^g value bytes, from its
+// place q in the window-major view.
+template <typename K>
+__global__ void k_key_major(const K *__restrict__ skey, const uint32_t *__restrict__ sval,
+                            uint32_t nb, const __grid_constant__ KeyArgs a) {
   for (uint32_t p = blockIdx.x * blockDim.x + threadIdx.x; p < nb; p += gridDim.x * blockDim.x) {
-    const uint64_t w0 = x[start[perm[p]]];
-    const uint64_t h = (w0 >> 8) & 0xFFFFFFull, k = w0 >> 32;
-    skey[p] = ((uint64_t)grp_sorted[p] << 56) | (h << 32) | k;
-    sval[p] = p;
+    const uint32_t g = (uint32_t)(skey[p] >> a.kb), q = sval[p];
+    const uint64_t rank = p - a.gstart[g], src = q - a.gstart[g];
+    a.header[g][rank] = __ldg(a.bh + q);
+    const uint8_t *from = a.wvals[g] + (src << g);
+    uint8_t *to = a.values[g] + (rank << g);
+    if (g >= 4) {
+      for (uint32_t s = 0; s < (1u << g); s += 16)
+        *reinterpret_cast<uint4 *>(to + s) = __ldg(reinterpret_cast<const uint4 *>(from + s));
+    } else if (g == 3) {
+      *reinterpret_cast<uint2 *>(to) = __ldg(reinterpret_cast<const uint2 *>(from));
+    } else if (g == 2) {
+      *reinterpret_cast<uint32_t *>(to) = __ldg(reinterpret_cast<const uint32_t *>(from));
+    } else if (g == 1) {
+      *reinterpret_cast<uint16_t *>(to) = __ldg(reinterpret_cast<const uint16_t *>(from));
+    } else {
+      *to = __ldg(from);
+    }
+  }
+}
+
+// keys[g][k] = group-g blocks with key < k: a binary search of (g, k) in the
+// sorted records.
+template <typename K>
+__global__ void k_row_ptrs(const K *__restrict__ skey, const __grid_constant__ KeyArgs a,
+                           uint32_t n_keys, uint32_t *__restrict__ keys) {
+  const uint32_t g = blockIdx.y;
+  for (uint64_t k = blockIdx.x * blockDim.x + threadIdx.x; k <= n_keys;
+       k += gridDim.x * blockDim.x) {
+    uint32_t lo = a.gstart[g], hi = a.gstart[g + 1];
+    const K t = ((K)g << a.kb) + (K)k;  // k == n_keys: past the group's last key
+    if (k == n_keys) lo = hi;
+    while (lo < hi) {
+      const uint32_t mid = lo + (hi - lo) / 2;
+      if (skey[mid] < t) lo = mid + 1; else hi = mid;
+    }
+    keys[(uint64_t)g * ((uint64_t)n_keys + 1) + k] = lo - a.gstart[g];
   }
 }
 
 struct WinPtrs {
   const uint32_t *p[kGroups];
 };
-
-struct WmArgs {
-  const uint8_t *values[kGroups];
-  uint32_t *wkey[kGroups];
-  uint8_t *wvals[kGroups];
-  uint32_t *wcnt;  // [9][n_win + 1]
-  uint32_t n_win;
-  unsigned long long gstart[kGroups + 1];
-};
-
-// q-th block in (g, h, k) order: store its key and copy its 2^g value bytes.
-__global__ void k_wm_emit(const uint64_t *__restrict__ skey, const uint32_t *__restrict__ sval,
-                          uint32_t nb, WmArgs a) {
-  for (uint32_t q = blockIdx.x * blockDim.x + threadIdx.x; q < nb; q += gridDim.x * blockDim.x) {
-    const uint64_t sk = skey[q];
-    const uint32_t g = (uint32_t)(sk >> 56), h = (uint32_t)((sk >> 32) & 0xFFFFFFu);
-    const uint64_t rank = q - a.gstart[g], src = sval[q] - a.gstart[g];
-    a.wkey[g][rank] = (uint32_t)sk;
-    const uint8_t *from = a.values[g] + (src << g);
-    uint8_t *to = a.wvals[g] + (rank << g);
-    if (g >= 2) {
-      for (uint32_t s = 0; s < (1u << g); s += 4)
-        *reinterpret_cast<uint32_t *>(to + s) = *reinterpret_cast<const uint32_t *>(from + s);
-    } else {
-      for (uint32_t s = 0; s < (1u << g); s++) to[s] = from[s];
-    }
-    atomicAdd(&a.wcnt[(uint64_t)g * (a.n_win + 1) + h], 1u);
-  }
-}
 
 // Bytes a window's segments of the window-major view occupy once each segment
 // is widened to 16-byte boundaries (the staging size of the fused scan).
@@ -191,9 +319,14 @@ __global__ void k_win_bytes(WinPtrs wp, uint32_t n_win, unsigned int *out_max) {
     mc = max(mc, (uint32_t)min(chunks, (uint64_t)0xFFFFFFFFu));
     ms = max(ms, (uint32_t)min(slots, (uint64_t)0xFFFFFFFFu));
   }
-  atomicMax(out_max, mx);
-  atomicMax(out_max + 1, mc);
-  atomicMax(out_max + 2, ms);
+  mx = __reduce_max_sync(0xffffffffu, mx);
+  mc = __reduce_max_sync(0xffffffffu, mc);
+  ms = __reduce_max_sync(0xffffffffu, ms);
+  if ((threadIdx.x & 31) == 0) {
+    atomicMax(out_max, mx);
+    atomicMax(out_max + 1, mc);
+    atomicMax(out_max + 2, ms);
+  }
 }
 
 inline int grid_for(uint64_t n, int threads = 256, int cap = 1 << 16) {
@@ -210,23 +343,62 @@ inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
 using namespace ebr;
 
+// Bits that hold every value below n.
+static int bits_for(uint64_t n) {
+  int b = 0;
+  while (b < 64 && (1ull << b) < n) b++;
+  return b;
+}
+
+// True where a kernel can read p in place (device memory of this device).
+static bool on_device(const void *p, int device) {
+  cudaPointerAttributes at;
+  if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return at.type == cudaMemoryTypeDevice && at.device == device;
+}
+
+// The (g, k) sort of the blocks and the key-major arrays from it.
+template <typename K>
+static int build_key_major(ebr_index *ix, uint32_t nb, KeyArgs &ka, void *k0, void *k1, void *k2,
+                           uint32_t *v0, uint32_t *v1, uint32_t *v2, void *scratch,
+                           uint32_t *flags, cudaStream_t st) {
+  const K *sk = (const K *)k0;
+  const uint32_t *sv = v0;
+  if (nb) {
+    bool in_b = false;
+    EBR_TRY((prims::radix_sort<K, true>(prims::ArrayLoad<K>{(const K *)k0}, v0, (K *)k1, (K *)k2,
+                                        v1, v2, nb, ka.kb + 4, scratch, flags, &in_b, st)));
+    sk = (const K *)(in_b ? k2 : k1);
+    sv = in_b ? v2 : v1;
+    k_key_major<K><<<grid_for(nb), 256, 0, st>>>(sk, sv, nb, ka);
+    EBR_CUDA_TRY(cudaGetLastError());
+  }
+  k_row_ptrs<K><<<dim3(grid_for((uint64_t)ix->n_keys + 1), kGroups), 256, 0, st>>>(
+      sk, ka, ix->n_keys, (uint32_t *)ix->mem_keys.p);
+  EBR_CUDA_TRY(cudaGetLastError());
+  return EBR_OK;
+}
+
+// Device words the build reads back in one copy.
+struct BuildCounts {
+  uint32_t flags, n_dup, max_keys, gc[kGroups], win_max[3], m_unique;
+};
+
 static int build_impl(const ebr_index_desc *desc, ebr_index *ix, cudaStream_t st) {
   const uint64_t nnz = desc->nnz;
-  const uint32_t n_keys = desc->n_keys, n_ads = desc->n_ads;
-  DevBuf d_key, d_ad, w0, w1, tmp, bs, bid, start, grp, grp2, perm, perm2, cnt, gcount, flags;
-  DevBuf skey, skey2, sval, sval2, wcnt;
-  std::vector<DevBuf *> temps = {&d_key, &d_ad, &w0, &w1, &tmp, &bs, &bid, &start,
-                                 &grp, &grp2, &perm, &perm2, &cnt, &gcount, &flags,
-                                 &skey, &skey2, &sval, &sval2, &wcnt};
-  auto cleanup = [&]() {
-    for (auto *b : temps) dev_free(*b);
-  };
+  const uint32_t n_keys = desc->n_keys, n_ads = desc->n_ads, n_win = (n_ads + 255) / 256;
+  const int kb = bits_for(n_keys), hb = bits_for(n_win);
+  ix->n_win = n_win;
+  DevBuf in, pool, wpool, blocks;
   int rc = EBR_OK;
-  cudaEvent_t e0 = nullptr, e1 = nullptr;
+  cudaEvent_t ev[4] = {nullptr, nullptr, nullptr, nullptr};
 #define BTRY(expr)                  \
   do {                              \
     rc = (expr);                    \
-    if (rc != EBR_OK) goto fail;    \
+    if (rc != EBR_OK) goto done;    \
   } while (0)
 #define BCUDA(expr)                                                                       \
   do {                                                                                    \
@@ -234,248 +406,183 @@ static int build_impl(const ebr_index_desc *desc, ebr_index *ix, cudaStream_t st
     if (_e != cudaSuccess) {                                                              \
       set_error("%s: %s", #expr, cudaGetErrorString(_e));                                 \
       rc = EBR_ECUDA;                                                                     \
-      goto fail;                                                                          \
+      goto done;                                                                          \
     }                                                                                     \
   } while (0)
   {
-    uint64_t m_host = 0;
-    uint32_t nb = 0;
-    unsigned long long gc[kGroups] = {0};
-    uint32_t hflags = 0;
-    uint32_t *d_num = nullptr;
-    size_t need = 0;
     const uint32_t *pk = desc->post_key, *pa = desc->post_ad;
-    int end_bit = 32;
-    EmitArgs ea;
-    size_t hdr_off[kGroups], val_off[kGroups], hdr_total = 0, val_total = 0;
+    for (auto &e : ev) BCUDA(cudaEventCreate(&e));
+    // Inputs on the host are brought over first (not part of build_ms).
+    if (nnz && !(on_device(pk, ix->device) && on_device(pa, ix->device))) {
+      BTRY(dev_alloc(in, nnz * 8));
+      BCUDA(cudaMemcpyAsync(in.p, pk, nnz * 4, cudaMemcpyDefault, st));
+      BCUDA(cudaMemcpyAsync((uint32_t *)in.p + nnz, pa, nnz * 4, cudaMemcpyDefault, st));
+      pk = (const uint32_t *)in.p;
+      pa = pk + nnz;
+    }
+    // words and the sort's scratch in one allocation, per-window arrays in another
+    const size_t words_b = align_up(nnz * 8, 256);
+    const size_t scr_b = align_up(
+        std::max(prims::sort_scratch(nnz), (nnz + prims::scan_scratch(nnz) + 64) * 4), 256);
+    const size_t gw_b = align_up((size_t)kGroups * (n_win + 1) * 4, 256);
+    const size_t ws_b = align_up(((size_t)n_win + 1) * 4, 256);
+    const size_t st_b = align_up(prims::scan_scratch((uint64_t)kGroups * (n_win + 1)) * 4, 256);
+    BTRY(dev_alloc(pool, 2 * words_b + scr_b));
+    BTRY(dev_alloc(wpool, 256 + ws_b + gw_b + st_b));
+    BTRY(dev_alloc(ix->ad_nkeys, (size_t)n_ads * 2));
+    BTRY(dev_alloc(ix->mem_winptr, (size_t)kGroups * (n_win + 1) * 4));
+    uint64_t *wa = (uint64_t *)pool.p, *wb = (uint64_t *)((char *)pool.p + words_b);
+    void *scratch = (char *)pool.p + 2 * words_b;
+    BuildCounts *cnt = (BuildCounts *)wpool.p;
+    uint32_t *win_start = (uint32_t *)((char *)wpool.p + 256);
+    uint32_t *gcnt = (uint32_t *)((char *)wpool.p + 256 + ws_b);
+    uint32_t *stmp = (uint32_t *)((char *)wpool.p + 256 + ws_b + gw_b);
+    BuildCounts hc;
+    memset(&hc, 0, sizeof(hc));
+    uint32_t m = (uint32_t)nnz;
+    WinArgs w;
+    memset(&w, 0, sizeof(w));
+    w.win_start = win_start;
+    w.n_dup = &cnt->n_dup;
+    w.n_win = n_win;
+    w.n_ads = n_ads;
+    w.kb = kb;
+    w.gcnt = gcnt;
+    w.ad_nkeys = (uint16_t *)ix->ad_nkeys.p;
+    w.max_keys = &cnt->max_keys;
+    for (int g = 0; g < kGroups; g++) {
+      ix->win_ptr[g] = (uint32_t *)ix->mem_winptr.p + (size_t)g * (n_win + 1);
+      w.win_ptr[g] = ix->win_ptr[g];
+    }
 
-    BCUDA(cudaEventCreate(&e0));
-    BCUDA(cudaEventCreate(&e1));
-    // Inputs may live on the host: bring them over first (not part of build_ms).
+    BCUDA(cudaEventRecord(ev[0], st));
+    BCUDA(cudaMemsetAsync(wpool.p, 0, 256 + ws_b + gw_b, st));
     if (nnz) {
-      BTRY(dev_alloc(d_key, nnz * 4));
-      BTRY(dev_alloc(d_ad, nnz * 4));
-      BCUDA(cudaMemcpyAsync(d_key.p, pk, nnz * 4, cudaMemcpyDefault, st));
-      BCUDA(cudaMemcpyAsync(d_ad.p, pa, nnz * 4, cudaMemcpyDefault, st));
+      bool in_b = false;
+      BTRY((prims::radix_sort<uint64_t, false>(PairLoad{pk, pa, n_keys, n_ads, kb, &cnt->flags},
+                                               nullptr, wa, wb, nullptr, nullptr, nnz,
+                                               hb + kb + 8, scratch, &cnt->flags, &in_b, st)));
+      if (in_b) std::swap(wa, wb);  // wa: sorted
     }
-    BTRY(dev_alloc(w0, (nnz + 1) * 8));
-    BTRY(dev_alloc(w1, (nnz + 1) * 8));
-    BTRY(dev_alloc(flags, 64));
-    BTRY(dev_alloc(gcount, kGroups * 8));
-    BTRY(dev_alloc(cnt, (size_t)kGroups * (n_keys + 1) * 4));
-    BCUDA(cudaMemsetAsync(flags.p, 0, 64, st));
-    BCUDA(cudaMemsetAsync(gcount.p, 0, kGroups * 8, st));
-    BCUDA(cudaMemsetAsync(cnt.p, 0, (size_t)kGroups * (n_keys + 1) * 4, st));
-    BCUDA(cudaEventRecord(e0, st));
-    if (nnz) {
-      k_pack<<<grid_for(nnz), 256, 0, st>>>((const uint32_t *)d_key.p, (const uint32_t *)d_ad.p,
-                                            nnz, n_keys, n_ads, (uint64_t *)w0.p,
-                                            (uint32_t *)flags.p);
-      BCUDA(cudaGetLastError());
-    }
-    // key bits needed: 32 + ceil(log2 n_keys)
-    while (end_bit < 64 && ((uint64_t)1 << (end_bit - 32)) < n_keys) end_bit++;
-    {
-      // scratch of every primitive below: the sort's counts, the scans' tile
-      // sums, the unique's flags, and a word for the unique count
-      need = std::max<size_t>(prims::sort_scratch(nnz),
-                              (nnz + prims::scan_scratch(nnz) + 64) * 4);
-      need = std::max<size_t>(need, (prims::scan_scratch((uint64_t)n_keys + 1) + 64) * 4);
-      BTRY(dev_alloc(tmp, need + 256));
-      d_num = (uint32_t *)((char *)tmp.p + align_up(need, 16));
-      bool in_alt = false;
-      BTRY(prims::radix_sort<uint64_t>((uint64_t *)w0.p, (uint64_t *)w1.p, nullptr, nullptr, nnz,
-                                       end_bit, tmp.p, &in_alt, st));
-      uint64_t *sorted = in_alt ? (uint64_t *)w1.p : (uint64_t *)w0.p;
-      uint64_t *other = in_alt ? (uint64_t *)w0.p : (uint64_t *)w1.p;
-      uint32_t *uflags = (uint32_t *)tmp.p;
-      BTRY(prims::unique_sorted(sorted, other, nnz, uflags, uflags + nnz, d_num, st));
-      uint32_t m_i = 0;
-      BCUDA(cudaMemcpyAsync(&m_i, d_num, 4, cudaMemcpyDeviceToHost, st));
-      BCUDA(cudaMemcpyAsync(&hflags, flags.p, 4, cudaMemcpyDeviceToHost, st));
-      BCUDA(cudaStreamSynchronize(st));
-      if (hflags) {
-        rc = check_device_flags(hflags, "ebr_build_index");
-        goto fail;
-      }
-      m_host = (uint64_t)m_i;
-      // swap roles so that w0 holds the unique words
-      if (other != (uint64_t *)w0.p) std::swap(w0, w1);
-    }
-    const uint64_t *x = (const uint64_t *)w0.p;
-    const uint32_t m = (uint32_t)m_host;
-    ix->nnz_unique = m_host;
-    if (m > 0) {
-      // most keys any ad has (bounds the fused scan's exact accumulators)
-      BTRY(dev_alloc(bs, (size_t)std::max<uint64_t>(m, n_ads) * 4));
-      BCUDA(cudaMemsetAsync(bs.p, 0, (size_t)n_ads * 4, st));
-      BCUDA(cudaMemsetAsync(flags.p, 0, 4, st));
-      k_keys_per_ad<<<grid_for(m), 256, 0, st>>>(x, m, (uint32_t *)bs.p);
-      k_max_u32<<<grid_for(n_ads), 256, 0, st>>>((const uint32_t *)bs.p, n_ads,
-                                                (unsigned int *)flags.p);
-      BCUDA(cudaMemcpyAsync(&ix->max_keys_per_ad, flags.p, 4, cudaMemcpyDeviceToHost, st));
-      BCUDA(cudaStreamSynchronize(st));
-      if (ix->max_keys_per_ad <= 65535) {  // per-ad slot counts of the batched scan
-        BTRY(dev_alloc(ix->ad_nkeys, (size_t)n_ads * 2));
-        k_u32_to_u16<<<grid_for(n_ads), 256, 0, st>>>((const uint32_t *)bs.p, n_ads,
-                                                      (uint16_t *)ix->ad_nkeys.p);
+    // blocks and keys per window; taken again when repeated words turn up
+    for (int round = 0; round < 2; round++) {
+      w.x = wa;
+      if (m) {
+        k_window_starts<<<grid_for(m), 256, 0, st>>>(wa, m, kb + 8, n_win, win_start,
+                                                     &cnt->n_dup);
         BCUDA(cudaGetLastError());
-        BCUDA(cudaStreamSynchronize(st));
       }
-      dev_free(bs);
-      BTRY(dev_alloc(bs, (size_t)m * 4));
-      BTRY(dev_alloc(bid, (size_t)m * 4));
-      k_block_flags<<<grid_for(m), 256, 0, st>>>(x, m, (uint32_t *)bs.p);
+      k_windows<false, uint32_t><<<std::min<uint32_t>(n_win, 1u << 20), kWinThreads, 0, st>>>(w);
       BCUDA(cudaGetLastError());
-      BTRY((prims::scan<uint32_t, prims::AddU32, true>((const uint32_t *)bs.p, (uint32_t *)bid.p, m,
-                                                       prims::AddU32(), 0u, (uint32_t *)tmp.p,
-                                                       nullptr, st)));
-      BCUDA(cudaMemcpyAsync(&nb, (uint32_t *)bid.p + (m - 1), 4, cudaMemcpyDeviceToHost, st));
+      BTRY((prims::scan<uint32_t, prims::AddU32, false>(gcnt, gcnt, (uint64_t)kGroups * (n_win + 1),
+                                                        prims::AddU32(), 0u, stmp, nullptr, st)));
+      k_win_ptrs<<<dim3(grid_for((uint64_t)n_win + 1, 256, 256), kGroups), 256, 0, st>>>(
+          gcnt, n_win, (uint32_t *)ix->mem_winptr.p, cnt->gc);
+      BCUDA(cudaGetLastError());
+      WinPtrs wp;
+      for (int g = 0; g < kGroups; g++) wp.p[g] = ix->win_ptr[g];
+      k_win_bytes<<<grid_for(n_win), 256, 0, st>>>(wp, n_win, cnt->win_max);
+      BCUDA(cudaGetLastError());
+      BCUDA(cudaMemcpyAsync(&hc, cnt, sizeof(hc), cudaMemcpyDeviceToHost, st));
       BCUDA(cudaStreamSynchronize(st));
-      BTRY(dev_alloc(start, ((size_t)nb + 1) * 4));
-      k_block_start<<<grid_for(m), 256, 0, st>>>((const uint32_t *)bs.p,
-                                                 (const uint32_t *)bid.p, m,
-                                                 (uint32_t *)start.p);
-      BCUDA(cudaGetLastError());
-      BTRY(dev_alloc(grp, nb));
-      BTRY(dev_alloc(grp2, nb));
-      BTRY(dev_alloc(perm, (size_t)nb * 4));
-      BTRY(dev_alloc(perm2, (size_t)nb * 4));
-      k_block_info<<<grid_for(nb), 256, 0, st>>>(x, (const uint32_t *)start.p, nb, n_keys,
-                                                 (uint8_t *)grp.p, (uint32_t *)cnt.p,
-                                                 (unsigned long long *)gcount.p);
-      BCUDA(cudaGetLastError());
-      k_iota<<<grid_for(nb), 256, 0, st>>>((uint32_t *)perm.p, nb);
-      BCUDA(cudaGetLastError());
-      {
-        // blocks by size group, stably (one 8-bit pass: grp2 / perm2 hold the result)
-        bool alt = false;
-        BTRY(prims::radix_sort<uint8_t>((uint8_t *)grp.p, (uint8_t *)grp2.p, (uint32_t *)perm.p,
-                                        (uint32_t *)perm2.p, nb, 8, tmp.p, &alt, st));
-        if (!alt) {  // a single block: nothing moved
-          BCUDA(cudaMemcpyAsync(grp2.p, grp.p, nb, cudaMemcpyDeviceToDevice, st));
-          BCUDA(cudaMemcpyAsync(perm2.p, perm.p, (size_t)nb * 4, cudaMemcpyDeviceToDevice, st));
-        }
+      if (hc.flags) {
+        rc = check_device_flags(hc.flags, "ebr_build_index");
+        goto done;
       }
+      if (!hc.n_dup) break;
+      uint32_t *uflags = (uint32_t *)scratch;
+      BTRY(prims::unique_sorted(wa, wb, m, uflags, uflags + m, &cnt->m_unique, st));
+      std::swap(wa, wb);
+      m -= hc.n_dup;
+      BCUDA(cudaMemsetAsync(wpool.p, 0, 256 + ws_b + gw_b, st));
     }
-    // per-key row pointers: exclusive scan of counts over n_keys + 1 entries
-    BTRY(dev_alloc(ix->mem_keys, (size_t)kGroups * (n_keys + 1) * 4));
+    ix->nnz_unique = m;
+    ix->max_keys_per_ad = hc.max_keys;
+    ix->max_win_bytes = hc.win_max[0];
+    ix->max_win_chunks = hc.win_max[1];
+    ix->max_win_slots = hc.win_max[2];
+    if (m == 0 || ix->max_keys_per_ad > 65535) dev_free(ix->ad_nkeys);  // counts that do not fit
+
+    size_t hdr_off[kGroups], val_off[kGroups], hdr_total = 0, val_total = 0;
+    KeyArgs ka;
+    memset(&ka, 0, sizeof(ka));
+    ka.kb = kb;
     for (int g = 0; g < kGroups; g++) {
-      BTRY((prims::scan<uint32_t, prims::AddU32, false>(
-          (const uint32_t *)cnt.p + (size_t)g * (n_keys + 1),
-          (uint32_t *)ix->mem_keys.p + (size_t)g * (n_keys + 1), (uint64_t)n_keys + 1,
-          prims::AddU32(), 0u, (uint32_t *)tmp.p, nullptr, st)));
-      ix->keys[g] = (uint32_t *)ix->mem_keys.p + (size_t)g * (n_keys + 1);
-    }
-    BCUDA(cudaMemcpyAsync(gc, gcount.p, sizeof(gc), cudaMemcpyDeviceToHost, st));
-    BCUDA(cudaStreamSynchronize(st));
-    for (int g = 0; g < kGroups; g++) {
-      ix->n_blocks[g] = gc[g];
+      ix->n_blocks[g] = hc.gc[g];
       hdr_off[g] = hdr_total;
       val_off[g] = val_total;
-      hdr_total += align_up(gc[g] * 4, 256);
-      val_total += align_up(gc[g] << g, 256);
+      hdr_total += align_up((size_t)hc.gc[g] * 4, 256);
+      val_total += align_up((size_t)hc.gc[g] << g, 256);
+      ka.gstart[g + 1] = w.gstart[g + 1] = w.gstart[g] + hc.gc[g];
     }
+    const uint32_t nb = w.gstart[kGroups];
+    BTRY(dev_alloc(ix->mem_keys, (size_t)kGroups * ((size_t)n_keys + 1) * 4));
     BTRY(dev_alloc(ix->mem_header, hdr_total + 256));
     BTRY(dev_alloc(ix->mem_values, val_total + 256));
-    BCUDA(cudaMemsetAsync(ix->mem_values.p, 0, val_total + 256, st));
-    ea.gstart[0] = 0;
+    BTRY(dev_alloc(ix->mem_wkey, hdr_total + 256));
+    BTRY(dev_alloc(ix->mem_wvals, val_total + 256));
     for (int g = 0; g < kGroups; g++) {
+      ix->keys[g] = (uint32_t *)ix->mem_keys.p + (size_t)g * ((size_t)n_keys + 1);
       ix->header[g] = (uint32_t *)((char *)ix->mem_header.p + hdr_off[g]);
       ix->values[g] = (uint8_t *)ix->mem_values.p + val_off[g];
-      ea.header[g] = ix->header[g];
-      ea.values[g] = ix->values[g];
-      ea.gstart[g + 1] = ea.gstart[g] + gc[g];
+      ix->wkey[g] = (uint32_t *)((char *)ix->mem_wkey.p + hdr_off[g]);
+      ix->wvals[g] = (uint8_t *)ix->mem_wvals.p + val_off[g];
+      w.wkey[g] = ix->wkey[g];
+      w.wvals[g] = ix->wvals[g];
+      ka.header[g] = ix->header[g];
+      ka.values[g] = ix->values[g];
+      ka.wvals[g] = ix->wvals[g];
     }
+    // blocks: window of each, then (key, place) records three times over (the
+    // sort's input and its two buffers); the sort's scratch is the words'
+    const bool k32 = kb + 4 <= 32;
+    const size_t rk_b = align_up((size_t)nb * (k32 ? 4 : 8), 256), rv_b = align_up((size_t)nb * 4, 256);
+    const size_t bscr_b = align_up(prims::sort_scratch(nb), 256);
+    BTRY(dev_alloc(blocks, 4 * rv_b + 3 * rk_b + bscr_b));
+    char *bp = (char *)blocks.p;
+    w.bh = (uint32_t *)bp;
+    w.sval = (uint32_t *)(bp + rv_b);
+    uint32_t *v1 = (uint32_t *)(bp + 2 * rv_b), *v2 = (uint32_t *)(bp + 3 * rv_b);
+    w.skey = bp + 4 * rv_b;
+    void *k1 = bp + 4 * rv_b + rk_b, *k2 = bp + 4 * rv_b + 2 * rk_b;
+    void *bscr = bp + 4 * rv_b + 3 * rk_b;
+    ka.bh = w.bh;
+
+    BCUDA(cudaEventRecord(ev[1], st));
+    BCUDA(cudaMemsetAsync(ix->mem_wvals.p, 0, val_total + 256, st));
     if (nb) {
-      k_emit<<<grid_for(nb), 256, 0, st>>>(x, (const uint32_t *)start.p,
-                                           (const uint32_t *)perm2.p, (const uint8_t *)grp2.p,
-                                           nb, ea);
+      const uint32_t grid = std::min<uint32_t>(n_win, 1u << 20);
+      if (k32)
+        k_windows<true, uint32_t><<<grid, kWinThreads, 0, st>>>(w);
+      else
+        k_windows<true, uint64_t><<<grid, kWinThreads, 0, st>>>(w);
       BCUDA(cudaGetLastError());
     }
-    BCUDA(cudaEventRecord(e1, st));
-    BCUDA(cudaEventSynchronize(e1));
-    BCUDA(cudaEventElapsedTime(&ix->build_ms, e0, e1));
-
-    // ---- window-major view of the same blocks (for the fused dense scan)
-    {
-      const uint32_t n_win = (n_ads + 255) / 256;
-      ix->n_win = n_win;
-      BCUDA(cudaEventRecord(e0, st));
-      BTRY(dev_alloc(ix->mem_wkey, hdr_total + 256));
-      BTRY(dev_alloc(ix->mem_wvals, val_total + 256));
-      BTRY(dev_alloc(ix->mem_winptr, (size_t)kGroups * (n_win + 1) * 4));
-      BTRY(dev_alloc(wcnt, (size_t)kGroups * (n_win + 1) * 4));
-      BCUDA(cudaMemsetAsync(wcnt.p, 0, (size_t)kGroups * (n_win + 1) * 4, st));
-      WmArgs wa;
-      wa.wcnt = (uint32_t *)wcnt.p;
-      wa.n_win = n_win;
-      for (int g = 0; g < kGroups; g++) {
-        ix->wkey[g] = (uint32_t *)((char *)ix->mem_wkey.p + hdr_off[g]);
-        ix->wvals[g] = (uint8_t *)ix->mem_wvals.p + val_off[g];
-        ix->win_ptr[g] = (uint32_t *)ix->mem_winptr.p + (size_t)g * (n_win + 1);
-        wa.values[g] = ix->values[g];
-        wa.wkey[g] = ix->wkey[g];
-        wa.wvals[g] = ix->wvals[g];
-        wa.gstart[g] = ea.gstart[g];
-      }
-      wa.gstart[kGroups] = ea.gstart[kGroups];
-      if (nb) {
-        BTRY(dev_alloc(skey, (size_t)nb * 8));
-        BTRY(dev_alloc(skey2, (size_t)nb * 8));
-        BTRY(dev_alloc(sval, (size_t)nb * 4));
-        BTRY(dev_alloc(sval2, (size_t)nb * 4));
-        k_wm_keys<<<grid_for(nb), 256, 0, st>>>(x, (const uint32_t *)start.p,
-                                                (const uint32_t *)perm2.p,
-                                                (const uint8_t *)grp2.p, nb, (uint64_t *)skey.p,
-                                                (uint32_t *)sval.p);
-        BCUDA(cudaGetLastError());
-        BTRY(dev_reserve(tmp, std::max<size_t>(prims::sort_scratch(nb),
-                                               (prims::scan_scratch((uint64_t)n_win + 1) + 64) * 4) +
-                                  256));
-        bool alt = false;
-        BTRY(prims::radix_sort<uint64_t>((uint64_t *)skey.p, (uint64_t *)skey2.p,
-                                         (uint32_t *)sval.p, (uint32_t *)sval2.p, nb, 60, tmp.p,
-                                         &alt, st));
-        if (!alt) {  // the result ended in the first buffers
-          std::swap(skey, skey2);
-          std::swap(sval, sval2);
-        }
-        k_wm_emit<<<grid_for(nb), 256, 0, st>>>((const uint64_t *)skey2.p,
-                                                (const uint32_t *)sval2.p, nb, wa);
-        BCUDA(cudaGetLastError());
-      }
-      BTRY(dev_reserve(tmp, (prims::scan_scratch((uint64_t)n_win + 1) + 64) * 4 + 256));
-      for (int g = 0; g < kGroups; g++)
-        BTRY((prims::scan<uint32_t, prims::AddU32, false>(
-            (const uint32_t *)wcnt.p + (size_t)g * (n_win + 1), ix->win_ptr[g],
-            (uint64_t)n_win + 1, prims::AddU32(), 0u, (uint32_t *)tmp.p, nullptr, st)));
-      {
-        WinPtrs wp;
-        for (int g = 0; g < kGroups; g++) wp.p[g] = ix->win_ptr[g];
-        BCUDA(cudaMemsetAsync(flags.p, 0, 12, st));
-        k_win_bytes<<<grid_for(n_win), 256, 0, st>>>(wp, n_win, (unsigned int *)flags.p);
-        BCUDA(cudaGetLastError());
-        uint32_t mm[3] = {0, 0, 0};
-        BCUDA(cudaMemcpyAsync(mm, flags.p, 12, cudaMemcpyDeviceToHost, st));
-        BCUDA(cudaStreamSynchronize(st));
-        ix->max_win_bytes = mm[0];
-        ix->max_win_chunks = mm[1];
-        ix->max_win_slots = mm[2];
-      }
-      BCUDA(cudaEventRecord(e1, st));
-      BCUDA(cudaEventSynchronize(e1));
-      BCUDA(cudaEventElapsedTime(&ix->wm_build_ms, e0, e1));
+    BCUDA(cudaEventRecord(ev[2], st));
+    if (k32)
+      BTRY(build_key_major<uint32_t>(ix, nb, ka, w.skey, k1, k2, w.sval, v1, v2, bscr, &cnt->flags,
+                                     st));
+    else
+      BTRY(build_key_major<uint64_t>(ix, nb, ka, w.skey, k1, k2, w.sval, v1, v2, bscr, &cnt->flags,
+                                     st));
+    BCUDA(cudaEventRecord(ev[3], st));
+    BCUDA(cudaMemcpyAsync(&hc, cnt, sizeof(hc), cudaMemcpyDeviceToHost, st));
+    BCUDA(cudaStreamSynchronize(st));
+    if (hc.flags) {
+      rc = check_device_flags(hc.flags, "ebr_build_index");
+      goto done;
     }
+    // Algorithm 1 is everything but the walk that writes the window-major view
+    float a1 = 0.f, a2 = 0.f;
+    BCUDA(cudaEventElapsedTime(&a1, ev[0], ev[1]));
+    BCUDA(cudaEventElapsedTime(&ix->wm_build_ms, ev[1], ev[2]));
+    BCUDA(cudaEventElapsedTime(&a2, ev[2], ev[3]));
+    ix->build_ms = a1 + a2;
   }
-  cleanup();
-  cudaEventDestroy(e0);
-  cudaEventDestroy(e1);
-  return EBR_OK;
-fail:
-  cleanup();
-  if (e0) cudaEventDestroy(e0);
-  if (e1) cudaEventDestroy(e1);
+done:
+  for (DevBuf *b : {&in, &pool, &wpool, &blocks}) dev_free(*b);
+  for (auto &e : ev)
+    if (e) cudaEventDestroy(e);
   return rc;
 #undef BTRY
 #undef BCUDA
@@ -514,7 +621,7 @@ extern "C" void ebr_index_free(ebr_index *ix) {
   dev_free(ix->emb_q);
   dev_free(ix->emb_scale);
   Workspace &w = ix->ws;
-  for (DevBuf *b : {&w.wide, &w.w_dense, &w.lens, &w.scan, &w.work, &w.scan_tmp, &w.cand,
+  for (DevBuf *b : {&w.wide, &w.w_dense, &w.wq, &w.lens, &w.scan, &w.work, &w.scan_tmp, &w.cand,
                     &w.ctrl, &w.io_in, &w.io_out, &w.route_stats})
     dev_free(*b);
   batch_ws_free(ix->bws);
