@@ -302,6 +302,41 @@ __device__ __forceinline__ uint64_t hist_threshold(const uint32_t *hist_c, const
   return ((uint64_t)(((uint32_t)cb << 24) | ((uint32_t)fb << 16))) << 32;
 }
 
+// Candidate-score histogram shared by all CTAs (for a global K-th bound):
+// bins are the top 11 bits of the order-preserving score key (sign, 8
+// exponent bits, 2 mantissa bits).  CTAs count in shared memory and add
+// their counts to the global histogram every few windows.
+constexpr int kCandBins = 2048;
+constexpr int kBinShift = 53;
+
+// Largest bin edge b << kBinShift with at least K candidates at or above it,
+// scanning the global histogram down from its highest bin to bin b_lo (a
+// bound already known); 0 if none.  Counts only grow, so racy snapshots give
+// a smaller, still valid, bound.  One full warp.
+__device__ __forceinline__ uint64_t hist_top_threshold(const uint32_t *gh, uint32_t b_lo,
+                                                       uint32_t K) {
+  const int lane = threadIdx.x & 31;
+  const int top = (int)min(__ldcg(gh + kCandBins), (uint32_t)kCandBins - 1u);
+  uint32_t run = 0;
+  for (int hi = top; hi >= (int)b_lo; hi -= 32) {
+    const int bin = hi - lane;
+    const uint32_t c = bin >= (int)b_lo ? __ldcg(gh + bin) : 0u;
+    uint32_t incl = c;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t v = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += v;
+    }
+    const uint32_t hit = __ballot_sync(0xffffffffu, run + incl >= K);
+    if (hit) {
+      const int src = __ffs(hit) - 1;
+      return (uint64_t)(hi - src) << kBinShift;
+    }
+    run += __shfl_sync(0xffffffffu, incl, 31);
+  }
+  return 0ull;
+}
+
 // ------------------------------------------------- fixed-point wide terms
 // The window accumulators hold each ad's wide term in 32-bit fixed point
 // (shared-memory integer atomics run several times faster than FP32 or 64-bit

@@ -86,6 +86,7 @@ __device__ __forceinline__ uint32_t ceil_log2(uint32_t n) {
 constexpr int kWinThreads = 256, kWinWarps = kWinThreads / 32;
 constexpr uint32_t kWinChunk = 4096;  // words walked at a time; a block has at most 256
 constexpr uint32_t kWinRows = kWinChunk / kWinThreads;
+constexpr uint32_t kFwdMaxWinQuads = 128;  // most forward quads of one window (48 KB)
 
 struct WinArgs {
   const uint64_t *x;            // sorted distinct words
@@ -97,6 +98,7 @@ struct WinArgs {
   uint32_t *gcnt;               // [9][n_win + 1] blocks of each group and window
   uint16_t *ad_nkeys;           // [n_ads]
   uint32_t *max_keys;           // most keys of one ad
+  uint32_t *run_quads;          // [8 n_win + 1] quads of each run of 32 ads; second walk: first quad
   // layout (second walk)
   const uint32_t *win_ptr[kGroups];
   uint32_t gstart[kGroups + 1];  // blocks of the groups before g
@@ -105,12 +107,18 @@ struct WinArgs {
   uint32_t *bh;                 // [blocks] window of each block, in (g, h, k) order
   void *skey;                   // [blocks] (g, k) of each block, in that order
   uint32_t *sval;               // [blocks] its place in that order
+  uint8_t *fwd;                 // forward table, or null
+  const uint32_t *key_id;       // [n_keys] the keys' ids in it
+  uint32_t quad_bytes, null_key;
 };
 
 // One CTA walks one window's words, kWinChunk at a time.  EMIT = false: blocks
 // per group and keys per ad.  EMIT = true: the window's part of the
-// window-major view, and the sort records of its blocks.  Bound by the read
-// of the words (EMIT = false) and by the byte stores of the values (true).
+// window-major view, its part of the forward table (put together in shared
+// memory: an ad's keys are ranked in word order, which is ascending, like the
+// digits of a sort pass) and the sort records of its blocks.  Bound by the
+// read of the words (EMIT = false) and by the ranking and the byte stores of
+// the values (true).
 // K: type of a sort record, (g << kb) | k.
 template <bool EMIT, typename K>
 __global__ void __launch_bounds__(kWinThreads) k_windows(const __grid_constant__ WinArgs a) {
@@ -119,17 +127,33 @@ __global__ void __launch_bounds__(kWinThreads) k_windows(const __grid_constant__
   __shared__ uint32_t s_g[kWinWarps][16];           // blocks per group: warp counts, then prefixes
   __shared__ uint32_t s_run[16];                    // blocks of each group in the chunks before
   __shared__ uint32_t s_blk[EMIT ? kWinChunk : 1];  // at a head: group << 16 | rank in its warp
+  __shared__ uint16_t s_fr[EMIT ? kWinChunk : 1];   // rank of the word among its ad's in its warp
+  __shared__ uint16_t s_lw[EMIT ? kWinWarps : 1][256];  // words per ad: warp counts, then prefixes
+  __shared__ uint16_t s_lrun[256];                  // words per ad in the chunks before
+  extern __shared__ __align__(16) uint8_t s_fwd[];  // the window's quads
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   if (*a.n_dup) return;  // blocks are sets; the caller drops the repeated words first
   for (uint32_t w = blockIdx.x; w < a.n_win; w += gridDim.x) {
     const uint32_t b0 = a.win_start[w], b1 = a.win_start[w + 1];
     s_adcnt[tid] = 0;
     if (tid < 16) s_run[tid] = 0;
+    const bool fwd = EMIT && a.fwd != nullptr;
+    uint32_t q0 = 0, nq = 0;  // the window's first quad, and quads
+    if (fwd) {
+      s_lrun[tid] = 0;
+      q0 = __ldg(a.run_quads + 8 * w);
+      nq = __ldg(a.run_quads + 8 * w + 8) - q0;
+      const uint32_t lo = (a.null_key & 0xFFFFu) * 0x10001u, hi = (a.null_key >> 16) * 0x1010101u;
+      for (uint32_t i = tid; i < nq * a.quad_bytes / 4; i += kWinThreads)
+        reinterpret_cast<uint32_t *>(s_fwd)[i] = (4 * i) % a.quad_bytes < 256u ? lo : hi;
+    }
     uint32_t c0 = b0;
     while (c0 < b1) {
       __syncthreads();
       if (tid < 16)
         for (int q = 0; q < kWinWarps; q++) s_g[q][tid] = 0;
+      if (fwd)
+        for (int q = 0; q < kWinWarps; q++) s_lw[q][tid] = 0;
       // head bits of words [c0, c0 + chunk + 288); the end counts as a head
       for (uint32_t i = tid; i < kWinChunk + 288u; i += kWinThreads) {
         const uint32_t p = c0 + i;
@@ -171,6 +195,16 @@ __global__ void __launch_bounds__(kWinThreads) k_windows(const __grid_constant__
         if (EMIT) {
           old = __shfl_sync(0xffffffffu, old, leader);
           if (head) s_blk[i] = (g << 16) | (old + __popc(peers & ((1u << lane) - 1u)));
+          if (fwd) {
+            const uint32_t l = in ? (uint32_t)__ldg(a.x + c0 + i) & 255u : 256u + lane;
+            const uint32_t same = __match_any_sync(0xffffffffu, l);
+            const uint32_t below = __popc(same & ((1u << lane) - 1u));
+            const uint32_t was = in ? s_lw[warp][l] : 0u;
+            __syncwarp();
+            if (in && below == 0) s_lw[warp][l] = (uint16_t)(was + __popc(same));
+            __syncwarp();
+            if (in) s_fr[i] = (uint16_t)(was + below);
+          }
         } else if (in) {
           atomicAdd(&s_adcnt[(uint32_t)__ldg(a.x + c0 + i) & 255u], 1u);
         }
@@ -184,6 +218,15 @@ __global__ void __launch_bounds__(kWinThreads) k_windows(const __grid_constant__
           acc += c;
         }
         s_run[tid] = acc;
+      }
+      if (fwd) {
+        uint32_t acc = s_lrun[tid];
+        for (int q = 0; q < kWinWarps; q++) {
+          const uint32_t c = s_lw[q][tid];
+          s_lw[q][tid] = (uint16_t)acc;
+          acc += c;
+        }
+        s_lrun[tid] = (uint16_t)acc;
       }
       __syncthreads();
       if (EMIT) {
@@ -200,9 +243,17 @@ __global__ void __launch_bounds__(kWinThreads) k_windows(const __grid_constant__
           const uint32_t e = s_blk[hp], g = e >> 16;
           const uint32_t rank =
               a.win_ptr[g][w] + s_g[hp / (32 * kWinRows)][g] + (e & 0xFFFFu);
+          const uint32_t key = (uint32_t)((word >> 8) & ((1ull << a.kb) - 1ull));
           a.wvals[g][((uint64_t)rank << g) + (i - hp)] = (uint8_t)word;
+          if (fwd) {
+            const uint32_t l = (uint32_t)word & 255u, fr = s_lw[warp][l] + s_fr[i];
+            uint8_t *quad = s_fwd + (__ldg(a.run_quads + 8 * w + (l >> 5)) - q0 + (fr >> 2)) *
+                                        a.quad_bytes;
+            const uint32_t id = __ldg(a.key_id + key);
+            reinterpret_cast<uint16_t *>(quad)[(l & 31u) * 4 + (fr & 3u)] = (uint16_t)id;
+            if (a.quad_bytes > 256u) quad[256 + (l & 31u) * 4 + (fr & 3u)] = (uint8_t)(id >> 16);
+          }
           if (hp == i) {
-            const uint32_t key = (uint32_t)((word >> 8) & ((1ull << a.kb) - 1ull));
             const uint32_t q = a.gstart[g] + rank;
             a.wkey[g][rank] = key;
             a.bh[q] = w;
@@ -220,6 +271,12 @@ __global__ void __launch_bounds__(kWinThreads) k_windows(const __grid_constant__
       if (ad < a.n_ads) a.ad_nkeys[ad] = (uint16_t)c;
       const uint32_t mx = __reduce_max_sync(0xffffffffu, c);
       if (lane == 0 && mx) atomicMax(a.max_keys, mx);
+      if (lane == 0) a.run_quads[8 * w + warp] = (mx + 3) / 4;
+    } else if (fwd) {
+      __syncthreads();
+      uint4 *dst = reinterpret_cast<uint4 *>(a.fwd + (uint64_t)q0 * a.quad_bytes);
+      for (uint32_t i = tid; i < nq * a.quad_bytes / 16; i += kWinThreads)
+        dst[i] = reinterpret_cast<const uint4 *>(s_fwd)[i];
     }
     __syncthreads();
   }
@@ -329,6 +386,47 @@ __global__ void k_win_bytes(WinPtrs wp, uint32_t n_win, unsigned int *out_max) {
   }
 }
 
+// Key popularity from a sample of the sorted words (every step-th one).
+__global__ void k_sample_keys(const uint64_t *__restrict__ x, uint32_t m, uint32_t step, int kb,
+                              uint32_t *__restrict__ cnt) {
+  for (uint64_t i = (blockIdx.x * (uint64_t)blockDim.x + threadIdx.x) * step; i < m;
+       i += (uint64_t)gridDim.x * blockDim.x * step)
+    atomicAdd(&cnt[(x[i] >> 8) & ((1ull << kb) - 1ull)], 1u);
+}
+// Sort records that put the most frequent keys first (equal counts: by key).
+constexpr int kPopBits = 24;
+__global__ void k_pop_records(uint32_t *__restrict__ cnt, uint32_t n, uint32_t *__restrict__ key) {
+  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+    cnt[i] = (1u << kPopBits) - 1u - min(cnt[i], (1u << kPopBits) - 1u);
+    key[i] = i;
+  }
+}
+__global__ void k_pop_ids(const uint32_t *__restrict__ key, uint32_t n, uint32_t *__restrict__ id) {
+  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
+    id[key[i]] = i;
+}
+
+// Most quads of 1, 2, 4 and 8 aligned runs (out[0 .. 3]) and all of them (out[4]).
+__global__ void k_fwd_max(const uint32_t *__restrict__ off, uint32_t n_win,
+                          uint32_t *__restrict__ out) {
+  uint32_t mx[4] = {0, 0, 0, 0};
+  for (uint32_t w = blockIdx.x * blockDim.x + threadIdx.x; w < n_win; w += gridDim.x * blockDim.x) {
+    uint32_t o[9];
+#pragma unroll
+    for (int i = 0; i < 9; i++) o[i] = off[8 * (uint64_t)w + i];
+#pragma unroll
+    for (int g = 0; g < 4; g++)
+#pragma unroll
+      for (int i = 0; i < 8; i += 1 << g) mx[g] = max(mx[g], o[i + (1 << g)] - o[i]);
+    if (w == n_win - 1) out[4] = o[8];
+  }
+#pragma unroll
+  for (int g = 0; g < 4; g++) {
+    const uint32_t m = __reduce_max_sync(0xffffffffu, mx[g]);
+    if ((threadIdx.x & 31) == 0) atomicMax(out + g, m);
+  }
+}
+
 inline int grid_for(uint64_t n, int threads = 256, int cap = 1 << 16) {
   uint64_t b = (n + threads - 1) / threads;
   if (b < 1) b = 1;
@@ -384,7 +482,7 @@ static int build_key_major(ebr_index *ix, uint32_t nb, KeyArgs &ka, void *k0, vo
 
 // Device words the build reads back in one copy.
 struct BuildCounts {
-  uint32_t flags, n_dup, max_keys, gc[kGroups], win_max[3], m_unique;
+  uint32_t flags, n_dup, max_keys, gc[kGroups], win_max[3], fwd[5], m_unique;
 };
 
 static int build_impl(const ebr_index_desc *desc, ebr_index *ix, cudaStream_t st) {
@@ -392,7 +490,7 @@ static int build_impl(const ebr_index_desc *desc, ebr_index *ix, cudaStream_t st
   const uint32_t n_keys = desc->n_keys, n_ads = desc->n_ads, n_win = (n_ads + 255) / 256;
   const int kb = bits_for(n_keys), hb = bits_for(n_win);
   ix->n_win = n_win;
-  DevBuf in, pool, wpool, blocks;
+  DevBuf in, pool, wpool, blocks, pop;
   int rc = EBR_OK;
   cudaEvent_t ev[4] = {nullptr, nullptr, nullptr, nullptr};
 #define BTRY(expr)                  \
@@ -427,10 +525,13 @@ static int build_impl(const ebr_index_desc *desc, ebr_index *ix, cudaStream_t st
     const size_t gw_b = align_up((size_t)kGroups * (n_win + 1) * 4, 256);
     const size_t ws_b = align_up(((size_t)n_win + 1) * 4, 256);
     const size_t st_b = align_up(prims::scan_scratch((uint64_t)kGroups * (n_win + 1)) * 4, 256);
+    const uint64_t n_runs = 8ull * n_win;
     BTRY(dev_alloc(pool, 2 * words_b + scr_b));
     BTRY(dev_alloc(wpool, 256 + ws_b + gw_b + st_b));
     BTRY(dev_alloc(ix->ad_nkeys, (size_t)n_ads * 2));
     BTRY(dev_alloc(ix->mem_winptr, (size_t)kGroups * (n_win + 1) * 4));
+    BTRY(dev_alloc(ix->mem_fwd_off, (n_runs + 1) * 4));
+    ix->fwd_off = (uint32_t *)ix->mem_fwd_off.p;
     uint64_t *wa = (uint64_t *)pool.p, *wb = (uint64_t *)((char *)pool.p + words_b);
     void *scratch = (char *)pool.p + 2 * words_b;
     BuildCounts *cnt = (BuildCounts *)wpool.p;
@@ -450,6 +551,7 @@ static int build_impl(const ebr_index_desc *desc, ebr_index *ix, cudaStream_t st
     w.gcnt = gcnt;
     w.ad_nkeys = (uint16_t *)ix->ad_nkeys.p;
     w.max_keys = &cnt->max_keys;
+    w.run_quads = ix->fwd_off;
     for (int g = 0; g < kGroups; g++) {
       ix->win_ptr[g] = (uint32_t *)ix->mem_winptr.p + (size_t)g * (n_win + 1);
       w.win_ptr[g] = ix->win_ptr[g];
@@ -457,6 +559,7 @@ static int build_impl(const ebr_index_desc *desc, ebr_index *ix, cudaStream_t st
 
     BCUDA(cudaEventRecord(ev[0], st));
     BCUDA(cudaMemsetAsync(wpool.p, 0, 256 + ws_b + gw_b, st));
+    BCUDA(cudaMemsetAsync(ix->fwd_off, 0, (n_runs + 1) * 4, st));
     if (nnz) {
       bool in_b = false;
       BTRY((prims::radix_sort<uint64_t, false>(PairLoad{pk, pa, n_keys, n_ads, kb, &cnt->flags},
@@ -483,6 +586,10 @@ static int build_impl(const ebr_index_desc *desc, ebr_index *ix, cudaStream_t st
       for (int g = 0; g < kGroups; g++) wp.p[g] = ix->win_ptr[g];
       k_win_bytes<<<grid_for(n_win), 256, 0, st>>>(wp, n_win, cnt->win_max);
       BCUDA(cudaGetLastError());
+      BTRY((prims::scan<uint32_t, prims::AddU32, false>(ix->fwd_off, ix->fwd_off, n_runs + 1,
+                                                        prims::AddU32(), 0u, stmp, nullptr, st)));
+      k_fwd_max<<<grid_for(n_win), 256, 0, st>>>(ix->fwd_off, n_win, cnt->fwd);
+      BCUDA(cudaGetLastError());
       BCUDA(cudaMemcpyAsync(&hc, cnt, sizeof(hc), cudaMemcpyDeviceToHost, st));
       BCUDA(cudaStreamSynchronize(st));
       if (hc.flags) {
@@ -495,6 +602,7 @@ static int build_impl(const ebr_index_desc *desc, ebr_index *ix, cudaStream_t st
       std::swap(wa, wb);
       m -= hc.n_dup;
       BCUDA(cudaMemsetAsync(wpool.p, 0, 256 + ws_b + gw_b, st));
+      BCUDA(cudaMemsetAsync(ix->fwd_off, 0, (n_runs + 1) * 4, st));
     }
     ix->nnz_unique = m;
     ix->max_keys_per_ad = hc.max_keys;
@@ -533,6 +641,42 @@ static int build_impl(const ebr_index_desc *desc, ebr_index *ix, cudaStream_t st
       ka.values[g] = ix->values[g];
       ka.wvals[g] = ix->wvals[g];
     }
+    // The forward table: key spaces that fit 24 bits, windows whose quads fit
+    // the emitting CTA's shared memory, and padding of at most twice the
+    // postings plus a quad per ad (one quad is what an ad with one key needs).
+    ix->fwd_quads = hc.fwd[4];
+    ix->fwd_quad_bytes = n_keys < 65536u ? 256u : 384u;
+    for (int g = 0; g < 4; g++) ix->fwd_max_quads[g] = hc.fwd[g];
+    if (m && n_keys < (1u << 24) - 1u && hc.fwd[3] <= kFwdMaxWinQuads &&
+        (uint64_t)hc.fwd[4] * 128 <= 2ull * m + 4ull * n_ads) {
+      BTRY(dev_alloc(ix->mem_fwd, (size_t)ix->fwd_quads * ix->fwd_quad_bytes + 256));
+      ix->fwd = w.fwd = (uint8_t *)ix->mem_fwd.p;
+      w.quad_bytes = ix->fwd_quad_bytes;
+      w.null_key = n_keys;
+      // The table names a key by its popularity rank (over a sample of up to
+      // 2^20 postings), so that the terms most gathers want are the first
+      // ones, which the scans hold in shared memory.
+      const size_t kn_b = align_up((size_t)n_keys * 4, 256);
+      BTRY(dev_alloc(ix->mem_key_id, kn_b));
+      ix->key_id = (uint32_t *)ix->mem_key_id.p;
+      w.key_id = ix->key_id;
+      BTRY(dev_alloc(pop, 6 * kn_b + prims::sort_scratch(n_keys)));
+      uint32_t *pc[6];
+      for (int i = 0; i < 6; i++) pc[i] = (uint32_t *)((char *)pop.p + i * kn_b);
+      const uint32_t step = std::max<uint32_t>(1, m >> 20);
+      bool in_b = false;
+      BCUDA(cudaMemsetAsync(pc[0], 0, kn_b, st));
+      k_sample_keys<<<grid_for(m / step + 1), 256, 0, st>>>(w.x, m, step, kb, pc[0]);
+      BCUDA(cudaGetLastError());
+      k_pop_records<<<grid_for(n_keys), 256, 0, st>>>(pc[0], n_keys, pc[1]);
+      BCUDA(cudaGetLastError());
+      BTRY((prims::radix_sort<uint32_t, true>(prims::ArrayLoad<uint32_t>{pc[0]}, pc[1], pc[2], pc[3],
+                                              pc[4], pc[5], n_keys, kPopBits,
+                                              (char *)pop.p + 6 * kn_b, &cnt->flags, &in_b, st)));
+      k_pop_ids<<<grid_for(n_keys), 256, 0, st>>>(in_b ? pc[5] : pc[4], n_keys, ix->key_id);
+      BCUDA(cudaGetLastError());
+    }
+    const size_t fwd_smem = w.fwd ? (size_t)hc.fwd[3] * w.quad_bytes : 0;
     // blocks: window of each, then (key, place) records three times over (the
     // sort's input and its two buffers); the sort's scratch is the words'
     const bool k32 = kb + 4 <= 32;
@@ -552,10 +696,10 @@ static int build_impl(const ebr_index_desc *desc, ebr_index *ix, cudaStream_t st
     BCUDA(cudaMemsetAsync(ix->mem_wvals.p, 0, val_total + 256, st));
     if (nb) {
       const uint32_t grid = std::min<uint32_t>(n_win, 1u << 20);
-      if (k32)
-        k_windows<true, uint32_t><<<grid, kWinThreads, 0, st>>>(w);
-      else
-        k_windows<true, uint64_t><<<grid, kWinThreads, 0, st>>>(w);
+      auto kern = k32 ? k_windows<true, uint32_t> : k_windows<true, uint64_t>;
+      BCUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)std::max<size_t>(fwd_smem, 16)));
+      kern<<<grid, kWinThreads, fwd_smem, st>>>(w);
       BCUDA(cudaGetLastError());
     }
     BCUDA(cudaEventRecord(ev[2], st));
@@ -580,7 +724,7 @@ static int build_impl(const ebr_index_desc *desc, ebr_index *ix, cudaStream_t st
     ix->build_ms = a1 + a2;
   }
 done:
-  for (DevBuf *b : {&in, &pool, &wpool, &blocks}) dev_free(*b);
+  for (DevBuf *b : {&in, &pool, &wpool, &blocks, &pop}) dev_free(*b);
   for (auto &e : ev)
     if (e) cudaEventDestroy(e);
   return rc;
@@ -616,6 +760,9 @@ extern "C" void ebr_index_free(ebr_index *ix) {
   dev_free(ix->mem_wkey);
   dev_free(ix->mem_wvals);
   dev_free(ix->mem_winptr);
+  dev_free(ix->mem_fwd);
+  dev_free(ix->mem_fwd_off);
+  dev_free(ix->mem_key_id);
   dev_free(ix->ad_nkeys);
   dev_free(ix->emb_f32);
   dev_free(ix->emb_q);

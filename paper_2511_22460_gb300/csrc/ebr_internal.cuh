@@ -183,6 +183,17 @@ struct ebr_index {
   uint32_t max_win_chunks = 0;  // most 32-unit work chunks in one window
   uint32_t max_keys_per_ad = 0; // most distinct keys any ad belongs to
   uint32_t max_win_slots = 0;   // most value slots (real + padding) in one window
+  // Forward key table (ebr_forward.cu): per run of 32 ads its keys row by row,
+  // four rows to a quad of fwd_quad_bytes (16 low bits of the keys, then the 8
+  // high ones when n_keys needs them); fwd_off[run] = first quad.  Absent
+  // (fwd null) for key spaces of 2^24 and more, and for very uneven key counts.
+  uint8_t *fwd = nullptr;
+  uint32_t *fwd_off = nullptr;  // [8 n_win + 1]
+  uint32_t fwd_quads = 0, fwd_quad_bytes = 256;
+  uint32_t fwd_max_quads[4] = {0, 0, 0, 0};  // most quads of 1, 2, 4, 8 aligned runs
+  // The table's key ids: key_id[k] = rank of key k by popularity (n_keys: padding).
+  uint32_t *key_id = nullptr;
+  ebr::DevBuf mem_fwd, mem_fwd_off, mem_key_id;
   ebr::DevBuf ad_nkeys;         // uint16 [N]: distinct keys of each ad (empty if any > 65535)
   ebr::DevBuf emb_f32;    // float [N][d]
   ebr::DevBuf emb_q;      // bf16 / e4m3 [N][d]
@@ -227,6 +238,29 @@ int launch_fused(const ebr_index *ix, const float *h_u, const float *w_hat, uint
                  const uint32_t *route = nullptr, int *n_launched = nullptr,
                  uint64_t *cta_cand = nullptr, size_t cta_cand_entries = 0);
 bool fused_fits(const ebr_index *ix, uint32_t k);
+// One launch of the scan over the forward key table (ebr_forward.cu): the
+// counterpart of the block-wise fused scan, with the same results.
+struct FwdCall {
+  ebr_dtype dtype;
+  uint32_t d, n_ads, n_keys, k;
+  const void *emb;
+  const float *scale, *h_u;
+  const uint32_t *wq;        // [n_keys + 1] by key id, the last term 0
+  const uint8_t *fwd;        // null: no keys (wide_in or no wide term at all)
+  const uint32_t *fwd_off;
+  uint32_t quad_bytes, total_quads;
+  const uint32_t *max_quads;  // [4], or null without keys
+  const uint64_t *filter;
+  uint64_t *cand_out, *cta_cand;
+  size_t cta_cand_entries;
+  Ctrl *ctrl;
+  float *all_out, *wide_out;
+  uint32_t *hist;
+  const float *wide_in;
+  const uint32_t *route;
+  int cls_shift, sms;
+};
+int launch_forward(const FwdCall &c, cudaStream_t st);
 constexpr size_t kHistWords = 4096;  // candidate-score histogram of the fused scan (2048 bins + top bin)
 constexpr size_t kCtrlBytes = 256;   // Ctrl block, then the histogram, in one buffer (one memset)
 inline uint32_t *ws_hist(const Workspace &w) { return (uint32_t *)((char *)w.ctrl.p + kCtrlBytes); }

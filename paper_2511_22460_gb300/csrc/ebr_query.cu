@@ -83,6 +83,7 @@ __device__ __forceinline__ uint64_t splitmix64(uint64_t x) {
 // is flagged.
 struct PackOut {
   uint32_t *wq;
+  const uint32_t *key_id;  // place of each key's term (null: the key itself)
   int *fx_out;
   int F, cls_shift;
   float wlimit;
@@ -136,7 +137,10 @@ __global__ void k_expand(CrossView cv, const uint32_t *__restrict__ users, uint3
   pdl_trigger();  // the fused scan may start streaming its embedding rows
   const float s0 = pow2f(po.F), s1 = pow2f(po.F + po.cls_shift),
               s2 = pow2f(po.F + 2 * po.cls_shift);
-  if (pack && blockIdx.x == 0 && threadIdx.x == 0) *po.fx_out = po.F;
+  if (pack && blockIdx.x == 0 && threadIdx.x == 0) {
+    *po.fx_out = po.F;
+    po.wq[cv.n_keys] = 0u;  // the forward table's padding key
+  }
   for (uint64_t t = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; t < total;
        t += (uint64_t)gridDim.x * blockDim.x) {
     const uint32_t b = (uint32_t)(t / cv.n_keys), key = (uint32_t)(t % cv.n_keys);
@@ -196,7 +200,7 @@ __global__ void k_expand(CrossView cv, const uint32_t *__restrict__ users, uint3
     w_hat[t] = acc;
     if (pack) {
       if (!(fabsf(acc) <= po.wlimit)) bad |= DEVERR_RANGE;
-      po.wq[t] = pack_term(acc, s0, s1, s2, po.cls_shift > 0);
+      po.wq[po.key_id ? po.key_id[t] : t] = pack_term(acc, s0, s1, s2, po.cls_shift > 0);
     }
     mx = max(mx, __float_as_uint(acc) & 0x7FFFFFFFu);
   }
@@ -1008,7 +1012,7 @@ int ws_prepare_one(ebr_index *ix, uint32_t n_q, uint32_t kcap) {
   Workspace &w = ix->ws;
   EBR_TRY(dev_reserve(w.wide, (size_t)ix->n_ads * 4));
   EBR_TRY(dev_reserve(w.w_dense, (size_t)ix->n_keys * 4));
-  EBR_TRY(dev_reserve(w.wq, (size_t)ix->n_keys * 4));
+  EBR_TRY(dev_reserve(w.wq, ((size_t)ix->n_keys + 4) / 4 * 16));  // whole 16-byte pieces
   const size_t entries = (size_t)kGroups * n_q + 1;
   EBR_TRY(dev_reserve(w.lens, entries * sizeof(LenPair)));
   EBR_TRY(dev_reserve(w.scan, entries * sizeof(LenPair)));
@@ -1155,7 +1159,7 @@ int expand_transposed(const ebr_cross *c, const uint32_t *users, const uint32_t 
 static int expand_into(const ebr_cross *c, const uint32_t *users, uint32_t batch, float *w_hat,
                        uint32_t *flags, cudaStream_t st, uint32_t *wmax = nullptr,
                        const uint32_t *user_ptr = nullptr, uint32_t n_uv = 0,
-                       PackOut po = PackOut{nullptr, nullptr, 0, 0, 0.f}) {
+                       PackOut po = PackOut{nullptr, nullptr, nullptr, 0, 0, 0.f}) {
   CrossView cv = cross_view(c);
   const uint64_t total = (uint64_t)batch * cv.n_keys;
   const size_t smem =
@@ -1226,11 +1230,11 @@ int query_one(const ebr_index *cix, const ebr_cross *cross, const ebr_query &q, 
     // single-valued user fields: the packed terms' exponent follows from the
     // cross model's bound on |w^|, so the expansion writes them directly;
     // otherwise the fused scan's launch packs w^ after its max |w^|
-    PackOut po{nullptr, nullptr, 0, 0, 0.f};
+    PackOut po{nullptr, nullptr, nullptr, 0, 0, 0.f};
     const float wb = cross->wbound * 1.001f;
     if (!q.user_ptr && wb < 3.0e38f && !(q.flags & EBR_QF_KEY_MAJOR)) {
       const uint32_t mk = std::max<uint32_t>(ix->max_keys_per_ad, 1);
-      po = PackOut{(uint32_t *)w.wq.p, &ctrl->fx, fix_exponent(wb, mk), class_shift(mk), wb};
+      po = PackOut{(uint32_t *)w.wq.p, ix->key_id, &ctrl->fx, fix_exponent(wb, mk), class_shift(mk), wb};
       packed = true;
     }
     EBR_TRY(expand_into(cross, q.user_vals, 1, (float *)w.w_dense.p, &ctrl->flags, st,
