@@ -229,48 +229,75 @@ extern "C" int ebr_debug_wait_timeout(uint32_t timeout_us, void *stream) {
 // =====================================================================
 // Batched scan: B users against every ad, one pass over the inventory
 // =====================================================================
-// Per window of 256 ads (one persistent CTA per SM, contiguous windows):
+// The users are scored in groups of 64 (blockIdx.y), each a pass of its own
+// over the inventory: 64 users' expanded weights of one key are 256 bytes, so
+// all of a group's warps share the lines they gather, and a group's slice of
+// w^T stays in L2 (5M ads with 257 k keys: 66 MB per group, 263 MB for 256
+// users, which does not).  The ad rows and the keys are read once per group;
+// that is a small part of the traffic.
+// Per window of 128 ads (256 without a forward table; one persistent CTA per SM,
+// contiguous windows):
 //   producer warp   -- tensor TMA of the window's BF16/FP8 ad rows into a
-//                      stage ring; the users' vectors are loaded once;
+//                      stage ring; the users' vectors (and, kForwardSw, the
+//                      group's slice of w^T) are loaded once;
 //   MMA warp        -- tcgen05.mma with the users as the M side and the
-//                      window's ads as N = 256, in two M-tiles: the even
+//                      window's ads as N, in two M-tiles: the even
 //                      users and the odd users (the user table is stored in
-//                      that pair order), each replicated down the 128 TMEM
-//                      lanes when the batch has fewer than 256 users;
-//                      deep[user][ad] (Eq. 1) lands in TMEM, FP32;
-//   list warps (2)  -- walk the window's blocks in the window-major view of
-//                      the compressed list and lay out, per run of 32 ads, a
-//                      key table T[r][i] = r-th key of ad i (the window's
-//                      slice of L, transposed; short ads padded with a zero
-//                      row of w^T);
-//   epilogue (8)    -- thread = user pair (2u, 2u + 1) at TMEM lane L
-//                      (u = L mod Bq/2), runs of 32 ads per warp:
+//                      that pair order), each replicated four times down the
+//                      128 TMEM lanes; deep[user][ad] (Eq. 1) lands in TMEM;
+//   list warps (2)  -- (kWalk, indexes without a forward table) lay out, per
+//                      run of 32 ads, a key table T[r][i] = r-th key of ad i
+//                      (the window's slice of L, transposed; short ads padded
+//                      with a zero row of w^T) by a walk over the window's
+//                      blocks in the window-major view of the compressed list;
+//                      between windows they raise the users' running
+//                      thresholds from the histograms all CTAs share (one of
+//                      them does only that when there is a forward table);
+//   epilogue (16)   -- thread = user pair (2u, 2u + 1) at TMEM lane u mod 32,
+//                      four ads per warp at a time; a warp copies its
+//                      ads' part of the forward table in by itself
+//                      (cp.async, a window ahead) and turns it into T:
 //                      wide[i] += w^T[T[r][i]][2u .. 2u + 1] for every row r
-//                      (32 independent coalesced 8-byte loads and 32 paired
-//                      FP32 adds per row, accumulators in registers), added
+//                      (coalesced 8-byte loads, three or four rows in flight, paired
+//                      FP32 adds, accumulators in registers), added
 //                      to both users' deep scores (TMEM columns c and
-//                      256 + c), filtered, and each user's candidates above
+//                      window + c), filtered, and each user's candidates above
 //                      its running threshold go to this CTA's per-user buffer
 //                      (top-m kept exactly).
-// With Bq/2 user pairs per replica (32, 64 or 128), the 256/(Bq/2) warps
-// that hold the same pairs split the window's ads, Bq/2 ads each.
+// kForwardSw: a key space whose slice of w^T fits shared memory beside the rest (up to
+// about 500 keys) is gathered from there.
+// What bounds it: the latency of the gathers and, between them, of each
+// window's chain of list, accumulators and candidates (without the gathers
+// 256 users x 5M ads take 4.5 ms); the L1 pipe alone would take 3.1 ms.  The
+// forward table lists an ad's keys in the order of the window-major view (rare
+// keys first), so the FP32 sums are the same as the walk's; rows of four ads are
+// refilled one by one to keep loads in flight within 96 registers (a spill here doubles the
+// time).  Measured scans, before and after: 256 users x 5M BF16 ads (24 keys)
+// 13.6 -> 8.3 ms, 128 users x 5M BF16 ads (32 keys, bitmaps) 10.6 -> 5.1 ms, 64
+// users x 10M FP8 ads (32 keys of 480) 9.0 -> 4.3 ms.
 namespace ebr {
 
 constexpr int kBWin = 256;
-constexpr int kEpiWarps = 8, kListWarps = 2;
+constexpr int kEpiWarps = 16, kListWarps = 2;
 constexpr int kEpiThreads = kEpiWarps * 32, kListThreads = kListWarps * 32;
 constexpr int kMmaWarp = kEpiWarps + kListWarps, kProdWarpB = kMmaWarp + 1;
-constexpr int kBatchThreads = (kProdWarpB + 1) * 32;  // 384
+constexpr int kBatchThreads = (kProdWarpB + 1) * 32;  // 640
 constexpr int kMaxUsers = 256;
 static_assert(kBWin % (kListWarps * 32) == 0, "list threads split the window's ads evenly");
 // List buffer: run_off[8], run_rows[8], fill[256], then the run tables.
 constexpr uint32_t kListHdr = 8 + 8 + kBWin;
 constexpr uint32_t kMaxBatchKeysPerAd = 64;  // longest key list the batched tables hold
+// Bins of a user's score histogram: sign, 8 exponent bits and 4 of the
+// mantissa (6 % wide; the bound is that much lower than the true score).
+constexpr uint32_t kUserBins = 8192;
+constexpr int kUserBinShift = 51;
 
-// Row of user b in the batch's user table: even users first, then odd ones
-// (the two M-tiles of the batched scan), `half` = Bq / 2 rows each.
-__host__ __device__ __forceinline__ uint32_t user_row(uint32_t b, uint32_t half) {
-  return (b & 1u) * half + (b >> 1);
+constexpr uint32_t kGroup = 64;   // users of one pass
+constexpr int kTrimWarps = 8;     // epilogue warps that trim buffers (each needs a histogram)
+// Row of user b in the batch's user table: per group of 64 the even users
+// first, then the odd ones (the two M-tiles of the batched scan).
+__host__ __device__ __forceinline__ uint32_t user_row(uint32_t b) {
+  return (b & ~(kGroup - 1u)) + (b & 1u) * (kGroup / 2) + ((b & (kGroup - 1u)) >> 1);
 }
 
 struct CandEntry {
@@ -281,34 +308,106 @@ struct CandEntry {
 
 struct BatchArgs {
   CUtensorMap ta;  // ad rows, BF16 or FP8 [N][d], box {tile row, 128}
-  CUtensorMap tu;  // users, same type [Bq][d] in pair order, box {tile row, Bq / 2}
+  CUtensorMap tu;  // users, same type [Bq][d] in pair order, box {tile row, 32}
   const uint32_t *wkey[kGroups];
   const uint8_t *wvals[kGroups];
   const uint32_t *win_ptr[kGroups];
   const uint16_t *ad_nkeys;    // [N] distinct keys of each ad
-  const float *wT;             // [n_keys + 1][Bq] expanded weights, user-minor; last row 0
+  const uint8_t *fwd;          // forward table (then w^T's rows go by its key ids), or null
+  const uint32_t *fwd_off;
+  uint32_t quad_bytes, max_quads;  // max_quads: of one run
+  const float *wT;             // [groups][n_keys + 1][64] expanded weights, user-minor; last row 0
+  uint32_t wt_rows;            // n_keys + 1
   const uint64_t *filters;     // [B][words] (rows of users without a filter are unused)
   const uint32_t *has_filter;  // [B]
-  uint32_t n_ads, n_win, B, Bq, d, m, cap_u, list_cap, words;  // B: users (buffer stride)
+  uint32_t n_ads, n_win, B, d, m, cap_u, list_cap, words;  // B: users (buffer stride)
   const uint32_t *B_dev;       // non-null: the active users (<= B) are read here at launch
-  uint32_t zero_row;           // n_keys * Bq / 2: the zero row of wT, in user-pair units
+  uint32_t zero_row;           // n_keys * 32: the zero row of wT, in user-pair units
   uint32_t sa, lb, tb;         // A stages, list buffers, TMEM buffers
   uint32_t tile_row, kb_n;     // bytes per K-tile row (128 or 64), K-tiles per row
   const float *ad_scale;       // FP8: [N] row scales of the ad table
   const float *user_scale;     // FP8: [Bq] row scales of the quantised users (pair order)
+  // Scores counted per user over all CTAs (bins: the top bits of the ranking
+  // key), for a bound on each user's kscan-th best.
+  uint32_t *uhist;             // [B][kUserBins], zeroed per call
+  uint32_t *utop;              // [B] highest bin counted, zeroed per call
+  const uint32_t *kscan;       // [B] candidates each user needs
   CandEntry *cand;             // [grid][B][cap_u]
   uint32_t *cand_n;            // [grid][B]
-  unsigned long long *cand_thr;  // [grid][B]
+  unsigned long long *cand_thr;  // [grid][B] cut of the CTA's own trims
   Ctrl *ctrl;
 };
+
+__device__ __forceinline__ uint4 lds_v4(uint32_t a) {
+  uint4 v;
+  asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];"
+               : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
+               : "r"(a));
+  return v;
+}
+__device__ __forceinline__ uint32_t lds_u32(uint32_t a) {
+  uint32_t v;
+  asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(a));
+  return v;
+}
+__device__ __forceinline__ void sts_u32(uint32_t a, uint32_t v) {
+  asm volatile("st.shared.u32 [%0], %1;" ::"r"(a), "r"(v) : "memory");
+}
+__device__ __forceinline__ void sts_u16(uint32_t a, uint32_t v) {
+  asm volatile("st.shared.u16 [%0], %1;" ::"r"(a), "h"((uint16_t)v) : "memory");
+}
+__device__ __forceinline__ float2 lds_f2(uint32_t a) {
+  float2 v;
+  asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(a));
+  return v;
+}
 
 struct BatchSmem {
   uint64_t a_full[2], a_empty[2], t_full[2], t_empty[2], l_full[2], l_empty[2], u_full;
   uint32_t tmem_base;
-  uint32_t cnt_u[kMaxUsers];
-  unsigned long long thr_u[kMaxUsers];
+  uint32_t cnt_u[kGroup], top_u[kGroup];
+  unsigned long long thr_u[kGroup];  // running threshold: the larger of the two bounds below
+  unsigned long long cut_u[kGroup];  // cut of this CTA's own trims (0: nothing was trimmed)
   uint32_t abort, stop_epi, stop_list, n_issued, n_mma;
+  uint32_t finished;    // the epilogue warps are done
+  uint32_t trim, meet;  // a buffer is nearly full; what a meeting of the epilogue warps is for
 };
+
+// Raises the running threshold of user g0 + b to the largest bin edge with at least
+// kscan[b] counted scores at or above it (every one a distinct ad): the user's
+// kscan-th best over the whole inventory is no lower, so what lies below the
+// edge cannot be selected, and the proof that the merge makes is not touched.
+// Counts only grow, so a snapshot gives a lower, still valid, bound.
+__device__ __forceinline__ void raise_threshold(const BatchArgs &a, BatchSmem &sm, uint32_t g0,
+                                                uint32_t b) {
+  const uint32_t top = __ldcg(a.utop + g0 + b);
+  if (!top) return;
+  const uint32_t need = __ldg(a.kscan + g0 + b);
+  const int g_lo = (int)((uint32_t)(*((volatile unsigned long long *)&sm.thr_u[b]) >> kUserBinShift) >> 4);
+  uint32_t cum = 0;
+  for (int g = (int)(top >> 4); g >= g_lo; g--) {
+    const uint4 *h = reinterpret_cast<const uint4 *>(a.uhist + (size_t)(g0 + b) * kUserBins) + 4 * g;
+    uint32_t c[16];
+#pragma unroll
+    for (int i = 0; i < 4; i++) {
+      const uint4 v = __ldcg(h + i);
+      c[4 * i] = v.x;
+      c[4 * i + 1] = v.y;
+      c[4 * i + 2] = v.z;
+      c[4 * i + 3] = v.w;
+    }
+    int bin = -1;
+#pragma unroll
+    for (int i = 15; i >= 0; i--) {
+      cum += c[i];
+      if (bin < 0 && cum >= need) bin = 16 * g + i;
+    }
+    if (bin >= 0) {
+      atomicMax(&sm.thr_u[b], (unsigned long long)bin << kUserBinShift);
+      return;
+    }
+  }
+}
 
 __device__ __forceinline__ uint32_t ushift(uint32_t g) { return g >= 2 ? g - 2 : 0; }
 
@@ -448,101 +547,41 @@ __device__ uint32_t warp_compact(CandEntry *buf, uint32_t n, uint64_t T) {
   return kept;
 }
 
-// The same selection and compaction on a buffer of at most 32 * NPL entries,
-// read once into registers: the eight digit passes then touch only the
-// shared-memory histogram, and the survivors are written back in one sweep.
-// Returns how many were kept; *T_out = the selected cut.
-constexpr int kSelNpl = 28;  // entries per lane of the register form (896 per buffer)
-template <int NPL>
-__device__ uint32_t warp_trim_regs(CandEntry *buf, uint32_t n, uint32_t need, uint32_t *hist,
-                                   uint64_t *T_out) {
-  const int lane = threadIdx.x & 31;
-  uint64_t x[NPL];
-  float wd[NPL];
-#pragma unroll
-  for (int e = 0; e < NPL; e++) {
-    const uint32_t i = lane + 32u * e;
-    x[e] = 0ull;
-    wd[e] = 0.f;
-    if (i < n) {
-      const CandEntry c = buf[i];
-      x[e] = c.key;
-      wd[e] = c.wide;
-    }
-  }
-  uint64_t prefix = 0;
-  for (int shift = 56; shift >= 0; shift -= 8) {
-    for (int i = lane; i < 256; i += 32) hist[i] = 0;
-    __syncwarp();
-    const uint64_t hi_mask = (shift == 56) ? 0ull : (~0ull << (shift + 8));
-#pragma unroll
-    for (int e = 0; e < NPL; e++)
-      if (lane + 32u * e < n && (x[e] & hi_mask) == prefix)
-        atomicAdd(&hist[(x[e] >> shift) & 255u], 1u);
-    __syncwarp();
-    uint32_t c[8], tot = 0;
-#pragma unroll
-    for (int e = 0; e < 8; e++) {
-      c[e] = hist[255 - 8 * lane - e];
-      tot += c[e];
-    }
-    uint32_t incl = tot;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const uint32_t v = __shfl_up_sync(0xffffffffu, incl, o);
-      if (lane >= o) incl += v;
-    }
-    uint32_t acc = incl - tot, dg = 0, nn = 0, whole = 0;
-    bool found = false;
-#pragma unroll
-    for (int e = 0; e < 8; e++) {
-      if (!found && acc < need && need <= acc + c[e]) {
-        found = true;
-        dg = 255 - 8 * lane - e;
-        nn = need - acc;
-        whole = (need - acc == c[e]) ? 1u : 0u;
-      }
-      acc += c[e];
-    }
-    const uint32_t bal = __ballot_sync(0xffffffffu, found);
-    const int src = __ffs(bal) - 1;
-    dg = __shfl_sync(0xffffffffu, dg, src);
-    need = __shfl_sync(0xffffffffu, nn, src);
-    whole = __shfl_sync(0xffffffffu, whole, src);
-    prefix |= (uint64_t)dg << shift;
-    __syncwarp();
-    if (whole) break;
-  }
-  uint32_t kept = 0;
-#pragma unroll
-  for (int e = 0; e < NPL; e++) {
-    const bool kp = lane + 32u * e < n && x[e] >= prefix;
-    const uint32_t bal = __ballot_sync(0xffffffffu, kp);
-    if (kp) {
-      CandEntry c;
-      c.key = x[e];
-      c.wide = wd[e];
-      c.pad = 0;
-      buf[kept + __popc(bal & ((1u << lane) - 1u))] = c;
-    }
-    kept += __popc(bal);
-  }
-  __syncwarp();
-  *T_out = prefix;
-  return kept;
-}
-
 // Exact top-`need` of a per-user buffer, in place; returns how many were kept.
+// (Trims are rare, so the keys are read again for every digit: a form that held
+// them in registers made the hot loop spill.)
 __device__ __forceinline__ uint32_t warp_trim(CandEntry *buf, uint32_t n, uint32_t need,
                                               uint32_t *hist, uint64_t *T_out) {
-  if (n <= 32u * kSelNpl) return warp_trim_regs<kSelNpl>(buf, n, need, hist, T_out);
   const uint64_t T = warp_radix_select(buf, n, need, hist);
   *T_out = T;
   return warp_compact(buf, n, T);
 }
 
-template <bool F8>
+struct Row4 {
+  float2 x[4];
+};
+
+// MODE: where an ad's keys come from (see above).
+enum { kWalk = 0, kForward = 1, kForwardSw = 2 };
+// Ads of a window: the block-wise lists are per 256 ads; with the forward table
+// 128, so that two windows' accumulators (2 x 128 columns each) fit TMEM and
+// the MMAs of one run while the other's are read.
+constexpr uint32_t kFwdWin = 128;
+
+// cp.async: 16 bytes global -> shared, asynchronously, and the wait for all of
+// the calling thread's.
+__device__ __forceinline__ void cp_async16(uint32_t dst, const void *src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async_wait() {
+  asm volatile("cp.async.wait_all;" ::: "memory");
+}
+
+template <bool F8, int MODE>
 __global__ void __launch_bounds__(kBatchThreads, 1) k_batch_window(const __grid_constant__ BatchArgs a) {
+  constexpr bool FWD = MODE != kWalk, SW = MODE == kForwardSw;
+  constexpr uint32_t kWin = FWD ? kFwdWin : kBWin;      // ads of a window
+  constexpr uint32_t kWarpAds = kWin / kEpiWarps;       // of them per epilogue warp
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   __shared__ BatchSmem sm;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -552,26 +591,38 @@ __global__ void __launch_bounds__(kBatchThreads, 1) k_batch_window(const __grid_
   const uint32_t tile_elems = tr / (F8 ? 1u : 2u);
   const uint32_t n_mt = 2;                        // M-tiles: even users, odd users
   const uint32_t u_tile = kb_n * 128u * tr;        // one M-tile: kb_n x [128 rows x tr]
-  const uint32_t a_stage = kb_n * 256u * tr;       // kb_n x [256 ad rows x tr]
+  const uint32_t a_stage = kb_n * kWin * tr;       // kb_n x [window's ad rows x tr]
   uint8_t *su = smem;                              // n_mt user tiles
   uint8_t *sa = su + (size_t)n_mt * u_tile;        // sa ad stages
   uint32_t *lists = reinterpret_cast<uint32_t *>(sa + (size_t)a.sa * a_stage);
-  const uint32_t list_words = kListHdr + a.list_cap;
-  uint32_t *whist = lists + (size_t)a.lb * list_words;  // [8][256] radix histograms
+  // key lists: kWalk a ring of window lists (32-bit row offsets in user
+  // pairs), else per epilogue warp the raw quads of its ads' next window and
+  // the list of its current one (row offsets, or, SW, 16-bit key ids)
+  const uint32_t list_words = FWD ? 0u : kListHdr + a.list_cap;
+  const uint32_t wlist_bytes = FWD ? a.max_quads * 4u * kWarpAds * (SW ? 2u : 4u) : 0u;
+  const uint32_t wraw_bytes = FWD ? a.max_quads * kWarpAds * (a.quad_bytes > 256u ? 12u : 8u) : 0u;
+  uint32_t *whist = lists + (FWD ? (size_t)kEpiWarps * (wlist_bytes + wraw_bytes) / 4
+                                 : (size_t)a.lb * list_words);  // [kTrimWarps][256]
+  float *s_wT = reinterpret_cast<float *>(whist + kTrimWarps * 256);  // SW: the slice of wT
+  const float *wT = a.wT + (size_t)blockIdx.y * a.wt_rows * kGroup;
 
   const uint32_t w_begin = (uint32_t)(((uint64_t)a.n_win * blockIdx.x) / gridDim.x);
   const uint32_t w_end = (uint32_t)(((uint64_t)a.n_win * (blockIdx.x + 1)) / gridDim.x);
   const uint32_t my_wins = w_end - w_begin;
-  const uint32_t tcols = 256u * n_mt;  // TMEM columns per window
+  const uint32_t tcols = kWin * n_mt;  // TMEM columns per window
   const uint32_t ncols = 512;
   // active users: all B, or the count a device-side loop wrote for this wave
   // (the same for every thread; none: nothing to do, nothing allocated)
   const uint32_t nB = a.B_dev ? min(*a.B_dev, a.B) : a.B;
-  if (nB == 0) return;
+  const uint32_t g0 = blockIdx.y * kGroup;  // the group's first user
+  if (nB <= g0) return;
+  const uint32_t nG = min(nB - g0, kGroup);
 
-  for (uint32_t b = tid; b < a.B; b += kBatchThreads) {
+  for (uint32_t b = tid; b < kGroup; b += kBatchThreads) {
     sm.cnt_u[b] = 0;
+    sm.top_u[b] = 0;
     sm.thr_u[b] = 0ull;
+    sm.cut_u[b] = 0ull;
   }
   if (warp == kMmaWarp) {
     tmem_alloc(&sm.tmem_base, ncols);
@@ -580,15 +631,17 @@ __global__ void __launch_bounds__(kBatchThreads, 1) k_batch_window(const __grid_
   if (tid == 0) {
     sm.abort = 0;
     sm.stop_epi = 0;
+    sm.trim = 0;
+    sm.finished = 0;
     sm.n_issued = 0;
     sm.n_mma = 0;
     for (int q = 0; q < 2; q++) {
       mbar_init(&sm.a_full[q], 1);
       mbar_init(&sm.a_empty[q], 1);
       mbar_init(&sm.t_full[q], 1);
-      mbar_init(&sm.t_empty[q], 1);
+      mbar_init(&sm.t_empty[q], kEpiWarps);
       mbar_init(&sm.l_full[q], kListThreads);
-      mbar_init(&sm.l_empty[q], 1);
+      mbar_init(&sm.l_empty[q], kEpiWarps);
     }
     mbar_init(&sm.u_full, 1);
     fence_mbar_init();
@@ -602,15 +655,17 @@ __global__ void __launch_bounds__(kBatchThreads, 1) k_batch_window(const __grid_
     // ---------------------------------------------------------- producer
     if (lane == 0) {
       const uint64_t pol = l2_evict_first_policy();
-      // users (stored in pair order: even users, then odd users): row r of
-      // M-tile mt holds user 2 (r mod Bq/2) + mt (replicas when Bq < 256)
-      const uint32_t box_u = a.Bq / 2;
-      mbar_arrive_expect_tx(&sm.u_full, n_mt * u_tile);
+      // users (per group: even users, then odd users): row r of M-tile mt
+      // holds the group's user 2 (r mod 32) + mt
+      constexpr uint32_t box_u = kGroup / 2;
+      const uint32_t wt_bytes = SW ? a.wt_rows * kGroup * 4u : 0u;
+      mbar_arrive_expect_tx(&sm.u_full, n_mt * u_tile + wt_bytes);
+      if (SW) bulk_g2s(s_wT, wT, wt_bytes, &sm.u_full);
       for (uint32_t mt = 0; mt < n_mt; mt++)
         for (uint32_t r0 = 0; r0 < 128; r0 += box_u)
           for (uint32_t kb = 0; kb < kb_n; kb++)
             tma_load_2d(su + mt * u_tile + kb * 128u * tr + r0 * tr, &a.tu,
-                        (int)(kb * tile_elems), (int)(mt * box_u), &sm.u_full);
+                        (int)(kb * tile_elems), (int)(g0 + mt * box_u), &sm.u_full);
       for (uint32_t j = 0; j < my_wins; j++) {
         const uint32_t s = j % a.sa;
         if (j >= a.sa && !mbar_wait_bounded(&sm.a_empty[s], ((j / a.sa) - 1) & 1u, kWaitTimeoutNs)) {
@@ -619,12 +674,12 @@ __global__ void __launch_bounds__(kBatchThreads, 1) k_batch_window(const __grid_
           break;
         }
         if (*((volatile uint32_t *)&sm.abort)) break;
-        const int row0 = (int)((w_begin + j) * kBWin);
+        const int row0 = (int)((w_begin + j) * kWin);
         uint8_t *dst = sa + (size_t)s * a_stage;
         mbar_arrive_expect_tx(&sm.a_full[s], a_stage);
         for (uint32_t kb = 0; kb < kb_n; kb++)
-          for (uint32_t h = 0; h < 2; h++)
-            tma_load_2d_hint(dst + kb * 256u * tr + h * 128u * tr, &a.ta, (int)(kb * tile_elems),
+          for (uint32_t h = 0; h < kWin / 128; h++)
+            tma_load_2d_hint(dst + kb * kWin * tr + h * 128u * tr, &a.ta, (int)(kb * tile_elems),
                              row0 + (int)h * 128, &sm.a_full[s], pol);
         sm.n_issued = j + 1;
       }
@@ -633,7 +688,7 @@ __global__ void __launch_bounds__(kBatchThreads, 1) k_batch_window(const __grid_
     // ---------------------------------------------------------- MMA issuer
     if (lane == 0) {
       bool ok = mbar_wait_bounded(&sm.u_full, 0, kWaitTimeoutNs);
-      const uint32_t idesc = F8 ? idesc_e4m3_f32(128, 256) : idesc_bf16_f32(128, 256);
+      const uint32_t idesc = F8 ? idesc_e4m3_f32(128, kWin) : idesc_bf16_f32(128, kWin);
       const uint32_t spt = tr / 32;  // 32-byte K-steps per tile row
       for (uint32_t j = 0; ok && j < my_wins; j++) {
         const uint32_t s = j % a.sa, tb = j % a.tb;
@@ -643,11 +698,11 @@ __global__ void __launch_bounds__(kBatchThreads, 1) k_batch_window(const __grid_
         tc_fence_after();
         const uint8_t *as = sa + (size_t)s * a_stage;
         for (uint32_t mt = 0; mt < n_mt; mt++) {
-          const uint32_t dcol = tmem + tb * tcols + mt * 256u;
+          const uint32_t dcol = tmem + tb * tcols + mt * kWin;
           for (uint32_t k = 0; k < kb_n * spt; k++) {
             const uint32_t kb = k / spt, kk = k % spt;
             const uint32_t ua = smem_u32(su + mt * u_tile + kb * 128u * tr + kk * 32);
-            const uint32_t aa = smem_u32(as + kb * 256u * tr + kk * 32);
+            const uint32_t aa = smem_u32(as + kb * kWin * tr + kk * 32);
             const uint64_t ud = tr == 128 ? sdesc_k_sw128(ua) : sdesc_k_sw64(ua);
             const uint64_t ad = tr == 128 ? sdesc_k_sw128(aa) : sdesc_k_sw64(aa);
             if (F8)
@@ -665,6 +720,14 @@ __global__ void __launch_bounds__(kBatchThreads, 1) k_batch_window(const __grid_
         sm.abort = 1;
       }
     }
+  } else if (FWD && warp >= kEpiWarps) {
+    // ---------------------------------------------------------- thresholds
+    // One warp, a lane per user, as long as the epilogue runs.
+    if (warp == kEpiWarps)
+      while (!*((volatile uint32_t *)&sm.finished) && !*((volatile uint32_t *)&sm.abort)) {
+        for (uint32_t b = lane; b < nG; b += 32) raise_threshold(a, sm, g0, b);
+        __nanosleep(2000);
+      }
   } else if (warp >= kEpiWarps) {
     // ---------------------------------------------------------- list builders
     // Per window: off[l] = first slot of ad l (exclusive scan of the ads' key
@@ -686,6 +749,9 @@ __global__ void __launch_bounds__(kBatchThreads, 1) k_batch_window(const __grid_
       named_sync(2, kListThreads);
       if (sm.stop_list) break;
       if (j >= a.lb) mbar_try_wait(&sm.l_empty[lbuf], ((j / a.lb) - 1) & 1u);
+      // a window has been scored since the last turn: a lane per user raises the thresholds
+      if (j >= a.lb)
+        for (uint32_t b = lt; b < nG; b += kListThreads) raise_threshold(a, sm, g0, b);
       uint32_t *run_off = lists + (size_t)lbuf * list_words;
       uint32_t *run_rows = run_off + 8;
       uint32_t *fill = run_off + 16;
@@ -733,7 +799,7 @@ __global__ void __launch_bounds__(kBatchThreads, 1) k_batch_window(const __grid_
       walk_window(a, w, lt, kListThreads, [&](uint32_t l, uint32_t key) {
         const uint32_t rank = atomicAdd(&fill[l], 1u);
         const uint32_t pos = run_off[l >> 5] + rank * 32u + (l & 31u);
-        if (rank < run_rows[l >> 5] && pos < a.list_cap) tab[pos] = key * (a.Bq / 2);
+        if (rank < run_rows[l >> 5] && pos < a.list_cap) tab[pos] = key * (kGroup / 2);
       });
       mbar_arrive(&sm.l_full[lbuf]);  // release: this thread's list writes
     }
@@ -744,147 +810,341 @@ __global__ void __launch_bounds__(kBatchThreads, 1) k_batch_window(const __grid_
     // reads both users' deep scores (columns c and 256 + c) and gathers
     // both users' weights with one 8-byte load of the user-minor w^T.
     const GroupSync gsync{1, kEpiThreads};
-    const uint32_t q = warp % 4;                  // TMEM lane quadrant of this warp
-    uint32_t *hist = whist + warp * 256;
-    const uint32_t U2 = a.Bq / 2;                 // user pairs (32, 64 or 128)
-    const uint32_t pair = (32u * q + lane) % U2;
-    const uint32_t ad_lo = ((warp / 4) * (128 / U2) + q / (U2 / 32)) * U2, n_ads_w = U2;
-    const uint32_t tl = tmem + ((32u * q) << 16);
-    const uint32_t user0 = 2 * pair, user1 = 2 * pair + 1;
-    const bool ok0 = user0 < nB, ok1 = user1 < nB;
+    const uint32_t ad_lo = warp * kWarpAds;       // this warp's ads in the window
+    const uint32_t tl = tmem + ((32u * (warp % 4)) << 16);  // its TMEM lane quadrant
+    const uint32_t user0 = 2 * lane, user1 = 2 * lane + 1;  // within the group
+    const bool ok0 = user0 < nG, ok1 = user1 < nG;
     // FP8: deep = TMEM x (user scale) x (the ad row's scale); user rows in pair order
-    const float usc0 = F8 && ok0 ? a.user_scale[pair] : 1.f;
-    const float usc1 = F8 && ok1 ? a.user_scale[U2 + pair] : 1.f;
-    const bool filt0 = ok0 && a.has_filter[user0], filt1 = ok1 && a.has_filter[user1];
-    const uint64_t *frow0 = a.filters + (uint64_t)(ok0 ? user0 : 0u) * a.words;
-    const uint64_t *frow1 = a.filters + (uint64_t)(ok1 ? user1 : 0u) * a.words;
-    const float2 *wcol = reinterpret_cast<const float2 *>(a.wT) + pair;
-    CandEntry *ubuf0 = a.cand + ((uint64_t)blockIdx.x * a.B + (ok0 ? user0 : 0u)) * a.cap_u;
-    CandEntry *ubuf1 = a.cand + ((uint64_t)blockIdx.x * a.B + (ok1 ? user1 : 0u)) * a.cap_u;
-    // one (user, ad) score: filtered, thresholded, appended to the user's buffer
-    auto offer = [&](uint32_t user, bool filt, const uint64_t *frow, CandEntry *ubuf,
-                     unsigned long long thr, float deep, float wide, uint32_t ad) {
-      const unsigned long long key = make_key(deep + wide, ad);
+    const float usc0 = F8 && ok0 ? a.user_scale[g0 + lane] : 1.f;
+    const float usc1 = F8 && ok1 ? a.user_scale[g0 + kGroup / 2 + lane] : 1.f;
+    // which of this thread's users have a bitmap (else every ad passes)
+    const bool filt0 = ok0 && a.has_filter[g0 + user0], filt1 = ok1 && a.has_filter[g0 + user1];
+    const float2 *wcol = reinterpret_cast<const float2 *>(wT) + lane;
+    const uint32_t s_wcol = smem_u32(s_wT) + 8u * lane;
+    auto user_buf = [&](uint32_t b) {
+      return a.cand + ((uint64_t)blockIdx.x * a.B + g0 + b) * a.cap_u;
+    };
+    // one (user, ad) score that passed the bitmap and the float test:
+    // thresholded exactly, appended to the user's buffer and counted
+    auto offer = [&](uint32_t user, unsigned long long thr, float score, float wide,
+                     uint32_t ad) {
+      const unsigned long long key = make_key(score, ad);
       if (key < thr) return;
-      if (filt && !((__ldg(frow + (ad >> 6)) >> (ad & 63)) & 1ull)) return;
       const uint32_t pos = atomicAdd(&sm.cnt_u[user], 1u);
       if (pos < a.cap_u) {
         CandEntry ce;
         ce.key = key;
         ce.wide = wide;
         ce.pad = 0;
-        ubuf[pos] = ce;
+        user_buf(user)[pos] = ce;
+        const uint32_t bin = (uint32_t)(key >> kUserBinShift);
+        atomicAdd(a.uhist + (size_t)(g0 + user) * kUserBins + bin, 1u);
+        if (bin > *((volatile uint32_t *)&sm.top_u[user])) {
+          sm.top_u[user] = bin;  // a lost race costs one more global max
+          atomicMax(a.utop + g0 + user, bin);
+        }
       } else {
         atomicOr(&a.ctrl->flags, DEVERR_OVERFLOW);
       }
     };
-    for (uint32_t j = 0; j < my_wins; j++) {
-      const uint32_t tb = j % a.tb, lbuf = j % a.lb;
-      if (tid == 0) {
-        uint32_t stop = *((volatile uint32_t *)&sm.abort);
-        if (!stop && !mbar_wait_bounded(&sm.t_full[tb], (j / a.tb) & 1u, kWaitTimeoutNs)) stop = 1;
-        if (!stop && !mbar_wait_bounded(&sm.l_full[lbuf], (j / a.lb) & 1u, kWaitTimeoutNs)) stop = 1;
-        if (stop && !*((volatile uint32_t *)&sm.abort)) {
-          atomicOr(&a.ctrl->flags, DEVERR_TIMEOUT);
-          sm.abort = 1;
-        }
-        sm.stop_epi = stop;
+    // The warps run free of each other (each hands the list and the
+    // accumulators back by itself) and meet only when a buffer is nearly full,
+    // and at the end: a check asks for 512 free places, because all warps
+    // together may add a window's 256 entries to a user before the next check
+    // and 256 more before every warp has seen the flag.
+    uint32_t j = 0;
+    // FWD: this warp's ads' quads of a window, 16 bytes at a time into raw_a
+    // (per quad the ads' low halves, then their high bytes); o0/o1: the run's
+    // first quad and its end, read a window ahead
+    const uint32_t list_a = smem_u32(lists) + warp * (wlist_bytes + wraw_bytes);
+    const uint32_t raw_a = list_a + wlist_bytes;
+    const uint32_t raw_q = kWarpAds * (a.quad_bytes > 256u ? 12u : 8u);
+    uint32_t nq = 0, o0 = 0, o1 = 0;
+    auto read_offsets = [&](uint32_t jj) {
+      if (FWD && jj < my_wins) {
+        const uint32_t r = (kWin / 32) * (w_begin + jj) + (ad_lo >> 5);
+        o0 = __ldg(a.fwd_off + r);
+        o1 = __ldg(a.fwd_off + r + 1);
       }
-      gsync();
-      if (sm.stop_epi) break;
-      mbar_try_wait(&sm.t_full[tb], (j / a.tb) & 1u);
-      mbar_try_wait(&sm.l_full[lbuf], (j / a.lb) & 1u);
-      tc_fence_after();
-      const uint32_t *run_off = lists + (size_t)lbuf * list_words;
-      const uint32_t *tab = run_off + kListHdr;
-      const uint32_t wbase = (w_begin + j) * kBWin;
-      const unsigned long long thr0 = ok0 ? sm.thr_u[user0] : ~0ull;
-      const unsigned long long thr1 = ok1 ? sm.thr_u[user1] : ~0ull;
-      for (uint32_t c = 0; c < n_ads_w; c += 32) {
-        const uint32_t a0 = ad_lo + c;  // first window-local ad of this run
-        const uint32_t run = a0 >> 5;
-        const uint32_t rows = run_off[8 + run];
-        const uint4 *t4 = reinterpret_cast<const uint4 *>(tab + run_off[run]);
-        float2 acc[32];
+    };
+    auto fetch_quads = [&](uint32_t jj) {  // of window jj, whose offsets are in o0, o1
+      if (!FWD || jj >= my_wins) return;
+      nq = o1 - o0;
+      const uint8_t *src = a.fwd + (uint64_t)o0 * a.quad_bytes + (ad_lo & 31u) * 8u;
+      constexpr uint32_t kLo = kWarpAds / 2, kHi = kWarpAds / 4;  // 16-byte pieces per quad
+      for (uint32_t i = lane; i < nq * kLo; i += 32)
+        cp_async16(raw_a + (i / kLo) * raw_q + (i % kLo) * 16u,
+                   src + (uint64_t)(i / kLo) * a.quad_bytes + (i % kLo) * 16u);
+      if (a.quad_bytes > 256u)
+        for (uint32_t i = lane; i < nq * kHi; i += 32)
+          cp_async16(raw_a + (i / kHi) * raw_q + kWarpAds * 8u + (i % kHi) * 16u,
+                     src - (ad_lo & 31u) * 4u + 256u + (uint64_t)(i / kHi) * a.quad_bytes +
+                         (i % kHi) * 16u);
+    };
+    // the list of the window whose quads have arrived: row r of this warp's
+    // ads; returns the rows that hold a key
+    auto make_list = [&]() -> uint32_t {
+      cp_async_wait();
+      __syncwarp();
+      constexpr uint32_t kStep = 32 / kWarpAds;  // quads at a time
+      const uint32_t ad = lane % kWarpAds;
+      uint32_t last = 0;
+      for (uint32_t q = lane / kWarpAds; q < nq; q += kStep) {
+        const uint32_t at = raw_a + q * raw_q;
+        const float2 lf = lds_f2(at + ad * 8u);
+        const uint32_t lx = __float_as_uint(lf.x), ly = __float_as_uint(lf.y);
+        const uint32_t hi = a.quad_bytes > 256u ? lds_u32(at + kWarpAds * 8u + ad * 4u) : 0u;
+        const uint32_t k[4] = {(lx & 0xFFFFu) | ((hi & 0xFFu) << 16), (lx >> 16) | ((hi & 0xFF00u) << 8),
+                               (ly & 0xFFFFu) | (hi & 0xFF0000u), (ly >> 16) | ((hi >> 24) << 16)};
 #pragma unroll
-        for (int i = 0; i < 32; i++) acc[i] = make_float2(0.f, 0.f);
-        for (uint32_t r = 0; r < rows; r++) {  // one row: 32 independent 8-byte loads
-          float2 v[32];
-#pragma unroll
-          for (int i4 = 0; i4 < 8; i4++) {
-            const uint4 k = t4[r * 8 + i4];
-            v[4 * i4 + 0] = __ldg(wcol + k.x);
-            v[4 * i4 + 1] = __ldg(wcol + k.y);
-            v[4 * i4 + 2] = __ldg(wcol + k.z);
-            v[4 * i4 + 3] = __ldg(wcol + k.w);
-          }
-#pragma unroll
-          for (int i = 0; i < 32; i++) acc[i] = add_f32x2(acc[i], v[i]);
+        for (uint32_t r = 0; r < 4; r++) {
+          const uint32_t e = (4 * q + r) * kWarpAds + ad;
+          if (k[r] != a.wt_rows - 1u) last = 4 * q + r + 1;
+          if (SW)
+            sts_u16(list_a + 2u * e, k[r]);
+          else
+            sts_u32(list_a + 4u * e, k[r] * (kGroup / 2));
         }
-        // lane i holds the row scale of the run's ad i (FP8)
-        const uint32_t ad_l = wbase + a0 + lane;
-        const float sa_l = F8 && ad_l < a.n_ads ? __ldg(a.ad_scale + ad_l) : 1.f;
-#pragma unroll
-        for (int h = 0; h < 2; h++) {
-          uint32_t d0[16], d1[16];  // deep scores of 16 ads for both users, two TMEM loads
-          tmem_ld16(tl + a0 + 16 * h, d0);
-          tmem_ld16(tl + 256u + a0 + 16 * h, d1);
-          tmem_ld_wait();
-#pragma unroll
-          for (int ii = 0; ii < 16; ii++) {
-            const int i = 16 * h + ii;
-            const float sa_i = F8 ? __shfl_sync(0xffffffffu, sa_l, i) : 1.f;
-            const uint32_t ad = wbase + a0 + i;
-            if (ad >= a.n_ads) continue;
-            const float deep0 = F8 ? __uint_as_float(d0[ii]) * (sa_i * usc0) : __uint_as_float(d0[ii]);
-            const float deep1 = F8 ? __uint_as_float(d1[ii]) * (sa_i * usc1) : __uint_as_float(d1[ii]);
-            if (ok0) offer(user0, filt0, frow0, ubuf0, thr0, deep0, acc[i].x, ad);
-            if (ok1) offer(user1, filt1, frow1, ubuf1, thr1, deep1, acc[i].y, ad);
+      }
+      last = __reduce_max_sync(0xffffffffu, last);  // (and the list is written)
+      __syncwarp();
+      return last;
+    };
+    read_offsets(0);
+    fetch_quads(0);
+    read_offsets(1);
+    if (SW) {  // the slice of wT
+      if (!mbar_wait_bounded(&sm.u_full, 0, kWaitTimeoutNs)) {
+        atomicOr(&a.ctrl->flags, DEVERR_TIMEOUT);
+        sm.abort = 1;
+      }
+      __syncwarp();
+    }
+    for (;;) {
+    while (j < my_wins && !__shfl_sync(0xffffffffu, *((volatile uint32_t *)&sm.trim), 0)) {
+      const uint32_t tb = j % a.tb, lbuf = j % a.lb;
+      uint32_t rows, tab_a;  // rows of the list, and its first entry of this warp's ads
+      constexpr uint32_t kRowEntries = FWD ? kWarpAds : 32;
+      if (FWD) {
+        if (*((volatile uint32_t *)&sm.abort)) j = my_wins;
+        j = __shfl_sync(0xffffffffu, j, 0);
+        if (j >= my_wins) break;
+        rows = make_list();
+        tab_a = list_a;
+        fetch_quads(j + 1);
+        read_offsets(j + 2);
+      } else {
+        bool go = true;
+        if (lane == 0)
+          go = !*((volatile uint32_t *)&sm.abort) &&
+               mbar_wait_bounded(&sm.l_full[lbuf], (j / a.lb) & 1u, kWaitTimeoutNs);
+        go = __shfl_sync(0xffffffffu, (int)go, 0) != 0;
+        if (!go) {
+          if (lane == 0 && !*((volatile uint32_t *)&sm.abort)) {
+            atomicOr(&a.ctrl->flags, DEVERR_TIMEOUT);
+            sm.abort = 1;
           }
+          j = my_wins;
+          break;
+        }
+        mbar_try_wait(&sm.l_full[lbuf], (j / a.lb) & 1u);
+        const uint32_t *run_off = lists + (size_t)lbuf * list_words;
+        rows = run_off[8 + (ad_lo >> 5)];
+        tab_a = smem_u32(run_off + kListHdr) + (run_off[ad_lo >> 5] + (ad_lo & 31u)) * 4u;
+      }
+      const uint32_t wbase = (w_begin + j) * kWin;
+      // this warp's ads in both users' bitmaps: in one word each, read
+      // before the gathers
+      const uint32_t ad_w = wbase + ad_lo;
+      uint32_t bits0 = ok0 ? ~0u : 0u, bits1 = ok1 ? ~0u : 0u;
+      if (ad_w < a.n_ads) {
+        const uint64_t *f = a.filters + (uint64_t)(g0 + user0) * a.words + (ad_w >> 6);
+        if (filt0) bits0 = (uint32_t)(__ldg(f) >> (ad_w & 63u));
+        if (filt1) bits1 = (uint32_t)(__ldg(f + a.words) >> (ad_w & 63u));
+      }
+      bool t_ok = false;  // the window's deep scores have been waited for
+      for (uint32_t c = 0; c < kWarpAds; c += 4) {
+        const uint32_t a0 = ad_lo + c;  // first window-local ad of these four
+        // lane i holds the row scale of ad i of the four (FP8)
+        const uint32_t ad_l = wbase + a0 + (lane & 3);
+        const float sa_l = F8 && ad_l < a.n_ads ? __ldg(a.ad_scale + ad_l) : 1.f;
+        Row4 acc;
+#pragma unroll
+        for (int i = 0; i < 4; i++) acc.x[i] = make_float2(0.f, 0.f);
+        // row r of the run: this user pair's weights of the four ads' r-th keys
+        auto load_row = [&](uint32_t r) {
+          const uint32_t at = tab_a + (r * kRowEntries + c) * (SW ? 2u : 4u);
+          Row4 v;
+          if (SW) {
+            const float2 kf = lds_f2(at);
+            const uint32_t k0 = __float_as_uint(kf.x), k1 = __float_as_uint(kf.y);
+            v.x[0] = lds_f2(s_wcol + (k0 & 0xFFFFu) * (kGroup * 4u));
+            v.x[1] = lds_f2(s_wcol + (k0 >> 16) * (kGroup * 4u));
+            v.x[2] = lds_f2(s_wcol + (k1 & 0xFFFFu) * (kGroup * 4u));
+            v.x[3] = lds_f2(s_wcol + (k1 >> 16) * (kGroup * 4u));
+          } else {
+            const uint4 k = lds_v4(at);
+            v.x[0] = __ldg(wcol + k.x);
+            v.x[1] = __ldg(wcol + k.y);
+            v.x[2] = __ldg(wcol + k.z);
+            v.x[3] = __ldg(wcol + k.w);
+          }
+          return v;
+        };
+        auto add_row = [&](const Row4 &v) {
+#pragma unroll
+          for (int i = 0; i < 4; i++) acc.x[i] = add_f32x2(acc.x[i], v.x[i]);
+        };
+        // rows in flight, refilled in turn: four from global memory (three:
+        // 8.7 ms instead of 8.3 with 256 users and 5M ads), three from shared
+        // memory (four: 4.49 ms instead of 4.27 with 64 users and 10M ads)
+        constexpr uint32_t kFly = SW ? 3 : 4;
+        Row4 v0, v1, v2, v3;
+        if (rows > 0) v0 = load_row(0);
+        if (rows > 1) v1 = load_row(1);
+        if (rows > 2) v2 = load_row(2);
+        if (kFly > 3 && rows > 3) v3 = load_row(3);
+        uint32_t r = 0;
+        for (; r + kFly <= rows; r += kFly) {
+          add_row(v0);
+          if (r + kFly < rows) v0 = load_row(r + kFly);
+          add_row(v1);
+          if (r + kFly + 1 < rows) v1 = load_row(r + kFly + 1);
+          add_row(v2);
+          if (r + kFly + 2 < rows) v2 = load_row(r + kFly + 2);
+          if (kFly > 3) {
+            add_row(v3);
+            if (r + kFly + 3 < rows) v3 = load_row(r + kFly + 3);
+          }
+        }
+        if (r < rows) add_row(v0);
+        if (r + 1 < rows) add_row(v1);
+        if (kFly > 3 && r + 2 < rows) add_row(v2);
+        if (!t_ok) {
+          // the deep scores are waited for only now: the MMAs ran behind the gathers
+          t_ok = mbar_wait_bounded(&sm.t_full[tb], (j / a.tb) & 1u, kWaitTimeoutNs);
+          t_ok = __all_sync(0xffffffffu, t_ok);
+          if (!t_ok) {
+            if (lane == 0) {
+              atomicOr(&a.ctrl->flags, DEVERR_TIMEOUT);
+              sm.abort = 1;
+            }
+            break;
+          }
+          tc_fence_after();
+        }
+        uint32_t d0[4], d1[4];  // deep scores of the four ads for both users
+        tmem_ld4(tl + tb * tcols + a0, d0);
+        tmem_ld4(tl + tb * tcols + kWin + a0, d1);
+        tmem_ld_wait();
+        const unsigned long long thr0 = *((volatile unsigned long long *)&sm.thr_u[user0]);
+        const unsigned long long thr1 = *((volatile unsigned long long *)&sm.thr_u[user1]);
+        const float thr0_f = key_score(thr0), thr1_f = key_score(thr1);  // NaN: no bound yet
+        // scores, and which of them pass the bitmap and the float test (bits
+        // 0-3: user0's four ads, 4-7: user1's); a NaN score passes
+        float sc[8];
+        uint32_t pass = 0;
+#pragma unroll
+        for (int i = 0; i < 4; i++) {
+          const float sa_i = F8 ? __shfl_sync(0xffffffffu, sa_l, i) : 1.f;
+          const float deep0 = F8 ? __uint_as_float(d0[i]) * (sa_i * usc0) : __uint_as_float(d0[i]);
+          const float deep1 = F8 ? __uint_as_float(d1[i]) * (sa_i * usc1) : __uint_as_float(d1[i]);
+          sc[i] = deep0 + acc.x[i].x;
+          sc[4 + i] = deep1 + acc.x[i].y;
+          pass |= (!(sc[i] < thr0_f) ? 1u << i : 0u) | (!(sc[4 + i] < thr1_f) ? 16u << i : 0u);
+        }
+        const uint32_t left = a.n_ads - min(a.n_ads, wbase + a0);  // ads of the four that exist
+        const uint32_t exist = left >= 4 ? 0xFu : (1u << left) - 1u;
+        pass &= ((bits0 >> c) & exist) | (((bits1 >> c) & exist) << 4);
+        // one candidate per thread and turn: few threads have any, and hardly
+        // one has two, so a turn or two do for the eight (one inlined copy
+        // instead of eight that each run for a lane or two)
+        while (__any_sync(0xffffffffu, pass != 0u)) {
+          if (pass) {
+            const uint32_t e = __ffs(pass) - 1;
+            pass &= pass - 1;
+            float score = sc[0], wide = acc.x[0].x;
+#pragma unroll
+            for (int i = 1; i < 8; i++)
+              if (e == (uint32_t)i) {
+                score = sc[i];
+                wide = i < 4 ? acc.x[i & 3].x : acc.x[i & 3].y;
+              }
+            offer(e < 4 ? user0 : user1, e < 4 ? thr0 : thr1, score, wide, wbase + a0 + (e & 3));
+          }
+          __syncwarp();
         }
       }
       tc_fence_before();
-      gsync();
-      if (tid == 0) {
+      __syncwarp();
+      if (lane == 0) {
         mbar_arrive(&sm.t_empty[tb]);
-        mbar_arrive(&sm.l_empty[lbuf]);
+        if (!FWD) mbar_arrive(&sm.l_empty[lbuf]);
       }
-      // keep each user's buffer below capacity: exact top-m by radix select
-      for (uint32_t b = warp; b < nB; b += kEpiWarps) {
-        const uint32_t n = sm.cnt_u[b];
-        if (n + kBWin <= a.cap_u) continue;
-        CandEntry *buf = a.cand + ((uint64_t)blockIdx.x * a.B + b) * a.cap_u;
-        const uint32_t nn = min(n, a.cap_u);
-        uint64_t T;
-        const uint32_t kept = warp_trim(buf, nn, a.m, hist, &T);
-        if (lane == 0) {
-          sm.cnt_u[b] = kept;
-          sm.thr_u[b] = T;
-        }
-        __syncwarp();
+      j++;
+      if (!t_ok) {  // timed out above
+        j = my_wins;
+        break;
       }
-      gsync();
+      if ((ok0 && *((volatile uint32_t *)&sm.cnt_u[user0]) + 2 * kBWin > a.cap_u) ||
+          (ok1 && *((volatile uint32_t *)&sm.cnt_u[user1]) + 2 * kBWin > a.cap_u))
+        *((volatile uint32_t *)&sm.trim) = 1u;
+      __syncwarp();
     }
     gsync();
-    // final trim to at most m candidates per user (the merge reads grid * m)
+    if (tid == 0) {
+      sm.stop_epi = *((volatile uint32_t *)&sm.abort);
+      sm.meet = sm.trim;
+      sm.trim = 0;
+    }
+    gsync();
+    if (sm.stop_epi || !sm.meet) break;
+    // make room: drop what the running threshold excludes, then, if that is
+    // not enough, keep the exact top-m by radix select
+    for (uint32_t b = warp; b < nG && warp < kTrimWarps; b += kTrimWarps) {
+      const uint32_t n = min(sm.cnt_u[b], a.cap_u);
+      if (n + 2 * kBWin <= a.cap_u) continue;
+      CandEntry *buf = user_buf(b);
+      uint32_t kept = warp_compact(buf, n, sm.thr_u[b]);
+      if (kept + 3 * kBWin > a.cap_u && kept > a.m) {
+        uint64_t T;
+        kept = warp_trim(buf, kept, a.m, whist + warp * 256, &T);
+        if (lane == 0) {
+          sm.cut_u[b] = max(sm.cut_u[b], (unsigned long long)T);
+          atomicMax(&sm.thr_u[b], (unsigned long long)T);
+        }
+      }
+      if (lane == 0) sm.cnt_u[b] = kept;
+      __syncwarp();
+    }
+    gsync();
+    }
+    if (FWD) cp_async_wait();  // nothing in flight (after an abort) when the CTA ends
+    if (tid == 0) *((volatile uint32_t *)&sm.finished) = 1u;
+    // at most m candidates per user for the merge (it reads grid * m): those
+    // above the latest bound, and if they are more, the best m
     if (!sm.stop_epi) {
-      for (uint32_t b = warp; b < nB; b += kEpiWarps) {
+      for (uint32_t b = tid; b < nG; b += kEpiThreads)
+        if (sm.cnt_u[b] > a.m) raise_threshold(a, sm, g0, b);
+      gsync();
+      for (uint32_t b = warp; b < nG && warp < kTrimWarps; b += kTrimWarps) {
         const uint32_t n = min(sm.cnt_u[b], a.cap_u);
         if (n <= a.m) continue;
-        CandEntry *buf = a.cand + ((uint64_t)blockIdx.x * a.B + b) * a.cap_u;
-        uint64_t T;
-        const uint32_t kept = warp_trim(buf, n, a.m, hist, &T);
-        if (lane == 0) {
-          sm.cnt_u[b] = kept;
-          sm.thr_u[b] = T > sm.thr_u[b] ? T : sm.thr_u[b];
+        CandEntry *buf = user_buf(b);
+        uint32_t kept = warp_compact(buf, n, sm.thr_u[b]);
+        if (kept > a.m) {
+          uint64_t T;
+          kept = warp_trim(buf, kept, a.m, whist + warp * 256, &T);
+          if (lane == 0) sm.cut_u[b] = max(sm.cut_u[b], (unsigned long long)T);
         }
+        if (lane == 0) sm.cnt_u[b] = kept;
         __syncwarp();
       }
     }
     gsync();
-    for (uint32_t b = tid; b < a.B; b += kEpiThreads) {
-      a.cand_n[(uint64_t)blockIdx.x * a.B + b] = min(sm.cnt_u[b], a.cap_u);
-      a.cand_thr[(uint64_t)blockIdx.x * a.B + b] = sm.thr_u[b];
+    for (uint32_t b = tid; b < nG; b += kEpiThreads) {
+      a.cand_n[(uint64_t)blockIdx.x * a.B + g0 + b] = min(sm.cnt_u[b], a.cap_u);
+      a.cand_thr[(uint64_t)blockIdx.x * a.B + g0 + b] = sm.cut_u[b];
     }
   }
   // Drain before teardown (matters only after an abort): the last issued
@@ -914,7 +1174,7 @@ __global__ void __launch_bounds__(kMergeThreads) k_batch_merge(
     const CandEntry *__restrict__ cand, const uint32_t *__restrict__ cand_n,
     const unsigned long long *__restrict__ cand_thr, uint32_t grid, uint32_t B, uint32_t cap_u,
     const uint32_t *__restrict__ kscan, const uint32_t *__restrict__ kout, uint32_t kmax,
-    const float *__restrict__ emb, uint32_t d, const float *__restrict__ h_u, uint32_t half,
+    const float *__restrict__ emb, uint32_t d, const float *__restrict__ h_u,
     uint64_t *__restrict__ scratch /* [B][kMergeCap + 8192] */, uint32_t *__restrict__ out_ids,
     float *__restrict__ out_scores, uint32_t *__restrict__ status /* [B] */,
     const uint32_t *__restrict__ B_dev, const uint32_t *__restrict__ slot_dev,
@@ -938,7 +1198,7 @@ __global__ void __launch_bounds__(kMergeThreads) k_batch_merge(
   // 1. gather this user's candidates into scratch (bounded by 8192: with the
   //    per-CTA thresholds far fewer survive; beyond that the request is flagged)
   if (threadIdx.x == 0) s_cnt = 0;
-  const uint64_t hrow = user_row(b, half);  // the user table is in pair order
+  const uint64_t hrow = user_row(b);  // the user table is in pair order
   for (uint32_t i = threadIdx.x; i < d; i += kMergeThreads) s_h[i] = h_u[hrow * d + i];
   __syncthreads();
   // count first, then copy (entries of all CTAs, in CTA order)
@@ -1074,7 +1334,7 @@ struct ReqSrc {
 };
 constexpr uint32_t kStageWords = 8192;  // filter words per block of the gather
 
-// Block (b, y): request b's user vector (to row user_row(b, half)), field
+// Block (b, y): request b's user vector (to row user_row(b)), field
 // values and field offsets (y == 0) and words [y * kStageWords, +kStageWords)
 // of its filter.  With B_dev (a device-side loop launching Bq blocks), blocks
 // past the wave's users zero their user row and stop.  With
@@ -1083,7 +1343,6 @@ constexpr uint32_t kStageWords = 8192;  // filter words per block of the gather
 // at n; offsets that fail it are flagged and every field is left empty.
 __global__ void __launch_bounds__(256) k_stage_requests(const ReqSrc *__restrict__ src,
                                                         uint32_t d, uint32_t fu, uint32_t words,
-                                                        uint32_t half,
                                                         float *__restrict__ users,
                                                         uint32_t *__restrict__ vals,
                                                         uint32_t *__restrict__ uptr,
@@ -1096,12 +1355,12 @@ __global__ void __launch_bounds__(256) k_stage_requests(const ReqSrc *__restrict
   if (B_dev && b >= *B_dev) {  // a device-side loop's wave has fewer users: zero the row
     if (blockIdx.y == 0)
       for (uint32_t t = threadIdx.x; t < d; t += blockDim.x)
-        users[(size_t)user_row(b, half) * d + t] = 0.f;
+        users[(size_t)user_row(b) * d + t] = 0.f;
     return;
   }
   const ReqSrc r = src[b];
   if (blockIdx.y == 0) {
-    const size_t row = (size_t)user_row(b, half);
+    const size_t row = (size_t)user_row(b);
     for (uint32_t t = threadIdx.x; t < d; t += blockDim.x) users[row * d + t] = r.h_u[t];
     for (uint32_t t = threadIdx.x; t < r.n; t += blockDim.x) vals[(size_t)r.base + t] = r.vals[t];
     if (uptr) {
@@ -1149,43 +1408,50 @@ static uint64_t user_vals_layout(const ebr_query *q, uint32_t B, uint32_t fu,
 
 struct BatchPlan {
   uint32_t Bq, m, cap_u, sa, lb, tb, list_cap, tile_row, kb_n;
+  int mode;  // kWalk, kForward, kForwardSw
   size_t smem;
 };
 
-// Users of the M-tiles: the batch rounded up to 64, 128 or 256 (two tiles of
-// Bq/2 user pairs' halves each).
-static uint32_t users_pow2(uint32_t B) {
-  uint32_t q = 64;
-  while (q < B) q <<= 1;
-  return q;
-}
+// The batch rounded up to whole groups of users.
+static uint32_t users_padded(uint32_t B) { return (B + kGroup - 1) / kGroup * kGroup; }
 
-// Shared-memory layout of k_batch_window: the users' M-tiles, `sa` ad
-// stages, `lb` per-ad key lists and the epilogue's per-warp score tiles.
-// Preference: two list buffers (list building then overlaps the epilogue),
-// then two ad stages.
+// Shared-memory layout of k_batch_window: a group's two M-tiles, `sa` ad
+// stages, the key lists, the trims' histograms and, for a small key space, a
+// group's slice of w^T.  One 256-ad stage (or two of 128) is enough, since the next window's MMAs
+// wait for this window's accumulators to be read anyway, and what is left is
+// L1 for the gathers.
 static bool plan_smem(const ebr_index *ix, uint32_t B, BatchPlan *p) {
-  p->Bq = users_pow2(B);
+  p->Bq = users_padded(B);
   p->list_cap = kBWin * ix->max_keys_per_ad;  // 8 runs x 32 ads x rows
-  const uint32_t n_mt = 2;  // even and odd users: 512 TMEM columns per window
-  p->tb = 1;
+  const uint32_t n_mt = 2;  // even and odd users
+  const uint32_t win = ix->fwd ? kFwdWin : kBWin;
+  p->tb = ix->fwd ? 2 : 1;
+  p->sa = ix->fwd ? 2 : 1;
   const uint32_t row_bytes = ix->d * (ix->dtype == EBR_FP8E4M3 ? 1u : 2u);
   p->tile_row = row_bytes >= 128 ? 128u : 64u;
   p->kb_n = row_bytes / p->tile_row;
   const size_t u_bytes = (size_t)n_mt * p->kb_n * 128 * p->tile_row;
-  const size_t a_stage = (size_t)p->kb_n * 256 * p->tile_row;
-  const size_t list_bytes = ((size_t)kListHdr + p->list_cap) * 4;
-  const size_t hist = (size_t)kEpiWarps * 256 * 4;
+  const size_t a_stage = (size_t)p->kb_n * win * p->tile_row;
+  const size_t hist = (size_t)kTrimWarps * 256 * 4;
+  const size_t fixed = 1024 + u_bytes + p->sa * a_stage + hist;
   const size_t budget = 220 * 1024;
-  const uint32_t order[4][2] = {{2, 2}, {1, 2}, {2, 1}, {1, 1}};  // {sa, lb}
-  for (const auto &o : order) {
-    const size_t need = 1024 + u_bytes + o[0] * a_stage + o[1] * list_bytes + hist;
-    if (need <= budget) {
-      p->sa = o[0];
-      p->lb = o[1];
-      p->smem = need;
-      return true;
-    }
+  const uint32_t mq = ix->fwd_max_quads[0];
+  const size_t raw = (size_t)mq * win * (ix->fwd_quad_bytes > 256u ? 12 : 8);
+  if (ix->fwd) {
+    const size_t wt = ((size_t)ix->n_keys + 1) * kGroup * 4;
+    p->lb = 1;
+    p->mode = kForwardSw;
+    p->smem = fixed + raw + (size_t)mq * 4 * win * 2 + wt;
+    if (ix->n_keys < 4096 && p->smem <= budget) return true;
+    p->mode = kForward;
+    p->smem = fixed + raw + (size_t)mq * 4 * win * 4;
+    if (p->smem <= budget) return true;
+    return false;
+  }
+  p->mode = kWalk;
+  for (p->lb = 2; p->lb >= 1; p->lb--) {
+    p->smem = fixed + p->lb * ((size_t)kListHdr + p->list_cap) * 4;
+    if (p->smem <= budget) return true;
   }
   return false;
 }
@@ -1196,7 +1462,7 @@ bool batch_index_ok(const ebr_index *ix, const ebr_cross *cross, uint32_t batch)
          batch >= 2 && batch <= (uint32_t)kMaxUsers && cross && cross->n_keys == ix->n_keys &&
          ix->n_win > 0 && ix->ad_nkeys.p && ix->max_keys_per_ad > 0 &&
          ix->max_keys_per_ad <= kMaxBatchKeysPerAd &&
-         (uint64_t)(ix->n_keys + 1) * users_pow2(batch) < (1ull << 32) &&
+         ((uint64_t)ix->n_keys + 1) * kGroup < (1ull << 32) &&
          plan_smem(ix, batch, &p);
 }
 
@@ -1215,7 +1481,7 @@ static bool plan_batch(const ebr_index *ix, uint32_t B, uint32_t kscan_max, int 
   if (!plan_smem(ix, B, p)) return false;
   const uint32_t per_cta = (kscan_max + grid - 1) / grid;
   p->m = std::max<uint32_t>(64, (2 * per_cta + 32 + 31) / 32 * 32);
-  p->cap_u = 4 * p->m + kBWin;  // a trim every 3m insertions at least
+  p->cap_u = 4 * p->m + 2 * kBWin;  // room for 4m entries and what the warps add before they meet
   return (uint64_t)grid * p->m <= kMergeCap;
 }
 
@@ -1227,22 +1493,25 @@ struct BatchSizes {
   BatchPlan pl;
   int grid;
   size_t users_f32, users_q, users_scale, user_vals, user_ptr, wT, filters, small, cand, cand_n,
-      cand_thr, scratch, ctrl, req, host;
+      cand_thr, uhist, scratch, ctrl, req, host;
   size_t total() const {
     size_t t = 0;
     for (size_t b : {users_f32, users_q, users_scale, user_vals, user_ptr, wT, filters, small,
-                     cand, cand_n, cand_thr, scratch, ctrl, req})
+                     cand, cand_n, cand_thr, uhist, scratch, ctrl, req})
       t += (b + 255) / 256 * 256;
     return t;
   }
 };
+
+// Per-user score histograms, then their top bins (one memset clears both).
+static size_t user_hist_bytes(uint32_t B) { return (size_t)B * (kUserBins + 1) * 4; }
 
 static size_t host_table_off(uint32_t B) { return ((size_t)4 * B * 4 + 15) / 16 * 16; }
 
 static bool batch_sizes(const ebr_index *ix, const ebr_cross *cross, uint32_t B,
                         uint32_t kscan_max, uint64_t n_vals, BatchSizes *z) {
   if (n_vals == 0) n_vals = (uint64_t)B * cross->f_u;
-  z->grid = std::max(1, std::min<int>(ix->num_sms, (int)ix->n_win));
+  z->grid = std::max(1, std::min<int>(ix->num_sms, (int)ix->n_win));  // CTAs per group
   if (!plan_batch(ix, B, kscan_max, z->grid, &z->pl)) return false;
   const size_t Bp = z->pl.Bq, d = ix->d, words = (ix->n_ads + 63) / 64;
   z->users_f32 = Bp * d * 4;
@@ -1256,6 +1525,7 @@ static bool batch_sizes(const ebr_index *ix, const ebr_cross *cross, uint32_t B,
   z->cand = (size_t)z->grid * B * z->pl.cap_u * sizeof(CandEntry);
   z->cand_n = (size_t)z->grid * B * 4;
   z->cand_thr = (size_t)z->grid * B * 8;
+  z->uhist = user_hist_bytes(B);
   z->scratch = (size_t)B * (kMergeCap + 8192) * 8;
   z->ctrl = sizeof(Ctrl);
   z->req = (size_t)B * sizeof(ReqSrc);
@@ -1290,6 +1560,7 @@ int batch_ws_reserve(const ebr_index *ix, const ebr_cross *cross, uint32_t B,
   EBR_TRY(dev_reserve(w.cand, z.cand));
   EBR_TRY(dev_reserve(w.cand_n, z.cand_n));
   EBR_TRY(dev_reserve(w.cand_thr, z.cand_thr));
+  EBR_TRY(dev_reserve(w.uhist, z.uhist));
   EBR_TRY(dev_reserve(w.scratch, z.scratch));
   EBR_TRY(dev_reserve(w.ctrl, z.ctrl));
   EBR_TRY(dev_reserve(w.req, z.req));
@@ -1315,11 +1586,26 @@ static int stage(void *dst, const void *src, size_t bytes, int io, cudaStream_t 
   return EBR_OK;
 }
 
+// The last row of every group's slice of w^T: the lists' padding key.
+static cudaError_t clear_zero_rows(const ebr_index *ix, BatchWs &w, uint32_t Bq, cudaStream_t st) {
+  const size_t slice = ((size_t)ix->n_keys + 1) * kGroup * 4;
+  return cudaMemset2DAsync((char *)w.wT.p + (size_t)ix->n_keys * kGroup * 4, slice, 0, kGroup * 4,
+                           Bq / kGroup, st);
+}
+
+static void (*window_kernel(bool f8, int mode))(BatchArgs) {
+  if (mode == kForwardSw)
+    return f8 ? k_batch_window<true, kForwardSw> : k_batch_window<false, kForwardSw>;
+  if (mode == kForward)
+    return f8 ? k_batch_window<true, kForward> : k_batch_window<false, kForward>;
+  return f8 ? k_batch_window<true, kWalk> : k_batch_window<false, kWalk>;
+}
+
 // The window kernel's arguments for a batch of B users (B: the candidate
 // buffers' user stride; B_dev: the active users, read on the device, or null).
 static int fill_batch_args(ebr_index *ix, uint32_t B, const BatchPlan &pl, BatchWs &w,
-                           const uint32_t *has_filter, Ctrl *ctrl, const uint32_t *B_dev,
-                           BatchArgs *out) {
+                           const uint32_t *kscan, const uint32_t *has_filter, Ctrl *ctrl,
+                           const uint32_t *B_dev, BatchArgs *out) {
   const bool f8 = ix->dtype == EBR_FP8E4M3;
   const uint32_t eb = f8 ? 1u : 2u, d = ix->d, Bp = pl.Bq;
   if (!w.tmap_ready || w.tmap_for != ix->emb_q.p) {
@@ -1331,7 +1617,7 @@ static int fill_batch_args(ebr_index *ix, uint32_t B, const BatchPlan &pl, Batch
   BatchArgs &a = *out;
   memset(&a, 0, sizeof(a));
   memcpy(&a.ta, w.tmap_bytes, sizeof(CUtensorMap));
-  EBR_TRY(make_tmap_2d(&a.tu, w.users_bf16.p, Bp, d, eb, Bp / 2));
+  EBR_TRY(make_tmap_2d(&a.tu, w.users_bf16.p, Bp, d, eb, kGroup / 2));
   a.tile_row = pl.tile_row;
   a.kb_n = pl.kb_n;
   a.ad_scale = f8 ? (const float *)ix->emb_scale.p : nullptr;
@@ -1342,19 +1628,23 @@ static int fill_batch_args(ebr_index *ix, uint32_t B, const BatchPlan &pl, Batch
     a.win_ptr[g] = ix->win_ptr[g];
   }
   a.ad_nkeys = (const uint16_t *)ix->ad_nkeys.p;
+  a.fwd = ix->fwd;
+  a.fwd_off = ix->fwd_off;
+  a.quad_bytes = ix->fwd_quad_bytes;
+  a.max_quads = ix->fwd_max_quads[0];
   a.wT = (const float *)w.wT.p;
   a.filters = (const uint64_t *)w.filters.p;
   a.has_filter = has_filter;
   a.n_ads = ix->n_ads;
-  a.n_win = ix->n_win;
+  a.n_win = pl.mode == kWalk ? ix->n_win : (ix->n_ads + kFwdWin - 1) / kFwdWin;
   a.B = B;
   a.B_dev = B_dev;
-  a.Bq = Bp;
+  a.wt_rows = ix->n_keys + 1;
   a.d = d;
   a.m = pl.m;
   a.cap_u = pl.cap_u;
   a.list_cap = pl.list_cap;
-  a.zero_row = ix->n_keys * (Bp / 2);  // in 8-byte pair units
+  a.zero_row = ix->n_keys * (kGroup / 2);  // in 8-byte pair units
   a.words = (ix->n_ads + 63) / 64;
   a.sa = pl.sa;
   a.lb = pl.lb;
@@ -1362,6 +1652,9 @@ static int fill_batch_args(ebr_index *ix, uint32_t B, const BatchPlan &pl, Batch
   a.cand = (CandEntry *)w.cand.p;
   a.cand_n = (uint32_t *)w.cand_n.p;
   a.cand_thr = (unsigned long long *)w.cand_thr.p;
+  a.uhist = (uint32_t *)w.uhist.p;
+  a.utop = a.uhist + (size_t)B * kUserBins;
+  a.kscan = kscan;
   a.ctrl = ctrl;
   return EBR_OK;
 }
@@ -1430,6 +1723,7 @@ int batch_launch(ebr_index *ix, const ebr_cross *cross, const ebr_query *q, uint
   EBR_CUDA_TRY(cudaMemsetAsync(ctrl, 0, sizeof(Ctrl), st));
   EBR_CUDA_TRY(cudaMemcpyAsync(kk, h_in, (size_t)3 * B * 4, cudaMemcpyHostToDevice, st));
   EBR_CUDA_TRY(cudaMemsetAsync(status, 0, B * 4, st));
+  EBR_CUDA_TRY(cudaMemsetAsync(w.uhist.p, 0, user_hist_bytes(B), st));
   // request inputs: device-resident requests are gathered by one kernel
   // through a table of their pointers; host requests are packed into the
   // pinned mirror and copied in two transfers (filters one per request)
@@ -1446,7 +1740,7 @@ int batch_launch(ebr_index *ix, const ebr_cross *cross, const ebr_query *q, uint
     uint32_t *hv = hp + (size_t)B * (fu + 2);
     if (Bp > B) memset(hu, 0, (size_t)Bp * d * 4);
     for (uint32_t b = 0; b < B; b++) {
-      memcpy(hu + (size_t)user_row(b, Bp / 2) * d, q[b].h_u, (size_t)d * 4);
+      memcpy(hu + (size_t)user_row(b) * d, q[b].h_u, (size_t)d * 4);
       memcpy(hv + vbase[b], q[b].user_vals, (size_t)nv[b] * 4);
       if (!multi) continue;
       uint32_t *up = hp + (size_t)b * (fu + 1);
@@ -1467,7 +1761,7 @@ int batch_launch(ebr_index *ix, const ebr_cross *cross, const ebr_query *q, uint
     EBR_CUDA_TRY(cudaMemcpyAsync(w.req.p, tab, (size_t)B * sizeof(ReqSrc), cudaMemcpyHostToDevice,
                                  st));
     const uint32_t ys = any_filter ? (words + kStageWords - 1) / kStageWords : 1u;
-    k_stage_requests<<<dim3(B, ys), 256, 0, st>>>((const ReqSrc *)w.req.p, d, fu, words, Bp / 2,
+    k_stage_requests<<<dim3(B, ys), 256, 0, st>>>((const ReqSrc *)w.req.p, d, fu, words,
                                                   (float *)w.users_f32.p,
                                                   (uint32_t *)w.user_vals.p, d_uptr, d_base,
                                                   (uint64_t *)w.filters.p, &ctrl->flags, nullptr);
@@ -1482,15 +1776,15 @@ int batch_launch(ebr_index *ix, const ebr_cross *cross, const ebr_query *q, uint
     EBR_TRY(launch_quantize((const float *)w.users_f32.p, (uint64_t)Bp * d, EBR_BF16,
                             w.users_bf16.p, st));
   EBR_TRY(expand_transposed(cross, (const uint32_t *)w.user_vals.p, d_uptr, d_base, B, Bp,
-                            (float *)w.wT.p, &ctrl->flags, st));
-  EBR_CUDA_TRY(cudaMemsetAsync((float *)w.wT.p + (size_t)ix->n_keys * Bp, 0, (size_t)Bp * 4, st));
+                            (float *)w.wT.p, &ctrl->flags, st, nullptr, ix->key_id));
+  EBR_CUDA_TRY(clear_zero_rows(ix, w, Bp, st));
   BatchArgs a;
-  EBR_TRY(fill_batch_args(ix, B, pl, w, has_filter, ctrl, nullptr, &a));
-  auto kern = f8 ? k_batch_window<true> : k_batch_window<false>;
+  EBR_TRY(fill_batch_args(ix, B, pl, w, kk, has_filter, ctrl, nullptr, &a));
+  auto kern = window_kernel(f8, pl.mode);
   EBR_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                     (int)pl.smem));
   if (prof) EBR_CUDA_TRY(cudaEventRecord(ev[1], st));
-  kern<<<grid, kBatchThreads, pl.smem, st>>>(a);
+  kern<<<dim3(grid, Bp / kGroup), kBatchThreads, pl.smem, st>>>(a);
   EBR_CUDA_TRY(cudaGetLastError());
   if (prof) EBR_CUDA_TRY(cudaEventRecord(ev[2], st));
   EBR_CUDA_TRY(cudaFuncSetAttribute(k_batch_merge, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -1498,7 +1792,7 @@ int batch_launch(ebr_index *ix, const ebr_cross *cross, const ebr_query *q, uint
   k_batch_merge<<<B, kMergeThreads, 8192 * 8, st>>>(
       (const CandEntry *)w.cand.p, (const uint32_t *)w.cand_n.p,
       (const unsigned long long *)w.cand_thr.p, (uint32_t)grid, B, pl.cap_u, kk, kk + B, kmax,
-      (const float *)ix->emb_f32.p, d, (const float *)w.users_f32.p, Bp / 2,
+      (const float *)ix->emb_f32.p, d, (const float *)w.users_f32.p,
       (uint64_t *)w.scratch.p, d_ids, d_scores, status, nullptr, nullptr, 0, 0);
   EBR_CUDA_TRY(cudaGetLastError());
   if (prof) {
@@ -1529,7 +1823,7 @@ int batch_finish(ebr_index *ix, const ebr_cross *cross, const ebr_query *q, uint
   for (uint32_t b = 0; b < B; b++) {
     if (!h_status[b]) continue;
     ebr_query dq = q[b];
-    dq.h_u = (const float *)w.users_f32.p + (size_t)user_row(b, users_pow2(B) / 2) * d;
+    dq.h_u = (const float *)w.users_f32.p + (size_t)user_row(b) * d;
     dq.user_vals = (const uint32_t *)w.user_vals.p + vbase[b];
     // the checked offsets staged for the batch (device memory)
     dq.user_ptr = q[b].user_ptr ? (const uint32_t *)w.user_ptr.p + (size_t)b * (fu + 1) : nullptr;
@@ -1548,7 +1842,7 @@ int batch_finish(ebr_index *ix, const ebr_cross *cross, const ebr_query *q, uint
 
 void batch_ws_free(BatchWs &w) {
   for (DevBuf *b : {&w.users_f32, &w.users_bf16, &w.users_scale, &w.user_vals, &w.user_ptr, &w.wT,
-                    &w.filters, &w.small, &w.cand, &w.cand_n, &w.cand_thr, &w.scratch, &w.res,
+                    &w.filters, &w.small, &w.cand, &w.cand_n, &w.cand_thr, &w.uhist, &w.scratch, &w.res,
                     &w.ctrl, &w.req})
     dev_free(*b);
   if (w.host) cudaFreeHost(w.host);
@@ -1804,7 +2098,7 @@ int loop_build(ebr_index *ix, const ebr_cross *cross, uint32_t max_user_vals, Ba
   const ReqSrc *srcs = (const ReqSrc *)(cur + desc_src_off(Bmax));
   uint32_t *d_uptr = (uint32_t *)w.user_ptr.p;
   uint32_t *d_base = d_uptr + (size_t)Bmax * (fu + 1);
-  auto kern = f8 ? k_batch_window<true> : k_batch_window<false>;
+  auto kern = window_kernel(f8, pl.mode);
   EBR_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                     (int)pl.smem));
   EBR_CUDA_TRY(cudaFuncSetAttribute(k_batch_merge, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -1873,13 +2167,13 @@ int loop_build(ebr_index *ix, const ebr_cross *cross, uint32_t max_user_vals, Ba
     pc.Bq = la.bq[c];
     const uint32_t Bp = pc.Bq;
     BatchArgs ba;
-    rc = fill_batch_args(ix, Bmax, pc, w, hf, L.ctrl, B_dev, &ba);
+    rc = fill_batch_args(ix, Bmax, pc, w, ks, hf, L.ctrl, B_dev, &ba);
     if (rc != EBR_OK) break;
     e = cudaStreamBeginCaptureToGraph(st, sp.conditional.phGraph_out[c], nullptr, nullptr, 0,
                                       cudaStreamCaptureModeRelaxed);
     if (e != cudaSuccess) break;
     const uint32_t ys = (words + kStageWords - 1) / kStageWords;
-    k_stage_requests<<<dim3(Bp, ys), 256, 0, st>>>(srcs, d, fu, words, Bp / 2,
+    k_stage_requests<<<dim3(Bp, ys), 256, 0, st>>>(srcs, d, fu, words,
                                                    (float *)w.users_f32.p,
                                                    (uint32_t *)w.user_vals.p, d_uptr, d_base,
                                                    (uint64_t *)w.filters.p, &L.ctrl->flags, B_dev);
@@ -1891,14 +2185,16 @@ int loop_build(ebr_index *ix, const ebr_cross *cross, uint32_t max_user_vals, Ba
                            w.users_bf16.p, st);
     if (rc == EBR_OK)
       rc = expand_transposed(cross, (const uint32_t *)w.user_vals.p, d_uptr, d_base,
-                             std::min(Bmax, Bp), Bp, (float *)w.wT.p, &L.ctrl->flags, st, B_dev);
+                             std::min(Bmax, Bp), Bp, (float *)w.wT.p, &L.ctrl->flags, st, B_dev,
+                             ix->key_id);
     if (rc == EBR_OK) {
-      cudaMemsetAsync((float *)w.wT.p + (size_t)ix->n_keys * Bp, 0, (size_t)Bp * 4, st);
-      kern<<<z.grid, kBatchThreads, pl.smem, st>>>(ba);
+      clear_zero_rows(ix, w, Bp, st);
+      cudaMemsetAsync(w.uhist.p, 0, user_hist_bytes(Bmax), st);
+      kern<<<dim3(z.grid, Bp / kGroup), kBatchThreads, pl.smem, st>>>(ba);
       k_batch_merge<<<std::min(Bmax, Bp), kMergeThreads, 8192 * 8, st>>>(
           (const CandEntry *)w.cand.p, (const uint32_t *)w.cand_n.p,
           (const unsigned long long *)w.cand_thr.p, (uint32_t)z.grid, Bmax, pl.cap_u, ks, ko,
-          L.kmax, (const float *)ix->emb_f32.p, d, (const float *)w.users_f32.p, Bp / 2,
+          L.kmax, (const float *)ix->emb_f32.p, d, (const float *)w.users_f32.p,
           (uint64_t *)w.scratch.p, L.out_ids, L.out_scores, L.status, B_dev, L.slot,
           (uint64_t)Bmax * L.kmax, Bmax);
     }

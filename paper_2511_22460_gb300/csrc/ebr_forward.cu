@@ -2,8 +2,8 @@
 //
 // The forward table (built with the index, ebr_index.cu) holds, for every run
 // of 32 consecutive ads, the ads' keys row by row: row r is the r-th key (in
-// ascending order) of each of the 32 ads, four rows to a quad, short ads
-// padded with the key n_keys whose term is zero.  It is the same binary
+// the order of the window-major view) of each of the 32 ads, four rows to a
+// quad, short ads padded with the key n_keys whose term is zero.  It is the same binary
 // feature->ad matrix L as the compressed lists of Algorithm 1 (Sec. 3.4),
 // transposed.  With it a warp evaluates the wide term of the HitMatch equation
 // (Sec. 3.3) for its 32 ads in registers, one ad per lane: two or three

@@ -17,7 +17,8 @@
 // (k_windows<true>) writes the window-major view; the key-major arrays then
 // come from a stable sort of the blocks, half as many as the words, by
 // (g, k) alone.  Measured, 2 M ads with 16 keys each (32 M pairs, 15 M
-// blocks): 2.7 ms of device time for all of it, against 8.0 ms when
+// blocks): 3.6 ms of device time for all of it with the forward table (2.7 ms
+// without), against 8.0 ms without one when
 // the words were sorted key-major by 7 three-kernel passes and the blocks
 // again by 8 passes into the window order.
 //
@@ -86,7 +87,7 @@ __device__ __forceinline__ uint32_t ceil_log2(uint32_t n) {
 constexpr int kWinThreads = 256, kWinWarps = kWinThreads / 32;
 constexpr uint32_t kWinChunk = 4096;  // words walked at a time; a block has at most 256
 constexpr uint32_t kWinRows = kWinChunk / kWinThreads;
-constexpr uint32_t kFwdMaxWinQuads = 128;  // most forward quads of one window (48 KB)
+constexpr uint32_t kFwdMaxWinQuads = 128;  // most forward quads of one window (176 KB to build)
 
 struct WinArgs {
   const uint64_t *x;            // sorted distinct words
@@ -116,7 +117,9 @@ struct WinArgs {
 // per group and keys per ad.  EMIT = true: the window's part of the
 // window-major view, its part of the forward table (put together in shared
 // memory: an ad's keys are ranked in word order, which is ascending, like the
-// digits of a sort pass) and the sort records of its blocks.  Bound by the
+// digits of a sort pass, and then put in the order in which the walk over the
+// window's blocks meets them, so that FP32 sums over the table are the walk's)
+// and the sort records of its blocks.  Bound by the
 // read of the words (EMIT = false) and by the ranking and the byte stores of
 // the values (true).
 // K: type of a sort record, (g << kb) | k.
@@ -130,6 +133,7 @@ __global__ void __launch_bounds__(kWinThreads) k_windows(const __grid_constant__
   __shared__ uint16_t s_fr[EMIT ? kWinChunk : 1];   // rank of the word among its ad's in its warp
   __shared__ uint16_t s_lw[EMIT ? kWinWarps : 1][256];  // words per ad: warp counts, then prefixes
   __shared__ uint16_t s_lrun[256];                  // words per ad in the chunks before
+  __shared__ uint32_t s_ubase[kGroups];
   extern __shared__ __align__(16) uint8_t s_fwd[];  // the window's quads
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   if (*a.n_dup) return;  // blocks are sets; the caller drops the repeated words first
@@ -139,10 +143,18 @@ __global__ void __launch_bounds__(kWinThreads) k_windows(const __grid_constant__
     if (tid < 16) s_run[tid] = 0;
     const bool fwd = EMIT && a.fwd != nullptr;
     uint32_t q0 = 0, nq = 0;  // the window's first quad, and quads
+    uint64_t *s_ent = nullptr;  // the quads' entries in key order: place in the walk << 32 | key id
     if (fwd) {
       s_lrun[tid] = 0;
       q0 = __ldg(a.run_quads + 8 * w);
       nq = __ldg(a.run_quads + 8 * w + 8) - q0;
+      s_ent = reinterpret_cast<uint64_t *>(s_fwd + nq * a.quad_bytes);
+      if (tid < kGroups) {  // the window's units in the groups before
+        uint32_t u = 0;
+        for (int g = 0; g < tid; g++)
+          u += (a.win_ptr[g][w + 1] - a.win_ptr[g][w]) << (g >= 2 ? g - 2 : 0);
+        s_ubase[tid] = u;
+      }
       const uint32_t lo = (a.null_key & 0xFFFFu) * 0x10001u, hi = (a.null_key >> 16) * 0x1010101u;
       for (uint32_t i = tid; i < nq * a.quad_bytes / 4; i += kWinThreads)
         reinterpret_cast<uint32_t *>(s_fwd)[i] = (4 * i) % a.quad_bytes < 256u ? lo : hi;
@@ -247,11 +259,15 @@ __global__ void __launch_bounds__(kWinThreads) k_windows(const __grid_constant__
           a.wvals[g][((uint64_t)rank << g) + (i - hp)] = (uint8_t)word;
           if (fwd) {
             const uint32_t l = (uint32_t)word & 255u, fr = s_lw[warp][l] + s_fr[i];
-            uint8_t *quad = s_fwd + (__ldg(a.run_quads + 8 * w + (l >> 5)) - q0 + (fr >> 2)) *
-                                        a.quad_bytes;
-            const uint32_t id = __ldg(a.key_id + key);
-            reinterpret_cast<uint16_t *>(quad)[(l & 31u) * 4 + (fr & 3u)] = (uint16_t)id;
-            if (a.quad_bytes > 256u) quad[256 + (l & 31u) * 4 + (fr & 3u)] = (uint8_t)(id >> 16);
+            const uint32_t qd = __ldg(a.run_quads + 8 * w + (l >> 5)) - q0 + (fr >> 2);
+            // its place in the walk of the batched scan (walk_window): unit U of
+            // the window's, slot s of the unit; 64 units at a time, in each
+            // all first slots before all second ones
+            const uint32_t in_g = s_g[hp / (32 * kWinRows)][g] + (e & 0xFFFFu), off = i - hp;
+            const uint32_t U = s_ubase[g] + (g >= 2 ? (in_g << (g - 2)) + (off >> 2) : in_g);
+            const uint32_t ord = ((U >> 6) << 8) | ((off & 3u) << 6) | (U & 63u);
+            s_ent[qd * 128 + (l & 31u) * 4 + (fr & 3u)] =
+                ((uint64_t)ord << 32) | __ldg(a.key_id + key);
           }
           if (hp == i) {
             const uint32_t q = a.gstart[g] + rank;
@@ -273,6 +289,31 @@ __global__ void __launch_bounds__(kWinThreads) k_windows(const __grid_constant__
       if (lane == 0 && mx) atomicMax(a.max_keys, mx);
       if (lane == 0) a.run_quads[8 * w + warp] = (mx + 3) / 4;
     } else if (fwd) {
+      __syncthreads();
+      // A warp per run, ad by ad: a lane per key (two with over 32), its row
+      // the number of the ad's keys before it in the walk.
+      const uint32_t qd = __ldg(a.run_quads + 8 * w + warp) - q0;
+      for (uint32_t l = 0; l < 32; l++) {
+        const uint32_t n = s_lrun[warp * 32 + l];
+        const uint64_t *ent = s_ent + qd * 128 + l * 4;
+        for (uint32_t i0 = 0; i0 < n; i0 += 32) {
+          const uint32_t i = i0 + lane;
+          const uint64_t x = i < n ? ent[(i >> 2) * 128 + (i & 3u)] : ~0ull;
+          uint32_t r = 0;
+          for (uint32_t j0 = 0; j0 < n; j0 += 32) {
+            const uint32_t j = j0 + lane;
+            const uint32_t o =
+                j < n ? (uint32_t)(ent[(j >> 2) * 128 + (j & 3u)] >> 32) : 0xFFFFFFFFu;
+            for (uint32_t t = 0; t < min(32u, n - j0); t++)
+              r += __shfl_sync(0xffffffffu, o, t) < (uint32_t)(x >> 32) ? 1u : 0u;
+          }
+          if (i < n) {
+            uint8_t *quad = s_fwd + (qd + (r >> 2)) * a.quad_bytes;
+            reinterpret_cast<uint16_t *>(quad)[l * 4 + (r & 3u)] = (uint16_t)x;
+            if (a.quad_bytes > 256u) quad[256 + l * 4 + (r & 3u)] = (uint8_t)(x >> 16);
+          }
+        }
+      }
       __syncthreads();
       uint4 *dst = reinterpret_cast<uint4 *>(a.fwd + (uint64_t)q0 * a.quad_bytes);
       for (uint32_t i = tid; i < nq * a.quad_bytes / 16; i += kWinThreads)
@@ -676,7 +717,7 @@ static int build_impl(const ebr_index_desc *desc, ebr_index *ix, cudaStream_t st
       k_pop_ids<<<grid_for(n_keys), 256, 0, st>>>(in_b ? pc[5] : pc[4], n_keys, ix->key_id);
       BCUDA(cudaGetLastError());
     }
-    const size_t fwd_smem = w.fwd ? (size_t)hc.fwd[3] * w.quad_bytes : 0;
+    const size_t fwd_smem = w.fwd ? (size_t)hc.fwd[3] * (w.quad_bytes + 1024) : 0;
     // blocks: window of each, then (key, place) records three times over (the
     // sort's input and its two buffers); the sort's scratch is the words'
     const bool k32 = kb + 4 <= 32;

@@ -94,7 +94,7 @@ struct BatchWs {
   DevBuf users_f32, users_bf16, users_scale, user_vals, wT, filters;  // users_bf16: BF16 or FP8
   DevBuf user_ptr;  // multi-valued users: field offsets [B][f_u + 1], then base [B]
   DevBuf small;  // uint32 [kscan B][kout B][has_filter B], then status [B]
-  DevBuf cand, cand_n, cand_thr, scratch;
+  DevBuf cand, cand_n, cand_thr, uhist, scratch;  // uhist: score histograms, then top bins
   DevBuf res;    // device staging of host-bound results
   DevBuf ctrl;   // Ctrl of this batch
   DevBuf req;    // pointer table of device-resident requests (staging gather)
@@ -290,13 +290,16 @@ int ws_prepare_one(ebr_index *ix, uint32_t n_q, uint32_t kcap);
 int launch_quantize(const float *x, uint64_t n, ebr_dtype dt, void *out, cudaStream_t st);
 int launch_quantize_rows_fp8(const float *x, uint64_t n, uint32_t d, uint8_t *q, float *scale,
                              cudaStream_t st);
-// Query expansion for a batch straight into user-minor layout wT[key][Bp].
+// Query expansion for a batch straight into user-minor layout, per group of 64
+// users: wT[b / 64][key or key_id[key]][b % 64], n_keys + 1 rows per group.
 // uptr/base null: users[b * f_u + i]; else user b's field i holds
 // users[base[b] + uptr[b][i] .. base[b] + uptr[b][i + 1]) (checked offsets).
 // batch_dev (optional): the users of this wave, read on the device (<= batch).
+// key_id (optional): the row of each key (the forward table's ids).
 int expand_transposed(const ebr_cross *c, const uint32_t *users, const uint32_t *uptr,
                       const uint32_t *base, uint32_t batch, uint32_t Bp, float *wT,
-                      uint32_t *flags, cudaStream_t st, const uint32_t *batch_dev = nullptr);
+                      uint32_t *flags, cudaStream_t st, const uint32_t *batch_dev = nullptr,
+                      const uint32_t *key_id = nullptr);
 // Batched tensor-core path; returns EBR_EINVAL (nothing launched) when the
 // batch does not qualify, so the caller can fall back to per-request scans.
 bool batch_qualifies(const ebr_index *ix, const ebr_cross *cross, const ebr_query *q,

@@ -1080,7 +1080,8 @@ static int run_wide(ebr_index *ix, const uint32_t *q_key, const float *q_w, uint
   return EBR_OK;
 }
 
-// w_hat transposed: wT[key][b] for b < Bp (zero for padding users b >= batch).
+// w_hat transposed, for b < Bp users (a multiple of 64; zero for padding users
+// b >= batch): wT[b / 64][row][b % 64], row = key_id[key] (or key).
 // User b's field values are users[base[b] + uptr[b][i] .. base[b] +
 // uptr[b][i+1]) for field i (MULTI; offsets already checked); without MULTI
 // every field holds one value, users[b * f_u + i].  Pairs are summed in pair
@@ -1090,7 +1091,8 @@ template <bool MULTI>
 __global__ void k_expand_T(CrossView cv, const uint32_t *__restrict__ users,
                            const uint32_t *__restrict__ uptr, const uint32_t *__restrict__ base,
                            uint32_t batch, uint32_t Bp, float *__restrict__ wT,
-                           uint32_t *__restrict__ flags, const uint32_t *__restrict__ batch_dev) {
+                           uint32_t *__restrict__ flags, const uint32_t *__restrict__ batch_dev,
+                           const uint32_t *__restrict__ key_id) {
   extern __shared__ uint32_t s_off2[];
   if (batch_dev) {  // a device-side loop: this wave's users (none: nothing to expand)
     batch = min(*batch_dev, batch);
@@ -1133,14 +1135,17 @@ __global__ void k_expand_T(CrossView cv, const uint32_t *__restrict__ users,
         }
       }
     }
-    wT[t] = acc;
+    // per group of 64 users a slice of n_keys + 1 rows
+    const uint32_t row = key_id ? __ldg(key_id + key) : key;
+    wT[((uint64_t)(b >> 6) * ((uint64_t)cv.n_keys + 1) + row) * 64u + (b & 63u)] = acc;
   }
   if (bad) atomicOr(flags, bad);
 }
 
 int expand_transposed(const ebr_cross *c, const uint32_t *users, const uint32_t *uptr,
                       const uint32_t *base, uint32_t batch, uint32_t Bp, float *wT,
-                      uint32_t *flags, cudaStream_t st, const uint32_t *batch_dev) {
+                      uint32_t *flags, cudaStream_t st, const uint32_t *batch_dev,
+                      const uint32_t *key_id) {
   CrossView cv = cross_view(c);
   const uint64_t total = (uint64_t)cv.n_keys * Bp;
   uint64_t blocks = (total + 255) / 256;
@@ -1148,10 +1153,10 @@ int expand_transposed(const ebr_cross *c, const uint32_t *users, const uint32_t 
   const size_t smem = (c->f_a + 1) * 4;
   if (uptr)
     k_expand_T<true><<<(int)blocks, 256, smem, st>>>(cv, users, uptr, base, batch, Bp, wT, flags,
-                                                     batch_dev);
+                                                     batch_dev, key_id);
   else
     k_expand_T<false><<<(int)blocks, 256, smem, st>>>(cv, users, nullptr, nullptr, batch, Bp, wT,
-                                                      flags, batch_dev);
+                                                      flags, batch_dev, key_id);
   EBR_CUDA_TRY(cudaGetLastError());
   return EBR_OK;
 }
