@@ -2105,8 +2105,9 @@ int loop_build(ebr_index *ix, const ebr_cross *cross, uint32_t max_user_vals, Ba
                                     8192 * 8));
   LoopArgs la;
   memset(&la, 0, sizeof(la));
-  la.nsw = 0;
-  for (uint32_t q = 64; q <= pl.Bq; q <<= 1) la.bq[la.nsw++] = q;
+  la.nsw = 0;  // 64, 128, ... and, last, the table's own width
+  for (uint32_t q = kGroup; q < pl.Bq; q <<= 1) la.bq[la.nsw++] = q;
+  la.bq[la.nsw++] = pl.Bq;
   cudaGraph_t g = nullptr;
   EBR_CUDA_TRY(cudaGraphCreate(&g, 0));
   int rc = EBR_OK;

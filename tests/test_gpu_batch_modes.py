@@ -82,3 +82,37 @@ def test_every_user_of_a_batch(n_ads, n_keys, most, even, d, dtype, B, k):
         kb = qs[b].k
         check_topk(ids[b, :kb], sc[b, :kb], ref, tol, kb, masks[b])
         assert np.all(ids[b, kb:] == 0xFFFFFFFF) and np.all(np.isneginf(sc[b, kb:]))
+
+
+def test_waves_wider_than_two_groups():
+    """A server whose user table is not a power of two of groups wide: 600
+    requests at once, each with the result that a batched call gives it."""
+    n_ads, n_keys, B, k = 1_000_000, 3000, 150, 50
+    rng = np.random.default_rng(5)
+    pk, pa = _postings(n_ads, n_keys, 4, True, rng)
+    emb = (rng.standard_normal((n_ads, 64)) / 8).astype(np.float32)
+    h = (rng.standard_normal((B, 64)) / 8).astype(np.float32)
+    users = rng.integers(0, 50, (B, 1)).astype(np.uint32)
+    ix = ebr.build_index(n_ads, n_keys, pk, pa, emb, dtype="bf16")
+    cross = ebr.cross_create([50], [n_keys], [(0, 0)],
+                             (rng.standard_normal(1 << 16) * 0.3).astype(np.float32),
+                             hashed=True, hash_bits=16)
+    hd, ud = _dev(h), _dev(users.view(np.int32))
+    ids = torch.empty((B, k), dtype=torch.int32, device=DEV)
+    sc = torch.empty((B, k), device=DEV)
+    ebr.score_topk(ix, cross, [ebr.Query(h_u=hd[b], k=k, user_vals=ud[b]) for b in range(B)],
+                   ids, sc)
+    torch.cuda.synchronize()
+    ids, sc = ids.cpu().numpy().view(np.uint32), sc.cpu().numpy()
+    srv = ebr.Server(ix, cross, max_batch=B, max_slots=4 * B, k_max=k)
+    try:
+        tickets = [srv.submit(h[i % B], users[i % B], k) for i in range(4 * B)]
+        for i, t in enumerate(tickets):
+            gi, gs = srv.wait(t, k)
+            b = i % B
+            # the same FP32 rescoring; an FP32 sum of 68 terms below 2 orders ties
+            assert np.max(np.abs(gs - sc[b])) <= 68 * 2.0 ** -22
+            assert np.intersect1d(gi, ids[b]).size >= k - 1
+        print("requests per wave: %.1f" % (4 * B / srv.stats().batches))
+    finally:
+        srv.close()
