@@ -326,8 +326,9 @@ int ebr_debug_wait_timeout(uint32_t timeout_us, void *stream);
  * boundary (its rows are staged by bulk copies); a misaligned emb returns
  * EBR_EINVAL before anything is launched.
  *
- * It allocates nothing: its scratch is a static device array of 1.25 MiB
- * (candidates of up to 160 CTAs x 1024, plus a 64-byte control block), held by
+ * It allocates nothing: its scratch is a static device array of 1.27 MiB
+ * (candidates of up to 160 CTAs x 1024, a control block and a score
+ * histogram), held by
  * every GPU that loads this library until the process exits.  The first call
  * on a device looks up that array's device address (cudaGetSymbolAddress),
  * so make the first call on each device before any stream capture; the

@@ -225,8 +225,22 @@ __device__ __forceinline__ bool wait_stage(FwdSmem &sm, uint32_t s, uint32_t tur
   return mbar_wait_bounded(&sm.full[s], turn & 1u, kWaitTimeoutNs);
 }
 
+// Sum over the chunks congruent to I modulo S: pairs S apart ... first, so
+// S = 1 is the order of a butterfly reduction over one lane per chunk.
+template <int I, int S, int N, typename F>
+__device__ __forceinline__ float tree_sum(F leaf) {
+  if constexpr (S == N)
+    return leaf(I);
+  else
+    return tree_sum<I, 2 * S, N>(leaf) + tree_sum<I + S, 2 * S, N>(leaf);
+}
+
+// TREE (FP32 only): the additions of the inner product in the order of the
+// allocation-free scan, a chain of four multiply-adds per chunk and a tree over
+// the chunks.  (The chunks are visited in the order i ^ rot here too: an XOR
+// only swaps the sides of the tree's additions.)
 // ALL: every term is in shared memory; else those with id < hot are.
-template <typename Elt, int D, bool ALL>
+template <typename Elt, int D, bool ALL, bool TREE>
 __global__ void __launch_bounds__((cons_warps<Elt>() + 2) * 32, 1)
     k_forward(const __grid_constant__ FwdArgs a) {
   constexpr int kConsWarps = cons_warps<Elt>(), kConsThreads = kConsWarps * 32;
@@ -362,7 +376,7 @@ __global__ void __launch_bounds__((cons_warps<Elt>() + 2) * 32, 1)
   if constexpr (!kMma) {
 #pragma unroll
     for (int i = 0; i < Sh::kCPT; i++) {
-      const uint32_t c = qd * Sh::kCPT + (i ^ rot);
+      const uint32_t c = TREE ? (i ^ rot) * Sh::kTPR + qd : qd * Sh::kCPT + (i ^ rot);
 #pragma unroll
       for (int e = 0; e < Tr::kVec; e++) hreg[i * Tr::kVec + e] = s_h[c * Tr::kVec + e];
     }
@@ -548,7 +562,15 @@ __global__ void __launch_bounds__((cons_warps<Elt>() + 2) * 32, 1)
           const uint32_t rw = Sh::kTPR == 1 ? lane : 16 * ps + lane / 2;
           const uint8_t *row = stage + (size_t)(rs * 32u + rw) * Sh::kRowBytes;
           float2 d2 = make_float2(0.f, 0.f);
-          if (run * 32u + rw < a.n_ads) {
+          if (TREE) {
+            d2.x = tree_sum<0, 1, Sh::kCPT>([&](int i) {
+              const float4 f = *reinterpret_cast<const float4 *>(
+                  row + ((i ^ rot) * Sh::kTPR + qd) * 16);
+              return fmaf(hreg[4 * i + 3], f.w,
+                          fmaf(hreg[4 * i + 2], f.z,
+                               fmaf(hreg[4 * i + 1], f.y, fmaf(hreg[4 * i], f.x, 0.f))));
+            });
+          } else if (run * 32u + rw < a.n_ads) {
 #pragma unroll
             for (int i = 0; i < Sh::kCPT; i++) {
               const uint32_t c = qd * Sh::kCPT + (i ^ rot);
@@ -558,7 +580,7 @@ __global__ void __launch_bounds__((cons_warps<Elt>() + 2) * 32, 1)
                               d2);
             }
           }
-          float dd = d2.x + d2.y;
+          float dd = TREE ? d2.x : d2.x + d2.y;
           if (Sh::kTPR == 2) {
             dd += __shfl_xor_sync(0xffffffffu, dd, 1);
             const float mine = __shfl_sync(0xffffffffu, dd, 2 * (lane & 15));
@@ -770,7 +792,10 @@ int launch_t(const FwdCall &c, FwdArgs a, cudaStream_t st) {
   }
   a.stages = stages;
   a.workers = std::min<uint32_t>(cons_warps<Elt>(), stages << lg);
-  auto kern = sw ? k_forward<Elt, D, true> : k_forward<Elt, D, false>;
+  auto kern = sw ? k_forward<Elt, D, true, false> : k_forward<Elt, D, false, false>;
+  if constexpr (std::is_same<Elt, float>::value) {
+    if (c.tree) kern = k_forward<float, D, false, true>;
+  }
   EBR_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   EBR_CUDA_TRY(launch_pdl(kern, grid, (cons_warps<Elt>() + 2) * 32, smem, st, a));
   return EBR_OK;

@@ -242,6 +242,7 @@ bool fused_fits(const ebr_index *ix, uint32_t k);
 // counterpart of the block-wise fused scan, with the same results.
 struct FwdCall {
   ebr_dtype dtype;
+  bool tree;                 // FP32: add the inner product's 4-element chunks as a tree
   uint32_t d, n_ads, n_keys, k;
   const void *emb;
   const float *scale, *h_u;

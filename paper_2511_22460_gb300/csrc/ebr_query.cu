@@ -3,6 +3,7 @@
 // and a per-CTA radix-select top-K, the final merge, and FP32 rescoring.
 
 #include <algorithm>
+#include <atomic>
 #include <array>
 #include <cstring>
 #include <mutex>
@@ -852,56 +853,181 @@ __device__ void bitonic_sort_desc(uint64_t *v, uint32_t n_pow2) {
   __syncthreads();
 }
 
-// Selects the best min(k, n) keys among n (global memory) and writes k_out
-// ids/scores sorted descending, padded with (0xFFFFFFFF, -inf), or the keys
-// themselves in no particular order, padded with zero keys.  Dynamic shared memory: 8 * (pow2(min(k, n)) + buf_cap)
-// bytes; when n <= buf_cap the keys are read from global memory once and the
-// radix select runs on the shared copy, otherwise on the global keys.
-// Waits (pdl_wait) for the kernel before it in the stream.
+// Selects the best min(k, n) keys among n (global memory; zero keys are absent
+// ones) and writes k_out ids/scores sorted descending, padded with
+// (0xFFFFFFFF, -inf), or the keys themselves, padded with zero keys.
+// One CTA, so what bounds it is the chain of barriers: a radix select of 8-bit
+// digits and a bitonic sort met 30 to 100 times.  Instead the scores are put
+// in 4096 equal bins between the smallest and the largest, one scan over the
+// bins gives each its place in the order and the bin that holds the k-th key,
+// the keys of that bin and above are scattered to their bins, and each counts
+// the larger keys of its own bin: six barriers.  Keys crowded into a few bins
+// (equal scores, mostly) take the radix select and the bitonic sort.  Measured: REPLACE_FINAL
+// Dynamic shared memory: final_smem(k).
+// Waits (pdl_wait) for the kernel before it in the stream.  (keys and ctrl are
+// not __restrict__: a load through such a pointer may be moved above the wait.)
+constexpr uint32_t kFinalBins = 4096, kFinalMaxBin = 192;
+static_assert(kFinalThreads == 1024, "a warp's lanes hold the warps' values");
+constexpr int kFinalRegs = 8;  // keys per thread held in registers between the passes
+static __host__ __device__ uint32_t final_cap(uint32_t k) {  // entries of the scattered keys
+  uint32_t p = 1;
+  while (p < k) p <<= 1;
+  return max(p, k + 1024u);
+}
+static size_t final_smem(uint32_t k) { return (size_t)final_cap(k) * 8 + kFinalBins * 8; }
+
 __global__ void __launch_bounds__(kFinalThreads) k_final_select(
-    const uint64_t *__restrict__ keys, const Ctrl *__restrict__ ctrl, uint32_t n_fixed,
+    const uint64_t *keys, const Ctrl *ctrl, uint32_t n_fixed,
     uint32_t k, uint32_t k_out, uint32_t *__restrict__ out_ids, float *__restrict__ out_scores,
-    uint64_t *__restrict__ out_keys, uint32_t buf_cap) {
+    uint64_t *__restrict__ out_keys) {
   extern __shared__ __align__(16) uint64_t s_v[];
-  __shared__ uint32_t s_hist[256];
-  __shared__ uint32_t s_misc[8];
-  __shared__ uint32_t s_cnt;
+  const uint32_t cap = final_cap(k);
+  uint32_t *s_cnt = reinterpret_cast<uint32_t *>(s_v + cap);  // keys of each bin
+  uint32_t *s_base = s_cnt + kFinalBins;                      // keys in higher bins
+  __shared__ uint32_t s_hist[256], s_misc[8];
+  __shared__ uint32_t s_w[3][32];
+  __shared__ uint32_t s_bin, s_m, s_crowded, s_n;
+  const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  for (uint32_t i = tid; i < kFinalBins; i += kFinalThreads) s_cnt[i] = 0;
+  if (tid == 0) {
+    s_crowded = 0;
+    s_n = 0;
+  }
   pdl_wait();
-  const uint32_t n = ctrl ? ctrl->n_cand : n_fixed;
-  const uint32_t take = min(n, k);
-  uint32_t p2 = 1;
-  while (p2 < take) p2 <<= 1;
-  const uint64_t *src = keys;
-  if (n <= buf_cap) {  // one read of the keys, then everything in shared memory
-    uint64_t *s_buf = s_v + p2;
-    for (uint32_t i = threadIdx.x; i < n; i += kFinalThreads) s_buf[i] = keys[i];
-    __syncthreads();
-    src = s_buf;
+  const uint32_t n = ctrl ? *((const volatile uint32_t *)&ctrl->n_cand) : n_fixed;
+  // pass 1: smallest and largest score, number of keys
+  uint64_t reg[kFinalRegs];
+  uint32_t mn = 0xFFFFFFFFu, mx = 0, real = 0;
+#pragma unroll
+  for (int e = 0; e < kFinalRegs; e++) {
+    const uint32_t i = tid + e * kFinalThreads;
+    reg[e] = i < n ? __ldcg(keys + i) : 0ull;
   }
-  uint64_t T = 0;
-  if (n > k) T = cta_radix_select<kFinalThreads>(src, n, k, s_hist, s_misc);
-  if (threadIdx.x == 0) s_cnt = 0;
+  auto for_keys = [&](auto f) {
+#pragma unroll
+    for (int e = 0; e < kFinalRegs; e++)
+      if (reg[e]) f(reg[e]);
+    for (uint32_t i = tid + kFinalRegs * kFinalThreads; i < n; i += kFinalThreads) {
+      const uint64_t x = __ldcg(keys + i);
+      if (x) f(x);
+    }
+  };
+  for_keys([&](uint64_t x) {
+    const uint32_t h = (uint32_t)(x >> 32);
+    mn = min(mn, h);
+    mx = max(mx, h);
+    real++;
+  });
+  mn = __reduce_min_sync(0xffffffffu, mn);
+  mx = __reduce_max_sync(0xffffffffu, mx);
+  real = __reduce_add_sync(0xffffffffu, real);
+  if (lane == 0) {
+    s_w[0][warp] = mn;
+    s_w[1][warp] = mx;
+    s_w[2][warp] = real;
+  }
   __syncthreads();
-  for (uint32_t base = 0; base < n; base += kFinalThreads) {
-    const uint32_t i = base + threadIdx.x;
-    const uint64_t x = i < n ? src[i] : 0ull;
-    const bool kp = i < n && x >= T;
-    const uint32_t pos = warp_append(kp, &s_cnt);
-    if (kp && pos < p2) s_v[pos] = x;
-  }
-  __syncthreads();
-  for (uint32_t i = take + threadIdx.x; i < p2; i += kFinalThreads) s_v[i] = 0ull;
-  if (out_keys) {  // keys for a later stage (FP32 rescoring): any order will do
+  mn = __reduce_min_sync(0xffffffffu, s_w[0][lane]);
+  mx = __reduce_max_sync(0xffffffffu, s_w[1][lane]);
+  real = __reduce_add_sync(0xffffffffu, s_w[2][lane]);
+  const uint32_t take = min(real, k);
+  if (take) {
+    const float lo_s = unord_f32(mn), range = unord_f32(mx) - lo_s;
+    const bool finite = range < INFINITY;  // else bins of the ordered integers
+    const float scale = range > 0.f ? fminf((float)kFinalBins / range, 3e38f) : 0.f;
+    const uint32_t shift = max(20 - (int)__clz(mx - mn), 0);  // (clz(0) = 32)
+    // monotone: subtraction, product and conversion round monotonically
+    auto bin_of = [&](uint64_t x) {
+      const uint32_t h = (uint32_t)(x >> 32);
+      if (!finite) return (h - mn) >> shift;
+      return min((uint32_t)((unord_f32(h) - lo_s) * scale), kFinalBins - 1);
+    };
+    // pass 2: keys per bin, then (a thread has four bins, from the top) the
+    // keys in the bins above
+    for_keys([&](uint64_t x) { atomicAdd(&s_cnt[bin_of(x)], 1u); });
     __syncthreads();
-  } else {
-    bitonic_sort_desc(s_v, p2);
+    {
+      constexpr uint32_t kPer = kFinalBins / kFinalThreads;
+      const uint32_t top = kFinalBins - 1 - kPer * tid;
+      uint32_t c[kPer], sum = 0;
+#pragma unroll
+      for (uint32_t e = 0; e < kPer; e++) {
+        c[e] = s_cnt[top - e];
+        sum += c[e];
+      }
+      uint32_t incl = sum;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= (uint32_t)o) incl += y;
+      }
+      if (lane == 31) s_w[0][warp] = incl;
+      __syncthreads();
+      uint32_t above = __reduce_add_sync(0xffffffffu, lane < warp ? s_w[0][lane] : 0u) + incl - sum;
+#pragma unroll
+      for (uint32_t e = 0; e < kPer; e++) {
+        s_base[top - e] = above;
+        if (above < take) {
+          if (c[e] > kFinalMaxBin) s_crowded = 1;
+          if (above + c[e] >= take) {
+            s_bin = top - e;
+            s_m = above + c[e];
+          }
+        }
+        above += c[e];
+      }
+    }
+    __syncthreads();
+    const uint32_t cut = s_bin, m = s_m;
+    if (!s_crowded && m <= cap) {
+      // pass 3: the keys of the cut's bin and above, by bin; then each key's
+      // place among its bin's
+      for_keys([&](uint64_t x) {
+        const uint32_t b = bin_of(x);
+        if (b >= cut) s_v[s_base[b] + atomicSub(&s_cnt[b], 1u) - 1u] = x;
+      });
+      __syncthreads();
+      for (uint32_t p = tid; p < m; p += kFinalThreads) {
+        const uint64_t x = s_v[p];
+        const uint32_t b = bin_of(x), lo = s_base[b], hi = b == cut ? m : s_base[b - 1];
+        uint32_t r = lo;
+        for (uint32_t q = lo; q < hi; q++) r += s_v[q] > x ? 1u : 0u;
+        if (r >= take) continue;
+        if (out_keys) {
+          out_keys[r] = x;
+        } else {
+          out_ids[r] = key_id(x);
+          out_scores[r] = key_score(x);
+        }
+      }
+    } else {
+      uint64_t T = 1;  // every key
+      if (real > k) T = cta_radix_select<kFinalThreads>(keys, n, k, s_hist, s_misc);
+      uint32_t p2 = 1;
+      while (p2 < take) p2 <<= 1;
+      for (uint32_t base = 0; base < n; base += kFinalThreads) {
+        const uint32_t i = base + tid;
+        const uint64_t x = i < n ? __ldcg(keys + i) : 0ull;
+        const bool kp = x && x >= T;
+        const uint32_t pos = warp_append(kp, &s_n);
+        if (kp && pos < p2) s_v[pos] = x;
+      }
+      __syncthreads();
+      for (uint32_t i = take + tid; i < p2; i += kFinalThreads) s_v[i] = 0ull;
+      bitonic_sort_desc(s_v, p2);
+      for (uint32_t i = tid; i < take; i += kFinalThreads) {
+        if (out_keys) {
+          out_keys[i] = s_v[i];
+        } else {
+          out_ids[i] = key_id(s_v[i]);
+          out_scores[i] = key_score(s_v[i]);
+        }
+      }
+    }
   }
-  for (uint32_t i = threadIdx.x; i < k_out; i += kFinalThreads) {
+  for (uint32_t i = take + tid; i < k_out; i += kFinalThreads) {
     if (out_keys) {
-      out_keys[i] = i < take ? s_v[i] : 0ull;
-    } else if (i < take) {
-      out_ids[i] = key_id(s_v[i]);
-      out_scores[i] = key_score(s_v[i]);
+      out_keys[i] = 0ull;
     } else {
       out_ids[i] = 0xFFFFFFFFu;
       out_scores[i] = -INFINITY;
@@ -909,10 +1035,19 @@ __global__ void __launch_bounds__(kFinalThreads) k_final_select(
   }
 }
 
-// Shared-memory keys k_final_select buffers beyond its pow2(k) sort area.
-constexpr uint32_t kFinalBufKeys = 16384;
-constexpr size_t kFinalMaxSmem = (8192 + kFinalBufKeys) * 8;  // largest k is 8192
-static size_t final_smem(uint32_t p2) { return ((size_t)p2 + kFinalBufKeys) * 8; }
+// Lets k_final_select have the shared memory of the largest k (8192), on each
+// device once.
+static int final_select_init() {
+  static std::atomic<uint64_t> done{0};
+  int dev = 0;
+  EBR_CUDA_TRY(cudaGetDevice(&dev));
+  const uint64_t bit = dev < 64 ? 1ull << dev : 0ull;
+  if (done.load() & bit) return EBR_OK;
+  EBR_CUDA_TRY(cudaFuncSetAttribute(k_final_select, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    (int)final_smem(8192)));
+  done.fetch_or(bit);
+  return EBR_OK;
+}
 
 // FP32 rescoring of candidate keys: s = <h_u, h_a (FP32 copy)> + wide[a].
 // One warp per candidate; D <= 128.
@@ -1219,12 +1354,7 @@ int query_one(const ebr_index *cix, const ebr_cross *cross, const ebr_query &q, 
   const bool quant = ix->dtype != EBR_F32;
   const uint32_t k = q.k;
   const uint32_t kscan = quant ? std::min<uint32_t>(k * ix->rescore_mult, ix->n_ads) : k;
-  static bool attr_set = false;  // per process; the attribute applies to every device
-  if (!attr_set) {
-    EBR_CUDA_TRY(cudaFuncSetAttribute(k_final_select, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)kFinalMaxSmem));
-    attr_set = true;
-  }
+  EBR_TRY(final_select_init());
   ProfMarks pm(ix, st);
   EBR_CUDA_TRY(cudaMemsetAsync(ctrl, 0, kCtrlBytes + kHistWords * 4, st));  // + histogram
   const uint32_t *q_key = q.q_key;
@@ -1330,24 +1460,23 @@ int query_one(const ebr_index *cix, const ebr_cross *cross, const ebr_query &q, 
   pm.mark(3, st);
   const uint32_t p2 = pow2_at_least(std::max<uint32_t>(kscan, 1));
   if (!quant) {
-    EBR_CUDA_TRY(launch_pdl(k_final_select, 1, kFinalThreads, final_smem(p2), st,
+    EBR_CUDA_TRY(launch_pdl(k_final_select, 1, kFinalThreads, final_smem(k), st,
                             (const uint64_t *)w.cand.p, (const Ctrl *)ctrl, 0u, k, kmax, ids,
-                            scores, (uint64_t *)nullptr, kFinalBufKeys));
+                            scores, (uint64_t *)nullptr));
     ix->launches += 1;
   } else {
     // R*K candidates -> FP32 rescoring -> K
     const uint64_t *ck = (const uint64_t *)w.cand.p;
     uint64_t *sel = (uint64_t *)w.cand.p + (w.cand.bytes / 8 - 2 * (size_t)p2);
     uint64_t *res = sel + p2;
-    EBR_CUDA_TRY(launch_pdl(k_final_select, 1, kFinalThreads, final_smem(p2), st, ck,
+    EBR_CUDA_TRY(launch_pdl(k_final_select, 1, kFinalThreads, final_smem(kscan), st, ck,
                             (const Ctrl *)ctrl, 0u, kscan, kscan, (uint32_t *)nullptr,
-                            (float *)nullptr, sel, kFinalBufKeys));
+                            (float *)nullptr, sel));
     k_rescore<<<launch_grid((uint64_t)kscan * 32, 256, 4096), 256, 0, st>>>(
         sel, kscan, (const float *)ix->emb_f32.p, ix->d, q.h_u, (const float *)w.wide.p, res);
     EBR_CUDA_TRY(cudaGetLastError());
-    const uint32_t p2k = pow2_at_least(std::max<uint32_t>(std::min(k, kscan), 1));
-    k_final_select<<<1, kFinalThreads, final_smem(p2k), st>>>(res, nullptr, kscan, k, kmax, ids,
-                                                               scores, nullptr, kFinalBufKeys);
+    k_final_select<<<1, kFinalThreads, final_smem(k), st>>>(res, nullptr, kscan, k, kmax, ids,
+                                                             scores, nullptr);
     EBR_CUDA_TRY(cudaGetLastError());
     ix->launches += 3;
   }
@@ -1921,9 +2050,10 @@ namespace {
 
 constexpr uint32_t kNoAllocMaxK = 1024;     // largest K accepted
 constexpr uint32_t kNoAllocMaxGrid = 160;   // CTAs of the scan (>= SM count of a GB300)
-constexpr uint32_t kNoAllocCtrlWords = 8;   // 64 bytes reserved for the Ctrl block
+// reserved for the Ctrl block and the candidate-score histogram, in 8-byte words
+constexpr uint32_t kNoAllocCtrlWords = (kCtrlBytes + kHistWords * 4) / 8;
 constexpr size_t kNoAllocWords = kNoAllocCtrlWords + (size_t)kNoAllocMaxGrid * kNoAllocMaxK;
-// 8 * (8 + 160 * 1024) bytes = 1.25 MiB.
+// 256 + 16384 + 8 * 160 * 1024 bytes = 1.27 MiB.
 static __device__ __align__(256) unsigned long long g_noalloc_scratch[kNoAllocWords];
 
 constexpr int kNoAllocMaxDevices = 64;
@@ -1949,28 +2079,6 @@ void *current_context() {
   CUcontext c = nullptr;
   if (g_ctx_get_current(&c) != CUDA_SUCCESS) return nullptr;
   return reinterpret_cast<void *>(c);
-}
-
-template <int D>
-int noalloc_launch(const ScanArgs &a0, int sms, cudaStream_t st) {
-  using Sh = ScanShape<float, D>;
-  ScanArgs a = a0;
-  a.cap = a.k + std::max<uint32_t>(a.k, 2 * Sh::kTileRows);
-  a.cap = (a.cap + 255) / 256 * 256;
-  const size_t cand_bytes = (size_t)2 * a.cap * 8;
-  uint32_t stages = 4;
-  while (stages > 2 && cand_bytes + (size_t)stages * Sh::kStageBytes > 200 * 1024) stages--;
-  a.stages = stages;
-  const size_t smem = cand_bytes + (size_t)stages * Sh::kStageBytes;
-  const uint32_t n_tiles = (a.n_ads + Sh::kTileRows - 1) / Sh::kTileRows;
-  const int grid = (int)std::min<uint32_t>(std::min<uint32_t>((uint32_t)sms, kNoAllocMaxGrid),
-                                           n_tiles);
-  auto kern = k_scan_topk<float, D, MODE_TOPK>;
-  EBR_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    (int)smem));
-  kern<<<grid, kScanThreads, smem, st>>>(a);
-  EBR_CUDA_TRY(cudaGetLastError());
-  return EBR_OK;
 }
 
 }  // namespace
@@ -2038,37 +2146,38 @@ extern "C" int ebr_scan_topk_noalloc(const float *emb, uint32_t n_ads, uint32_t 
   uint64_t *cand = reinterpret_cast<uint64_t *>(base) + kNoAllocCtrlWords;
   int rc = EBR_OK;
   // The array keeps the previous call's contents: clear the control block.
-  cudaError_t e = cudaMemsetAsync(ctrl, 0, sizeof(Ctrl), st);
+  cudaError_t e = cudaMemsetAsync(ctrl, 0, kNoAllocCtrlWords * 8, st);
   if (e != cudaSuccess) {
     set_error("ebr_scan_topk_noalloc: %s", cudaGetErrorString(e));
     rc = EBR_ECUDA;
   }
+  if (rc == EBR_OK) rc = final_select_init();
+  // The forward scan's kernel without keys: its ring of 40 KB copies and its
+  // running bound from all CTAs' score counts.  What was here, 16 KB tiles and
+  // a CTA-wide meeting at each, read 777777 x 128 at 1.7 TB/s (232 us, and 87
+  // for a selection from every CTA's k); now 78 us in all, 5.1 TB/s.
   if (rc == EBR_OK) {
-    ScanArgs a;
-    memset(&a, 0, sizeof(a));
-    a.emb = emb;
-    a.h_u = h_u;
-    a.wide = wide;
-    a.filter = filter;
-    a.n_ads = n_ads;
-    a.k = k;
-    a.cand_out = cand;
-    a.ctrl = ctrl;
-    switch (d) {
-      case 4: rc = noalloc_launch<4>(a, sms, st); break;
-      case 8: rc = noalloc_launch<8>(a, sms, st); break;
-      case 16: rc = noalloc_launch<16>(a, sms, st); break;
-      case 32: rc = noalloc_launch<32>(a, sms, st); break;
-      case 64: rc = noalloc_launch<64>(a, sms, st); break;
-      default: rc = noalloc_launch<128>(a, sms, st); break;
-    }
+    FwdCall c;
+    memset(&c, 0, sizeof(c));
+    c.dtype = EBR_F32;
+    c.tree = true;
+    c.d = d;
+    c.n_ads = n_ads;
+    c.k = k;
+    c.emb = emb;
+    c.h_u = h_u;
+    c.quad_bytes = 256;
+    c.filter = filter;
+    c.cand_out = cand;
+    c.ctrl = ctrl;
+    c.hist = reinterpret_cast<uint32_t *>(reinterpret_cast<char *>(base) + kCtrlBytes);
+    c.wide_in = wide;
+    c.sms = std::min<int>(sms, kNoAllocMaxGrid);
+    rc = launch_forward(c, st);
   }
   if (rc == EBR_OK) {
-    uint32_t p2 = 1;
-    while (p2 < k) p2 <<= 1;
-    k_final_select<<<1, kFinalThreads, (size_t)p2 * 8, st>>>(cand, ctrl, 0, k, k, out_ids,
-                                                             out_scores, nullptr, 0u);
-    e = cudaGetLastError();
+    e = launch_pdl(k_final_select, 1, kFinalThreads, final_smem(k), st, (const uint64_t *)cand,
+                   (const Ctrl *)ctrl, 0u, k, k, out_ids, out_scores, (uint64_t *)nullptr);
     if (e != cudaSuccess) {
       set_error("ebr_scan_topk_noalloc: %s", cudaGetErrorString(e));
       rc = EBR_ECUDA;
