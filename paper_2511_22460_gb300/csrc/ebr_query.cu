@@ -1222,57 +1222,102 @@ static int run_wide(ebr_index *ix, const uint32_t *q_key, const float *q_w, uint
 // every field holds one value, users[b * f_u + i].  Pairs are summed in pair
 // order and a field's values in their order, as in the single-request
 // expansion, so both give the same FP32 w^.
-template <bool MULTI>
-__global__ void k_expand_T(CrossView cv, const uint32_t *__restrict__ users,
-                           const uint32_t *__restrict__ uptr, const uint32_t *__restrict__ base,
-                           uint32_t batch, uint32_t Bp, float *__restrict__ wT,
-                           uint32_t *__restrict__ flags, const uint32_t *__restrict__ batch_dev,
-                           const uint32_t *__restrict__ key_id) {
-  extern __shared__ uint32_t s_off2[];
+// A CTA takes 32 keys of one field for a group of 64 users, a thread eight of
+// them for one user: a pair and its user value are read once for eight hashes
+// and gathers, which do not wait for one another.  With a thread per (key,
+// user) the instructions around each gather bounded it.  Measured, REPLACE_EXP
+constexpr int kExpThreads = 256;
+constexpr uint32_t exp_tile(uint32_t keys) { return kExpThreads / 64 * keys; }
+template <bool MULTI, bool HASHED, uint32_t kExpKeys>
+__global__ void __launch_bounds__(kExpThreads)
+    k_expand_T(CrossView cv, const uint32_t *__restrict__ users,
+               const uint32_t *__restrict__ uptr, const uint32_t *__restrict__ base,
+               uint32_t batch, uint32_t Bp, float *__restrict__ wT, uint32_t *__restrict__ flags,
+               const uint32_t *__restrict__ batch_dev, const uint32_t *__restrict__ key_id) {
+  constexpr uint32_t kExpTile = exp_tile(kExpKeys);
+  extern __shared__ uint32_t s_off2[];          // key_off[f_a + 1]
+  uint32_t *s_tile = s_off2 + cv.f_a + 1;       // tiles before each field [f_a + 1]
   if (batch_dev) {  // a device-side loop: this wave's users (none: nothing to expand)
     batch = min(*batch_dev, batch);
     if (batch == 0) return;
   }
-  for (uint32_t j = threadIdx.x; j <= cv.f_a; j += blockDim.x) s_off2[j] = cv.key_off[j];
+  const uint32_t tid = threadIdx.x, lane = tid & 31;
+  for (uint32_t j = tid; j <= cv.f_a; j += kExpThreads) s_off2[j] = cv.key_off[j];
   __syncthreads();
-  const uint64_t total = (uint64_t)cv.n_keys * Bp;
-  uint32_t bad = 0;
-  for (uint64_t t = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; t < total;
-       t += (uint64_t)gridDim.x * blockDim.x) {
-    const uint32_t key = (uint32_t)(t / Bp), b = (uint32_t)(t % Bp);
-    float acc = 0.f;
-    if (b < batch) {
-      uint32_t lo = 0, hi = cv.f_a;
-      while (hi - lo > 1) {
-        const uint32_t mid = (lo + hi) >> 1;
-        if (s_off2[mid] <= key) lo = mid; else hi = mid;
+  if (tid < 32) {
+    uint32_t before = 0;
+    for (uint32_t j0 = 0; j0 < cv.f_a; j0 += 32) {
+      const uint32_t j = j0 + lane;
+      const uint32_t n = j < cv.f_a ? (s_off2[j + 1] - s_off2[j] + kExpTile - 1) / kExpTile : 0u;
+      uint32_t incl = n;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t x = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= (uint32_t)o) incl += x;
       }
-      const uint32_t j = lo, v = key - s_off2[j];
+      if (j < cv.f_a) s_tile[j] = before + incl - n;
+      before += __shfl_sync(0xffffffffu, incl, 31);
+    }
+    if (lane == 0) s_tile[cv.f_a] = before;
+  }
+  __syncthreads();
+  const uint32_t groups = Bp / 64, total = s_tile[cv.f_a] * groups;
+  const uint64_t mask = (1ull << cv.hash_bits) - 1ull;
+  uint32_t bad = 0;
+  for (uint32_t t = blockIdx.x; t < total; t += gridDim.x) {
+    const uint32_t g = t % groups, tile = t / groups;
+    uint32_t lo = 0, hi = cv.f_a;  // the field: last j with s_tile[j] <= tile
+    while (hi - lo > 1) {
+      const uint32_t mid = (lo + hi) >> 1;
+      if (s_tile[mid] <= tile) lo = mid; else hi = mid;
+    }
+    const uint32_t j = lo, V = s_off2[j + 1] - s_off2[j];
+    const uint32_t v0 = (tile - s_tile[j]) * kExpTile + (tid >> 6) * kExpKeys;
+    const uint32_t n_v = v0 < V ? min(kExpKeys, V - v0) : 0u;
+    if (n_v == 0) continue;
+    const uint32_t b = g * 64 + (tid & 63u);
+    float acc[kExpKeys];
+#pragma unroll
+    for (uint32_t e = 0; e < kExpKeys; e++) acc[e] = 0.f;
+    if (b < batch) {
       const uint32_t *up = MULTI ? uptr + (uint64_t)b * (cv.f_u + 1) : nullptr;
       const uint32_t ub = MULTI ? __ldg(base + b) : b * cv.f_u;
-      for (uint32_t q = cv.pair_ptr[j]; q < cv.pair_ptr[j + 1]; q++) {
-        const uint32_t p = cv.pair_of[q];
-        const uint32_t i = cv.pair_user[p];
+      const uint32_t q1 = __ldg(cv.pair_ptr + j + 1);
+      for (uint32_t q = __ldg(cv.pair_ptr + j); q < q1; q++) {
+        const uint32_t p = __ldg(cv.pair_of + q);
+        const uint32_t i = __ldg(cv.pair_user + p);
+        const uint32_t vu = __ldg(cv.vocab_u + i);
         const uint32_t r0 = MULTI ? ub + __ldg(up + i) : ub + i;
         const uint32_t r1 = MULTI ? ub + __ldg(up + i + 1) : r0 + 1;
         for (uint32_t r = r0; r < r1; r++) {
           const uint32_t u = __ldg(users + r);
-          if (u >= cv.vocab_u[i]) { bad |= DEVERR_BAD_USER; continue; }
-          float w;
-          if (cv.hashed) {
-            const uint64_t x = ((uint64_t)p << 40) | ((uint64_t)u << 20) | (uint64_t)v;
-            w = cv.table[splitmix64(x) & ((1ull << cv.hash_bits) - 1ull)];
+          if (u >= vu) { bad |= DEVERR_BAD_USER; continue; }
+          float w[kExpKeys];
+          if (HASHED) {
+            const uint64_t x = ((uint64_t)p << 40) | ((uint64_t)u << 20);
+#pragma unroll
+            for (uint32_t e = 0; e < kExpKeys; e++)  // (past the field: some other entry)
+              w[e] = __ldg(cv.table + (splitmix64(x | (uint64_t)(v0 + e)) & mask));
           } else {
-            const uint64_t off = ((uint64_t)cv.w_hi[p] << 32) | cv.w_lo[p];
-            w = cv.table[off + (uint64_t)u * cv.vocab_a[j] + v];
+            const float *row = cv.table + (((uint64_t)__ldg(cv.w_hi + p) << 32) | __ldg(cv.w_lo + p)) +
+                               (uint64_t)u * V + v0;
+#pragma unroll
+            for (uint32_t e = 0; e < kExpKeys; e++) w[e] = e < n_v ? __ldg(row + e) : 0.f;
           }
-          acc += w;
+#pragma unroll
+          for (uint32_t e = 0; e < kExpKeys; e++) acc[e] += w[e];
         }
       }
     }
     // per group of 64 users a slice of n_keys + 1 rows
-    const uint32_t row = key_id ? __ldg(key_id + key) : key;
-    wT[((uint64_t)(b >> 6) * ((uint64_t)cv.n_keys + 1) + row) * 64u + (b & 63u)] = acc;
+    float *out = wT + (uint64_t)g * ((uint64_t)cv.n_keys + 1) * 64u + (tid & 63u);
+    const uint32_t key0 = s_off2[j] + v0;
+#pragma unroll
+    for (uint32_t e = 0; e < kExpKeys; e++)
+      if (e < n_v) {
+        const uint32_t row = key_id ? __ldg(key_id + key0 + e) : key0 + e;
+        out[(uint64_t)row * 64u] = acc[e];
+      }
   }
   if (bad) atomicOr(flags, bad);
 }
@@ -1281,17 +1326,25 @@ int expand_transposed(const ebr_cross *c, const uint32_t *users, const uint32_t 
                       const uint32_t *base, uint32_t batch, uint32_t Bp, float *wT,
                       uint32_t *flags, cudaStream_t st, const uint32_t *batch_dev,
                       const uint32_t *key_id) {
-  CrossView cv = cross_view(c);
-  const uint64_t total = (uint64_t)cv.n_keys * Bp;
-  uint64_t blocks = (total + 255) / 256;
-  if (blocks > 65535) blocks = 65535;
-  const size_t smem = (c->f_a + 1) * 4;
-  if (uptr)
-    k_expand_T<true><<<(int)blocks, 256, smem, st>>>(cv, users, uptr, base, batch, Bp, wT, flags,
-                                                     batch_dev, key_id);
-  else
-    k_expand_T<false><<<(int)blocks, 256, smem, st>>>(cv, users, nullptr, nullptr, batch, Bp, wT,
-                                                      flags, batch_dev, key_id);
+  const CrossView cv = cross_view(c);
+  const uint64_t groups = Bp / 64;
+  const bool few = (cv.n_keys / exp_tile(8) + cv.f_a) * groups < 152 * 8;
+  const uint64_t tiles = (cv.n_keys / exp_tile(few ? 1 : 8) + cv.f_a) * groups;  // or fewer
+  const uint32_t blocks = (uint32_t)std::min<uint64_t>(tiles, 152 * 8);
+  const size_t smem = (size_t)2 * (c->f_a + 1) * 4;
+  auto pick = [&](auto multi, auto hashed) {
+    constexpr bool M = decltype(multi)::value, H = decltype(hashed)::value;
+    return few ? k_expand_T<M, H, 1> : k_expand_T<M, H, 8>;
+  };
+  const std::true_type yes;
+  const std::false_type no;
+  auto kern = uptr ? (cv.hashed ? pick(yes, yes) : pick(yes, no))
+                   : (cv.hashed ? pick(no, yes) : pick(no, no));
+  if (smem > 48 * 1024)
+    EBR_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      (int)std::min<size_t>(smem, 200 * 1024)));
+  kern<<<blocks, kExpThreads, smem, st>>>(cv, users, uptr, base, batch, Bp, wT, flags, batch_dev,
+                                          key_id);
   EBR_CUDA_TRY(cudaGetLastError());
   return EBR_OK;
 }
