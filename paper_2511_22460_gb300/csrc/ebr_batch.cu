@@ -366,7 +366,7 @@ __device__ __forceinline__ float2 lds_f2(uint32_t a) {
 struct BatchSmem {
   uint64_t a_full[2], a_empty[2], t_full[2], t_empty[2], l_full[2], l_empty[2], u_full;
   uint32_t tmem_base;
-  uint32_t cnt_u[kGroup];
+  uint32_t cnt_u[kGroup], trim_u[kGroup];
   uint32_t map_u[kGroup][kMapWords];  // this CTA's part of umap
   unsigned long long thr_u[kGroup];  // running threshold: the larger of the two bounds below
   unsigned long long cut_u[kGroup];  // cut of this CTA's own trims (0: nothing was trimmed)
@@ -546,20 +546,31 @@ __device__ uint64_t warp_radix_select(const CandEntry *buf, uint32_t n, uint32_t
 }
 
 // Stable in-place compaction of buf[0..n) to the entries with key >= T;
-// returns how many were kept.
-__device__ uint32_t warp_compact(CandEntry *buf, uint32_t n, uint64_t T) {
+// returns how many were kept.  Four entries a lane are in flight: the chain of
+// reads is what it costs (with one, the end of a CTA whose 61 users had 300
+// entries each took 85 us).
+__device__ __noinline__ uint32_t warp_compact(CandEntry *buf, uint32_t n, uint64_t T) {
+  constexpr int kU = 4;
   const int lane = threadIdx.x & 31;
   uint32_t kept = 0;
-  for (uint32_t b0 = 0; b0 < n; b0 += 32) {
-    const uint32_t i = b0 + lane;
-    CandEntry e;
-    e.key = 0;
-    if (i < n) e = buf[i];
-    const bool kp = i < n && e.key >= T;
-    const uint32_t bal = __ballot_sync(0xffffffffu, kp);
-    __syncwarp();
-    if (kp) buf[kept + __popc(bal & ((1u << lane) - 1u))] = e;
-    kept += __popc(bal);
+  for (uint32_t b0 = 0; b0 < n; b0 += 32 * kU) {
+    CandEntry e[kU];
+    uint32_t bal[kU];
+#pragma unroll
+    for (int u = 0; u < kU; u++) {
+      const uint32_t i = b0 + 32 * u + lane;
+      e[u].key = 0;
+      if (i < n) e[u] = buf[i];
+    }
+#pragma unroll
+    for (int u = 0; u < kU; u++)
+      bal[u] = __ballot_sync(0xffffffffu, b0 + 32 * u + lane < n && e[u].key >= T);
+    __syncwarp();  // every entry of the round is read before any is written
+#pragma unroll
+    for (int u = 0; u < kU; u++) {
+      if ((bal[u] >> lane) & 1u) buf[kept + __popc(bal[u] & ((1u << lane) - 1u))] = e[u];
+      kept += __popc(bal[u]);
+    }
     __syncwarp();
   }
   return kept;
@@ -638,6 +649,7 @@ __global__ void __launch_bounds__(kBatchThreads, 1) k_batch_window(const __grid_
 
   for (uint32_t b = tid; b < kGroup; b += kBatchThreads) {
     sm.cnt_u[b] = 0;
+    sm.trim_u[b] = 0;
     for (int i = 0; i < kMapWords; i++) sm.map_u[b][i] = 0;
     sm.thr_u[b] = 0ull;
     sm.cut_u[b] = 0ull;
@@ -865,6 +877,22 @@ __global__ void __launch_bounds__(kBatchThreads, 1) k_batch_window(const __grid_
         }
       } else {
         atomicOr(&a.ctrl->flags, DEVERR_OVERFLOW);
+      }
+    };
+    // the users marked keep the exact best m (the warps with a histogram)
+    auto trim_users = [&]() {
+      for (uint32_t b = warp; b < nG && warp < kTrimWarps; b += kTrimWarps) {
+        if (!sm.trim_u[b]) continue;
+        uint64_t T;
+        const uint32_t kept = warp_trim(user_buf(b), sm.cnt_u[b], a.m, whist + warp * 256, &T);
+        __syncwarp();
+        if (lane == 0) {
+          sm.cut_u[b] = max(sm.cut_u[b], (unsigned long long)T);
+          atomicMax(&sm.thr_u[b], (unsigned long long)T);
+          sm.cnt_u[b] = kept;
+          sm.trim_u[b] = 0;
+        }
+        __syncwarp();
       }
     };
     // The warps run free of each other (each hands the list and the
@@ -1121,22 +1149,17 @@ __global__ void __launch_bounds__(kBatchThreads, 1) k_batch_window(const __grid_
     if (sm.stop_epi || !sm.meet) break;
     // make room: drop what the running threshold excludes, then, if that is
     // not enough, keep the exact top-m by radix select
-    for (uint32_t b = warp; b < nG && warp < kTrimWarps; b += kTrimWarps) {
+    for (uint32_t b = warp; b < nG; b += kEpiWarps) {
       const uint32_t n = min(sm.cnt_u[b], a.cap_u);
       if (n + 2 * kBWin <= a.cap_u) continue;
-      CandEntry *buf = user_buf(b);
-      uint32_t kept = warp_compact(buf, n, sm.thr_u[b]);
-      if (kept + 3 * kBWin > a.cap_u && kept > a.m) {
-        uint64_t T;
-        kept = warp_trim(buf, kept, a.m, whist + warp * 256, &T);
-        if (lane == 0) {
-          sm.cut_u[b] = max(sm.cut_u[b], (unsigned long long)T);
-          atomicMax(&sm.thr_u[b], (unsigned long long)T);
-        }
+      const uint32_t kept = warp_compact(user_buf(b), n, sm.thr_u[b]);
+      if (lane == 0) {
+        sm.cnt_u[b] = kept;
+        sm.trim_u[b] = kept + 3 * kBWin > a.cap_u && kept > a.m;
       }
-      if (lane == 0) sm.cnt_u[b] = kept;
-      __syncwarp();
     }
+    gsync();
+    trim_users();
     gsync();
     }
     if (FWD) cp_async_wait();  // nothing in flight (after an abort) when the CTA ends
@@ -1147,19 +1170,17 @@ __global__ void __launch_bounds__(kBatchThreads, 1) k_batch_window(const __grid_
       for (uint32_t b = tid; b < nG; b += kEpiThreads)
         if (sm.cnt_u[b] > a.m) raise_threshold(a, sm, g0, b);
       gsync();
-      for (uint32_t b = warp; b < nG && warp < kTrimWarps; b += kTrimWarps) {
+      for (uint32_t b = warp; b < nG; b += kEpiWarps) {
         const uint32_t n = min(sm.cnt_u[b], a.cap_u);
         if (n <= a.m) continue;
-        CandEntry *buf = user_buf(b);
-        uint32_t kept = warp_compact(buf, n, sm.thr_u[b]);
-        if (kept > a.m) {
-          uint64_t T;
-          kept = warp_trim(buf, kept, a.m, whist + warp * 256, &T);
-          if (lane == 0) sm.cut_u[b] = max(sm.cut_u[b], (unsigned long long)T);
+        const uint32_t kept = warp_compact(user_buf(b), n, sm.thr_u[b]);
+        if (lane == 0) {
+          sm.cnt_u[b] = kept;
+          sm.trim_u[b] = kept > a.m;
         }
-        if (lane == 0) sm.cnt_u[b] = kept;
-        __syncwarp();
       }
+      gsync();
+      trim_users();
     }
     gsync();
     for (uint32_t b = tid; b < nG; b += kEpiThreads) {
@@ -1187,23 +1208,34 @@ __global__ void __launch_bounds__(kBatchThreads, 1) k_batch_window(const __grid_
 
 // Per user: the best R*K of the CTAs' candidate buffers (exact if no CTA's
 // buffer threshold exceeds the selected cut), rescored in FP32, best K.
+// One CTA per user, and what bounds it is the chain of its steps: reads of the
+// candidates a warp per buffer (a thread per buffer, then buffer after buffer by
+// all threads: 100 us), both selections by score bins, four rows in flight per
+// warp in the rescoring.  Measured, 2000 of 280k FP8 ads for 152 users (4000
+// rescored each) 311 us, now 87; 250 users, two rounds of CTAs, 610 and 174.
+// (CTAs of 512 threads, two to an SM, for more users than SMs: no gain.)
+// Dynamic shared memory: merge_smem(kscan, kout) for the largest of the batch.
 constexpr int kMergeThreads = 1024;
 constexpr uint32_t kMergeCap = 32768;  // approximate candidates gathered per user
+static size_t merge_smem(uint32_t ks, uint32_t ko) { return ((size_t)ks + sel_buf(ko)) * 8; }
 
 __global__ void __launch_bounds__(kMergeThreads) k_batch_merge(
     const CandEntry *__restrict__ cand, const uint32_t *__restrict__ cand_n,
     const unsigned long long *__restrict__ cand_thr, uint32_t grid, uint32_t B, uint32_t cap_u,
     const uint32_t *__restrict__ kscan, const uint32_t *__restrict__ kout, uint32_t kmax,
     const float *__restrict__ emb, uint32_t d, const float *__restrict__ h_u,
-    uint64_t *__restrict__ scratch /* [B][kMergeCap + 8192] */, uint32_t *__restrict__ out_ids,
+    uint64_t *__restrict__ scratch /* [B][kMergeCap] */, uint32_t *__restrict__ out_ids,
     float *__restrict__ out_scores, uint32_t *__restrict__ status /* [B] */,
     const uint32_t *__restrict__ B_dev, const uint32_t *__restrict__ slot_dev,
     uint64_t out_slot_stride, uint32_t status_slot_stride) {
-  extern __shared__ __align__(16) uint64_t s_v[];  // 8192 keys
-  __shared__ uint32_t s_hist[256], s_misc[8], s_cnt;
-  __shared__ uint32_t s_base[1024];
+  constexpr uint32_t NT = kMergeThreads, NW = NT / 32;
+  extern __shared__ __align__(16) uint64_t s_v[];  // [kscan], then the sort's buffer
+  __shared__ SelSmem s_sel;
+  __shared__ uint32_t s_hist[256], s_misc[8], s_cnt, s_ncut;
+  __shared__ uint64_t s_cut[kSelMaxBin], s_T;  // the keys of the cut's bin
+  __shared__ float s_cutw[kSelMaxBin];
   __shared__ float s_h[128];
-  const uint32_t b = blockIdx.x;
+  const uint32_t b = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   // a device-side loop: only the wave's active users, results into its ring slot
   if (B_dev && b >= *B_dev) return;
   if (slot_dev) {
@@ -1213,126 +1245,141 @@ __global__ void __launch_bounds__(kMergeThreads) k_batch_merge(
     status += (uint64_t)slot * status_slot_stride;
   }
   const uint32_t ks = kscan[b], ko = kout[b];
-  uint64_t *keys = scratch + (uint64_t)b * (kMergeCap + 8192);  // gathered approximate keys
-  uint32_t inexact = 0;
-  // 1. gather this user's candidates into scratch (bounded by 8192: with the
-  //    per-CTA thresholds far fewer survive; beyond that the request is flagged)
-  if (threadIdx.x == 0) s_cnt = 0;
+  if (tid == 0) {
+    s_cnt = 0;
+    s_ncut = 0;
+    s_T = 0;
+  }
   const uint64_t hrow = user_row(b);  // the user table is in pair order
-  for (uint32_t i = threadIdx.x; i < d; i += kMergeThreads) s_h[i] = h_u[hrow * d + i];
-  __syncthreads();
-  // count first, then copy (entries of all CTAs, in CTA order)
-  uint32_t total = 0;
-  for (uint32_t c0 = 0; c0 < grid; c0 += kMergeThreads) {
-    const uint32_t c = c0 + threadIdx.x;
-    const uint32_t n = c < grid ? cand_n[(uint64_t)c * B + b] : 0u;
-    // block-wide exclusive scan of n (simple two-level)
-    uint32_t incl = n;
-    const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
-    for (int o = 1; o < 32; o <<= 1) {
-      const uint32_t v = __shfl_up_sync(0xffffffffu, incl, o);
-      if (lane >= o) incl += v;
-    }
-    if (lane == 31) s_base[wp] = incl;
-    __syncthreads();
-    if (threadIdx.x < 32) {
-      uint32_t x = s_base[threadIdx.x], in2 = x;
-      for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t v = __shfl_up_sync(0xffffffffu, in2, o);
-        if (threadIdx.x >= o) in2 += v;
-      }
-      s_base[threadIdx.x] = in2 - x;
-      if (threadIdx.x == 31) s_misc[4] = in2;
-    }
-    __syncthreads();
-    const uint32_t start = total + s_base[wp] + incl - n;
-    if (c < grid) {
+  for (uint32_t i = tid; i < d; i += NT) s_h[i] = h_u[hrow * d + i];
+  // this user's candidates, a warp per CTA's buffer
+  auto for_entries = [&](auto f) {
+    for (uint32_t c = warp; c < grid; c += NW) {
+      const uint32_t n = __ldg(cand_n + (uint64_t)c * B + b);
       const CandEntry *src = cand + ((uint64_t)c * B + b) * cap_u;
-      for (uint32_t i = 0; i < n; i++)
-        if (start + i < kMergeCap) keys[start + i] = src[i].key;
+      for (uint32_t i = lane; i < n; i += 32)
+        if (src[i].key) f(src + i);
     }
-    total += s_misc[4];
+  };
+  auto add = [&](uint64_t key, float wide) {  // one more to rescore: (wide, id)
+    const uint32_t pos = atomicAdd(&s_cnt, 1u);
+    if (pos < ks) s_v[pos] = ((uint64_t)__float_as_uint(wide) << 32) | key_id(key);
+  };
+  // 1. the best ks by approximate score (T = 0: all of them)
+  const SelCut c1 = sel_cut<NT>(
+      s_sel, ks, [&](auto f) { for_entries([&](const CandEntry *e) { f(e->key); }); });
+  if (c1.real <= ks) {
+    for_entries([&](const CandEntry *e) { add(e->key, e->wide); });
+  } else if (!c1.crowded) {
+    for_entries([&](const CandEntry *e) {
+      const uint64_t x = e->key;
+      const uint32_t bin = c1.bin(x);
+      if (bin > c1.cut) {
+        add(x, e->wide);
+      } else if (bin == c1.cut) {
+        const uint32_t pos = atomicAdd(&s_ncut, 1u);
+        s_cut[pos] = x;
+        s_cutw[pos] = e->wide;
+      }
+    });
     __syncthreads();
+    const uint32_t n = s_ncut, need = ks - (c1.m - n);
+    if (tid < n) {
+      const uint64_t x = s_cut[tid];
+      uint32_t rank = 0;
+      for (uint32_t q = 0; q < n; q++) rank += s_cut[q] > x ? 1u : 0u;
+      if (rank < need) add(x, s_cutw[tid]);
+      if (rank == need - 1) s_T = x;
+    }
+  } else {
+    uint64_t *keys = scratch + (uint64_t)b * kMergeCap;
+    for_entries([&](const CandEntry *e) {
+      const uint32_t pos = atomicAdd(&s_ncut, 1u);
+      if (pos < kMergeCap) keys[pos] = e->key;
+    });
+    __syncthreads();
+    const uint64_t T = cta_radix_select<NT>(keys, min(s_ncut, kMergeCap), ks, s_hist, s_misc);
+    if (tid == 0) s_T = T;
+    for_entries([&](const CandEntry *e) {
+      if (e->key >= T) add(e->key, e->wide);
+    });
   }
-  if (total > kMergeCap) {
-    inexact = 1;
-    total = kMergeCap;
-  }
-  // 2. the best ks of them by approximate score (T = 0: all of them)
-  uint64_t T = 0;
-  if (total > ks) T = cta_radix_select<kMergeThreads>(keys, total, ks, s_hist, s_misc);
+  __syncthreads();
   // Exactness: CTA c holds every one of its candidates with key >= its
   // threshold, so the union's best ks are the inventory's best ks when no
   // threshold lies above the selected cut T.
-  for (uint32_t c = threadIdx.x; c < grid; c += kMergeThreads)
-    if (cand_thr[(uint64_t)c * B + b] > T) inexact = 1;
+  uint32_t inexact = c1.real > kMergeCap;
+  for (uint32_t c = tid; c < grid; c += NT)
+    if (cand_thr[(uint64_t)c * B + b] > s_T) inexact = 1;
   if (inexact) atomicOr(&status[b], 1u);
-  // 3. FP32 rescoring of the survivors: gather (id, wide) into shared
-  //    memory, then one warp per candidate (coalesced FP32 row read).
-  if (threadIdx.x == 0) s_cnt = 0;
-  __syncthreads();
-  uint64_t *resc = keys + kMergeCap;
-  for (uint32_t c = 0; c < grid; c++) {
-    const uint32_t n = cand_n[(uint64_t)c * B + b];
-    const CandEntry *src = cand + ((uint64_t)c * B + b) * cap_u;
-    for (uint32_t i = threadIdx.x; i < n; i += kMergeThreads) {
-      const CandEntry e = src[i];
-      if (e.key < T || e.key == 0ull) continue;
-      const uint32_t pos = atomicAdd(&s_cnt, 1u);
-      if (pos < 8192) s_v[pos] = ((uint64_t)__float_as_uint(e.wide) << 32) | key_id(e.key);
-    }
-  }
-  __syncthreads();
-  const uint32_t nres = min(s_cnt, 8192u);
-  {
-    const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
-    for (uint32_t i = wp; i < nres; i += kMergeThreads / 32) {
-      const uint64_t e = s_v[i];
-      const uint32_t id = (uint32_t)e;
-      const float *row = emb + (uint64_t)id * d;
-      float dot = 0.f;
-      for (uint32_t t = lane; t < d; t += 32) dot = fmaf(s_h[t], __ldg(row + t), dot);
-      for (int o = 16; o; o >>= 1) dot += __shfl_xor_sync(0xffffffffu, dot, o);
-      if (lane == 0) resc[i] = make_key(dot + __uint_as_float((uint32_t)(e >> 32)), id);
-    }
-  }
-  __syncthreads();
-  // 4. best ko, sorted
-  uint64_t T2 = 0;
-  if (nres > ko) T2 = cta_radix_select<kMergeThreads>(resc, nres, ko, s_hist, s_misc);
-  if (threadIdx.x == 0) s_cnt = 0;
-  __syncthreads();
-  const uint32_t take = min(nres, ko);
-  uint32_t p2 = 1;
-  while (p2 < take) p2 <<= 1;
-  for (uint32_t i = threadIdx.x; i < nres; i += kMergeThreads) {
-    const uint64_t x = resc[i];
-    if (x >= T2) {
-      const uint32_t pos = atomicAdd(&s_cnt, 1u);
-      if (pos < p2) s_v[pos] = x;
-    }
-  }
-  __syncthreads();
-  for (uint32_t i = take + threadIdx.x; i < p2; i += kMergeThreads) s_v[i] = 0ull;
-  // bitonic sort, descending
-  for (uint32_t size = 2; size <= p2; size <<= 1)
-    for (uint32_t stride = size >> 1; stride > 0; stride >>= 1) {
-      __syncthreads();
-      for (uint32_t i = threadIdx.x; i < p2 / 2; i += kMergeThreads) {
-        const uint32_t lo = 2 * i - (i & (stride - 1)), hi = lo + stride;
-        const bool desc = (lo & size) == 0;
-        const uint64_t x = s_v[lo], y = s_v[hi];
-        if ((x < y) == desc) {
-          s_v[lo] = y;
-          s_v[hi] = x;
-        }
+  // 2. FP32 rescoring, a warp per candidate (coalesced rows), in place
+  const uint32_t nres = min(s_cnt, ks);
+  auto rescore = [&](auto d32, auto per) {  // d / 32, candidates in flight per warp
+    constexpr int kT = decltype(d32)::value, kU = decltype(per)::value;
+    for (uint32_t i0 = warp * kU; i0 < nres; i0 += NW * kU) {
+      uint64_t e[kU];
+      float x[kU][kT], dot[kU];
+#pragma unroll
+      for (int u = 0; u < kU; u++) {
+        e[u] = s_v[i0 + u < nres ? i0 + u : i0];  // (this warp's own entries only)
+        const float *row = emb + (uint64_t)(uint32_t)e[u] * (32 * kT) + lane;
+#pragma unroll
+        for (int t = 0; t < kT; t++) x[u][t] = __ldg(row + 32 * t);
       }
+#pragma unroll
+      for (int u = 0; u < kU; u++) {
+        dot[u] = 0.f;
+#pragma unroll
+        for (int t = 0; t < kT; t++) dot[u] = fmaf(s_h[32 * t + lane], x[u][t], dot[u]);
+      }
+#pragma unroll
+      for (int o = 16; o; o >>= 1)
+#pragma unroll
+        for (int u = 0; u < kU; u++) dot[u] += __shfl_xor_sync(0xffffffffu, dot[u], o);
+      __syncwarp();
+#pragma unroll
+      for (int u = 0; u < kU; u++)
+        if (lane == (uint32_t)u && i0 + u < nres)
+          s_v[i0 + u] = make_key(dot[u] + __uint_as_float((uint32_t)(e[u] >> 32)), (uint32_t)e[u]);
     }
+  };
+  if (d == 64)
+    rescore(std::integral_constant<int, 2>(), std::integral_constant<int, 8>());
+  else
+    rescore(std::integral_constant<int, 4>(), std::integral_constant<int, 4>());
   __syncthreads();
-  for (uint32_t i = threadIdx.x; i < kmax; i += kMergeThreads) {
-    const uint64_t x = i < take ? s_v[i] : 0ull;
-    out_ids[(uint64_t)b * kmax + i] = i < take ? key_id(x) : 0xFFFFFFFFu;
-    out_scores[(uint64_t)b * kmax + i] = i < take ? key_score(x) : -INFINITY;
+  // 3. best ko, sorted
+  uint64_t *buf = s_v + ks;
+  auto for_resc = [&](auto f) {
+    for (uint32_t i = tid; i < nres; i += NT) f(s_v[i]);
+  };
+  auto emit = [&](uint32_t r, uint64_t x) {
+    out_ids[(uint64_t)b * kmax + r] = key_id(x);
+    out_scores[(uint64_t)b * kmax + r] = key_score(x);
+  };
+  const SelCut c2 = sel_cut<NT>(s_sel, ko, for_resc);
+  if (c2.take && !c2.crowded && c2.m <= sel_buf(ko)) {
+    sel_sorted<NT>(s_sel, c2, buf, for_resc, emit);
+  } else if (c2.take) {
+    uint64_t T2 = 0;
+    if (nres > ko) T2 = cta_radix_select<NT>(s_v, nres, ko, s_hist, s_misc);
+    if (tid == 0) s_ncut = 0;
+    __syncthreads();
+    uint32_t p2 = 1;
+    while (p2 < c2.take) p2 <<= 1;
+    for_resc([&](uint64_t x) {
+      if (x < T2) return;
+      const uint32_t pos = atomicAdd(&s_ncut, 1u);
+      if (pos < p2) buf[pos] = x;
+    });
+    __syncthreads();
+    for (uint32_t i = c2.take + tid; i < p2; i += NT) buf[i] = 0ull;
+    bitonic_sort_desc<NT>(buf, p2);
+    for (uint32_t i = tid; i < c2.take; i += NT) emit(i, buf[i]);
+  }
+  for (uint32_t i = c2.take + tid; i < kmax; i += NT) {
+    out_ids[(uint64_t)b * kmax + i] = 0xFFFFFFFFu;
+    out_scores[(uint64_t)b * kmax + i] = -INFINITY;
   }
 }
 
@@ -1565,7 +1612,7 @@ static bool batch_sizes(const ebr_index *ix, const ebr_cross *cross, uint32_t B,
   z->cand_n = ctas * B * 4;
   z->cand_thr = ctas * B * 8;
   z->uhist = user_hist_bytes(B);
-  z->scratch = (size_t)B * (kMergeCap + 8192) * 8;
+  z->scratch = (size_t)B * kMergeCap * 8;
   z->ctrl = sizeof(Ctrl);
   z->req = (size_t)B * sizeof(ReqSrc);
   // after the words: the pointer table (device requests) or the packed user
@@ -1826,9 +1873,10 @@ int batch_launch(ebr_index *ix, const ebr_cross *cross, const ebr_query *q, uint
   kern<<<dim3(grid, Bp / kGroup), kBatchThreads, pl.smem, st>>>(a);
   EBR_CUDA_TRY(cudaGetLastError());
   if (prof) EBR_CUDA_TRY(cudaEventRecord(ev[2], st));
+  const size_t msm = merge_smem(kscan_max, kmax);
   EBR_CUDA_TRY(cudaFuncSetAttribute(k_batch_merge, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    8192 * 8));
-  k_batch_merge<<<B, kMergeThreads, 8192 * 8, st>>>(
+                                    (int)msm));
+  k_batch_merge<<<B, kMergeThreads, msm, st>>>(
       (const CandEntry *)w.cand.p, (const uint32_t *)w.cand_n.p,
       (const unsigned long long *)w.cand_thr.p, (uint32_t)grid, B, pl.cap_u, kk, kk + B, kmax,
       (const float *)ix->emb_f32.p, d, (const float *)w.users_f32.p,
@@ -2140,8 +2188,9 @@ int loop_build(ebr_index *ix, const ebr_cross *cross, uint32_t max_user_vals, Ba
   auto kern = window_kernel(f8, pl.mode);
   EBR_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                     (int)pl.smem));
+  const size_t msm = merge_smem(kscan_max, L.kmax);
   EBR_CUDA_TRY(cudaFuncSetAttribute(k_batch_merge, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    8192 * 8));
+                                    (int)msm));
   LoopArgs la;
   memset(&la, 0, sizeof(la));
   la.nsw = 0;  // 64, 128, ... and, last, the table's own width
@@ -2235,7 +2284,7 @@ int loop_build(ebr_index *ix, const ebr_cross *cross, uint32_t max_user_vals, Ba
       clear_zero_rows(ix, w, Bp, st);
       cudaMemsetAsync(w.uhist.p, 0, user_hist_bytes(Bmax), st);
       kern<<<dim3(grid, Bp / kGroup), kBatchThreads, pl.smem, st>>>(ba);
-      k_batch_merge<<<std::min(Bmax, Bp), kMergeThreads, 8192 * 8, st>>>(
+      k_batch_merge<<<std::min(Bmax, Bp), kMergeThreads, msm, st>>>(
           (const CandEntry *)w.cand.p, (const uint32_t *)w.cand_n.p,
           (const unsigned long long *)w.cand_thr.p, (uint32_t)grid, Bmax, pc.cap_u, ks, ko,
           L.kmax, (const float *)ix->emb_f32.p, d, (const float *)w.users_f32.p,

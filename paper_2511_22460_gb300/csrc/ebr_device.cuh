@@ -233,6 +233,159 @@ __device__ uint64_t cta_radix_select(const uint64_t *buf, uint32_t n, uint32_t n
   return group_radix_select<NT>(buf, n, need, hist, s_misc, threadIdx.x, CtaSync());
 }
 
+// ------------------------------------------------- selection by score bins
+// Keys placed by kSelBins equal bins between the smallest and the largest score:
+// the counts give each bin its place in the descending order and the bin that
+// holds the k-th key.  A CTA of NT threads; every thread calls.
+constexpr uint32_t kSelBins = 4096;
+constexpr uint32_t kSelMaxBin = 192;  // keys of a bin that are ranked one by one
+// Entries of the buffer that the k best are sorted in (a power of two for the
+// bitonic sort; room for the cut's bin).
+inline __host__ __device__ uint32_t sel_buf(uint32_t k) {
+  uint32_t p = 1;
+  while (p < k) p <<= 1;
+  return p > k + kSelMaxBin ? p : k + kSelMaxBin;
+}
+
+struct SelSmem {
+  uint32_t cnt[kSelBins];   // keys of each bin
+  uint32_t base[kSelBins];  // keys in higher bins (of the bins down to the cut)
+  uint32_t w[3][32];
+  uint32_t cut, m, crowded;
+};
+
+struct SelCut {
+  uint32_t real, take;    // keys that are not zero, min(real, k)
+  uint32_t cut, m;        // bin of the take-th key, keys in it and above
+  bool crowded;           // a bin down to the cut holds more than kSelMaxBin keys
+  uint32_t mn, shift;
+  float lo, scale;
+  bool finite;            // else bins of the scores' ordered integers
+  // monotone: subtraction, product and conversion round monotonically
+  __device__ __forceinline__ uint32_t bin(uint64_t x) const {
+    const uint32_t h = (uint32_t)(x >> 32);
+    if (!finite) return (h - mn) >> shift;
+    return min((uint32_t)((unord_f32(h) - lo) * scale), kSelBins - 1);
+  }
+};
+
+// for_keys(f) calls f(key) for this thread's share of the keys, none of them
+// zero, twice here.
+template <int NT, typename F>
+__device__ __forceinline__ SelCut sel_cut(SelSmem &s, uint32_t k, F for_keys) {
+  constexpr uint32_t NW = NT / 32, kPer = kSelBins / NT;
+  const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  SelCut r;
+  for (uint32_t i = tid; i < kSelBins; i += NT) s.cnt[i] = 0;
+  if (tid == 0) s.crowded = 0;
+  uint32_t mn = 0xFFFFFFFFu, mx = 0, real = 0;
+  for_keys([&](uint64_t x) {
+    const uint32_t h = (uint32_t)(x >> 32);
+    mn = min(mn, h);
+    mx = max(mx, h);
+    real++;
+  });
+  mn = __reduce_min_sync(0xffffffffu, mn);
+  mx = __reduce_max_sync(0xffffffffu, mx);
+  real = __reduce_add_sync(0xffffffffu, real);
+  if (lane == 0) {
+    s.w[0][warp] = mn;
+    s.w[1][warp] = mx;
+    s.w[2][warp] = real;
+  }
+  __syncthreads();
+  mn = __reduce_min_sync(0xffffffffu, lane < NW ? s.w[0][lane] : 0xFFFFFFFFu);
+  mx = __reduce_max_sync(0xffffffffu, lane < NW ? s.w[1][lane] : 0u);
+  r.real = __reduce_add_sync(0xffffffffu, lane < NW ? s.w[2][lane] : 0u);
+  r.take = min(r.real, k);
+  r.cut = r.m = 0;
+  r.crowded = false;
+  if (r.take == 0) return r;
+  r.mn = mn;
+  r.lo = unord_f32(mn);
+  const float range = unord_f32(mx) - r.lo;
+  r.finite = range < INFINITY;
+  r.scale = range > 0.f ? fminf((float)kSelBins / range, 3e38f) : 0.f;
+  r.shift = max(20 - (int)__clz(mx - mn), 0);  // (clz(0) = 32)
+  for_keys([&](uint64_t x) { atomicAdd(&s.cnt[r.bin(x)], 1u); });
+  __syncthreads();
+  {
+    // a thread has kPer bins, from the top; the keys in the bins above
+    const uint32_t top = kSelBins - 1 - kPer * tid;
+    uint32_t c[kPer], sum = 0;
+#pragma unroll
+    for (uint32_t e = 0; e < kPer; e++) {
+      c[e] = s.cnt[top - e];
+      sum += c[e];
+    }
+    uint32_t incl = sum;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= (uint32_t)o) incl += y;
+    }
+    if (lane == 31) s.w[0][warp] = incl;
+    __syncthreads();
+    uint32_t above = __reduce_add_sync(0xffffffffu, lane < warp ? s.w[0][lane] : 0u) + incl - sum;
+#pragma unroll
+    for (uint32_t e = 0; e < kPer; e++) {
+      s.base[top - e] = above;
+      if (above < r.take) {
+        if (c[e] > kSelMaxBin) s.crowded = 1;
+        if (above + c[e] >= r.take) {
+          s.cut = top - e;
+          s.m = above + c[e];
+        }
+      }
+      above += c[e];
+    }
+  }
+  __syncthreads();
+  r.cut = s.cut;
+  r.m = s.m;
+  r.crowded = s.crowded != 0u;
+  return r;
+}
+
+// The take best keys in order: emit(rank, key).  Not crowded; buf holds r.m
+// keys.  Scatters the keys by bin (for_keys once more), then each counts the
+// larger keys of its own bin.
+template <int NT, typename F, typename E>
+__device__ __forceinline__ void sel_sorted(SelSmem &s, const SelCut &r, uint64_t *buf, F for_keys,
+                                           E emit) {
+  for_keys([&](uint64_t x) {
+    const uint32_t b = r.bin(x);
+    if (b >= r.cut) buf[s.base[b] + atomicSub(&s.cnt[b], 1u) - 1u] = x;
+  });
+  __syncthreads();
+  for (uint32_t p = threadIdx.x; p < r.m; p += NT) {
+    const uint64_t x = buf[p];
+    const uint32_t b = r.bin(x), lo = s.base[b], hi = b == r.cut ? r.m : s.base[b - 1];
+    uint32_t rank = lo;
+    for (uint32_t q = lo; q < hi; q++) rank += buf[q] > x ? 1u : 0u;
+    if (rank < r.take) emit(rank, x);
+  }
+}
+
+// Sorts v[0..n_pow2) descending (shared memory, bitonic, any CTA width).
+template <int NT>
+__device__ void bitonic_sort_desc(uint64_t *v, uint32_t n_pow2) {
+  for (uint32_t size = 2; size <= n_pow2; size <<= 1)
+    for (uint32_t stride = size >> 1; stride > 0; stride >>= 1) {
+      __syncthreads();
+      for (uint32_t i = threadIdx.x; i < n_pow2 / 2; i += NT) {
+        const uint32_t lo = 2 * i - (i & (stride - 1)), hi = lo + stride;
+        const bool desc = (lo & size) == 0;
+        const uint64_t x = v[lo], y = v[hi];
+        if ((x < y) == desc) {
+          v[lo] = y;
+          v[hi] = x;
+        }
+      }
+    }
+  __syncthreads();
+}
+
 // ---------------------------------------------- histogram threshold (K-th bound)
 // hist_c[256] counts candidates by the top 8 bits of ord(score), hist_f[65536]
 // by the top 16 bits.  Every counted candidate is a distinct ad, so if at

@@ -834,70 +834,33 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_topk(ScanArgs a) {
 // =====================================================================
 constexpr int kFinalThreads = 1024;
 
-__device__ void bitonic_sort_desc(uint64_t *v, uint32_t n_pow2) {
-  for (uint32_t size = 2; size <= n_pow2; size <<= 1) {
-    for (uint32_t stride = size >> 1; stride > 0; stride >>= 1) {
-      __syncthreads();
-      for (uint32_t i = threadIdx.x; i < n_pow2 / 2; i += blockDim.x) {
-        const uint32_t lo = 2 * i - (i & (stride - 1));
-        const uint32_t hi = lo + stride;
-        const bool desc = ((lo & size) == 0);
-        const uint64_t x = v[lo], y = v[hi];
-        if ((x < y) == desc) {
-          v[lo] = y;
-          v[hi] = x;
-        }
-      }
-    }
-  }
-  __syncthreads();
-}
-
 // Selects the best min(k, n) keys among n (global memory; zero keys are absent
 // ones) and writes k_out ids/scores sorted descending, padded with
 // (0xFFFFFFFF, -inf), or the keys themselves, padded with zero keys.
 // One CTA, so what bounds it is the chain of barriers: a radix select of 8-bit
-// digits and a bitonic sort met 30 to 100 times.  Instead the scores are put
-// in 4096 equal bins between the smallest and the largest, one scan over the
-// bins gives each its place in the order and the bin that holds the k-th key,
-// the keys of that bin and above are scattered to their bins, and each counts
-// the larger keys of its own bin: six barriers.  Keys crowded into a few bins
-// (equal scores, mostly) take the radix select and the bitonic sort.  Measured: REPLACE_FINAL
+// digits and a bitonic sort met 30 to 100 times, placing the keys by score bins
+// (sel_cut, sel_sorted) six.  Keys crowded into a few bins (equal scores, mostly)
+// take the radix select and the bitonic sort.  Measured, a request of 1000 of
+// 10M FP8 ads (two of these, 48 us each) 388 -> 347 us, 500 of 2M FP32 139 ->
+// 129, 100 of 10k 33 -> 28.
 // Dynamic shared memory: final_smem(k).
 // Waits (pdl_wait) for the kernel before it in the stream.  (keys and ctrl are
 // not __restrict__: a load through such a pointer may be moved above the wait.)
-constexpr uint32_t kFinalBins = 4096, kFinalMaxBin = 192;
-static_assert(kFinalThreads == 1024, "a warp's lanes hold the warps' values");
 constexpr int kFinalRegs = 8;  // keys per thread held in registers between the passes
-static __host__ __device__ uint32_t final_cap(uint32_t k) {  // entries of the scattered keys
-  uint32_t p = 1;
-  while (p < k) p <<= 1;
-  return max(p, k + 1024u);
-}
-static size_t final_smem(uint32_t k) { return (size_t)final_cap(k) * 8 + kFinalBins * 8; }
+static size_t final_smem(uint32_t k) { return (size_t)sel_buf(k) * 8; }
 
 __global__ void __launch_bounds__(kFinalThreads) k_final_select(
     const uint64_t *keys, const Ctrl *ctrl, uint32_t n_fixed,
     uint32_t k, uint32_t k_out, uint32_t *__restrict__ out_ids, float *__restrict__ out_scores,
     uint64_t *__restrict__ out_keys) {
   extern __shared__ __align__(16) uint64_t s_v[];
-  const uint32_t cap = final_cap(k);
-  uint32_t *s_cnt = reinterpret_cast<uint32_t *>(s_v + cap);  // keys of each bin
-  uint32_t *s_base = s_cnt + kFinalBins;                      // keys in higher bins
-  __shared__ uint32_t s_hist[256], s_misc[8];
-  __shared__ uint32_t s_w[3][32];
-  __shared__ uint32_t s_bin, s_m, s_crowded, s_n;
-  const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  for (uint32_t i = tid; i < kFinalBins; i += kFinalThreads) s_cnt[i] = 0;
-  if (tid == 0) {
-    s_crowded = 0;
-    s_n = 0;
-  }
+  __shared__ SelSmem s_sel;
+  __shared__ uint32_t s_hist[256], s_misc[8], s_n;
+  const uint32_t tid = threadIdx.x;
+  if (tid == 0) s_n = 0;
   pdl_wait();
   const uint32_t n = ctrl ? *((const volatile uint32_t *)&ctrl->n_cand) : n_fixed;
-  // pass 1: smallest and largest score, number of keys
   uint64_t reg[kFinalRegs];
-  uint32_t mn = 0xFFFFFFFFu, mx = 0, real = 0;
 #pragma unroll
   for (int e = 0; e < kFinalRegs; e++) {
     const uint32_t i = tid + e * kFinalThreads;
@@ -912,120 +875,35 @@ __global__ void __launch_bounds__(kFinalThreads) k_final_select(
       if (x) f(x);
     }
   };
-  for_keys([&](uint64_t x) {
-    const uint32_t h = (uint32_t)(x >> 32);
-    mn = min(mn, h);
-    mx = max(mx, h);
-    real++;
-  });
-  mn = __reduce_min_sync(0xffffffffu, mn);
-  mx = __reduce_max_sync(0xffffffffu, mx);
-  real = __reduce_add_sync(0xffffffffu, real);
-  if (lane == 0) {
-    s_w[0][warp] = mn;
-    s_w[1][warp] = mx;
-    s_w[2][warp] = real;
-  }
-  __syncthreads();
-  mn = __reduce_min_sync(0xffffffffu, s_w[0][lane]);
-  mx = __reduce_max_sync(0xffffffffu, s_w[1][lane]);
-  real = __reduce_add_sync(0xffffffffu, s_w[2][lane]);
-  const uint32_t take = min(real, k);
-  if (take) {
-    const float lo_s = unord_f32(mn), range = unord_f32(mx) - lo_s;
-    const bool finite = range < INFINITY;  // else bins of the ordered integers
-    const float scale = range > 0.f ? fminf((float)kFinalBins / range, 3e38f) : 0.f;
-    const uint32_t shift = max(20 - (int)__clz(mx - mn), 0);  // (clz(0) = 32)
-    // monotone: subtraction, product and conversion round monotonically
-    auto bin_of = [&](uint64_t x) {
-      const uint32_t h = (uint32_t)(x >> 32);
-      if (!finite) return (h - mn) >> shift;
-      return min((uint32_t)((unord_f32(h) - lo_s) * scale), kFinalBins - 1);
-    };
-    // pass 2: keys per bin, then (a thread has four bins, from the top) the
-    // keys in the bins above
-    for_keys([&](uint64_t x) { atomicAdd(&s_cnt[bin_of(x)], 1u); });
-    __syncthreads();
-    {
-      constexpr uint32_t kPer = kFinalBins / kFinalThreads;
-      const uint32_t top = kFinalBins - 1 - kPer * tid;
-      uint32_t c[kPer], sum = 0;
-#pragma unroll
-      for (uint32_t e = 0; e < kPer; e++) {
-        c[e] = s_cnt[top - e];
-        sum += c[e];
-      }
-      uint32_t incl = sum;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= (uint32_t)o) incl += y;
-      }
-      if (lane == 31) s_w[0][warp] = incl;
-      __syncthreads();
-      uint32_t above = __reduce_add_sync(0xffffffffu, lane < warp ? s_w[0][lane] : 0u) + incl - sum;
-#pragma unroll
-      for (uint32_t e = 0; e < kPer; e++) {
-        s_base[top - e] = above;
-        if (above < take) {
-          if (c[e] > kFinalMaxBin) s_crowded = 1;
-          if (above + c[e] >= take) {
-            s_bin = top - e;
-            s_m = above + c[e];
-          }
-        }
-        above += c[e];
-      }
-    }
-    __syncthreads();
-    const uint32_t cut = s_bin, m = s_m;
-    if (!s_crowded && m <= cap) {
-      // pass 3: the keys of the cut's bin and above, by bin; then each key's
-      // place among its bin's
-      for_keys([&](uint64_t x) {
-        const uint32_t b = bin_of(x);
-        if (b >= cut) s_v[s_base[b] + atomicSub(&s_cnt[b], 1u) - 1u] = x;
-      });
-      __syncthreads();
-      for (uint32_t p = tid; p < m; p += kFinalThreads) {
-        const uint64_t x = s_v[p];
-        const uint32_t b = bin_of(x), lo = s_base[b], hi = b == cut ? m : s_base[b - 1];
-        uint32_t r = lo;
-        for (uint32_t q = lo; q < hi; q++) r += s_v[q] > x ? 1u : 0u;
-        if (r >= take) continue;
-        if (out_keys) {
-          out_keys[r] = x;
-        } else {
-          out_ids[r] = key_id(x);
-          out_scores[r] = key_score(x);
-        }
-      }
+  auto emit = [&](uint32_t r, uint64_t x) {
+    if (out_keys) {
+      out_keys[r] = x;
     } else {
-      uint64_t T = 1;  // every key
-      if (real > k) T = cta_radix_select<kFinalThreads>(keys, n, k, s_hist, s_misc);
-      uint32_t p2 = 1;
-      while (p2 < take) p2 <<= 1;
-      for (uint32_t base = 0; base < n; base += kFinalThreads) {
-        const uint32_t i = base + tid;
-        const uint64_t x = i < n ? __ldcg(keys + i) : 0ull;
-        const bool kp = x && x >= T;
-        const uint32_t pos = warp_append(kp, &s_n);
-        if (kp && pos < p2) s_v[pos] = x;
-      }
-      __syncthreads();
-      for (uint32_t i = take + tid; i < p2; i += kFinalThreads) s_v[i] = 0ull;
-      bitonic_sort_desc(s_v, p2);
-      for (uint32_t i = tid; i < take; i += kFinalThreads) {
-        if (out_keys) {
-          out_keys[i] = s_v[i];
-        } else {
-          out_ids[i] = key_id(s_v[i]);
-          out_scores[i] = key_score(s_v[i]);
-        }
-      }
+      out_ids[r] = key_id(x);
+      out_scores[r] = key_score(x);
     }
+  };
+  const SelCut c = sel_cut<kFinalThreads>(s_sel, k, for_keys);
+  if (c.take && !c.crowded && c.m <= sel_buf(k)) {
+    sel_sorted<kFinalThreads>(s_sel, c, s_v, for_keys, emit);
+  } else if (c.take) {
+    uint64_t T = 1;  // every key
+    if (c.real > k) T = cta_radix_select<kFinalThreads>(keys, n, k, s_hist, s_misc);
+    uint32_t p2 = 1;
+    while (p2 < c.take) p2 <<= 1;
+    for (uint32_t base = 0; base < n; base += kFinalThreads) {
+      const uint32_t i = base + tid;
+      const uint64_t x = i < n ? __ldcg(keys + i) : 0ull;
+      const bool kp = x && x >= T;
+      const uint32_t pos = warp_append(kp, &s_n);
+      if (kp && pos < p2) s_v[pos] = x;
+    }
+    __syncthreads();
+    for (uint32_t i = c.take + tid; i < p2; i += kFinalThreads) s_v[i] = 0ull;
+    bitonic_sort_desc<kFinalThreads>(s_v, p2);
+    for (uint32_t i = tid; i < c.take; i += kFinalThreads) emit(i, s_v[i]);
   }
-  for (uint32_t i = take + tid; i < k_out; i += kFinalThreads) {
+  for (uint32_t i = c.take + tid; i < k_out; i += kFinalThreads) {
     if (out_keys) {
       out_keys[i] = 0ull;
     } else {

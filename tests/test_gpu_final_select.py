@@ -114,3 +114,28 @@ def test_noalloc_inner_products(n, d):
     if left.size:
         assert np.all(ref[left] - tol[left] <= sc[-1])
     assert np.all(np.diff(sc) <= 0)
+
+
+@pytest.mark.parametrize("kind", ["normal", "equal", "few", "outlier", "rising"])
+@pytest.mark.parametrize("n,k,B", [(5_000, 100, 3), (40, 64, 2), (9_000, 2000, 160)])
+def test_batch_selects_what_a_sort_does(kind, n, k, B):
+    rng = np.random.default_rng(n + k)
+    s = torch.from_numpy(_scores(kind, n, rng)).bfloat16().float().numpy()  # exact in the table
+    emb = np.zeros((n, 64), np.float32)
+    emb[:, 1] = s
+    ix = ebr.build_index(n, 4, np.array([3], np.uint32), np.array([0], np.uint32), emb,
+                         dtype="bf16")
+    cross = ebr.cross_create([2], [4], [(0, 0)], np.zeros(16, np.float32), hashed=True, hash_bits=4)
+    h = torch.zeros((B, 64), device=DEV)
+    h[:, 1] = torch.tensor([1.0 if b % 2 else -1.0 for b in range(B)], device=DEV)
+    users = torch.zeros((B, 1), dtype=torch.int32, device=DEV)
+    ids = torch.full((B, k), -7, dtype=torch.int32, device=DEV)
+    sc = torch.full((B, k), float("nan"), device=DEV)
+    ebr.score_topk(ix, cross, [ebr.Query(h_u=h[b], k=k, user_vals=users[b]) for b in range(B)],
+                   ids, sc)
+    torch.cuda.synchronize()
+    ids, sc = ids.cpu().numpy().view(np.uint32), sc.cpu().numpy()
+    for b in range(B):
+        want, want_sc = _want(s if b % 2 else -s, k)
+        assert np.array_equal(sc[b], want_sc)
+        assert np.array_equal(ids[b], want)
