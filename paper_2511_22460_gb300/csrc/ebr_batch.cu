@@ -958,6 +958,26 @@ __global__ void __launch_bounds__(kBatchThreads, 1) k_batch_window(const __grid_
       __syncwarp();
       return last;
     };
+    // A window starts when every warp has handed back the accumulators and the
+    // list that it needs: what is waited for after that comes without the other
+    // epilogue warps.  (They may be in a meeting, which this warp has to join: 2.)
+    // 0: abort.
+    auto may_start = [&](uint32_t w) -> uint32_t {
+      const uint32_t tb = w % a.tb, lbuf = w % a.lb;
+      const uint64_t t0 = global_timer_ns();
+      for (;;) {
+        if (*((volatile uint32_t *)&sm.abort)) return 0;
+        if ((w < a.tb || mbar_try_wait(&sm.t_empty[tb], ((w / a.tb) - 1) & 1u)) &&
+            (FWD || w < a.lb || mbar_try_wait(&sm.l_empty[lbuf], ((w / a.lb) - 1) & 1u)))
+          return 1;
+        if (*((volatile uint32_t *)&sm.trim)) return 2;
+        if (global_timer_ns() - t0 > kWaitTimeoutNs) {
+          atomicOr(&a.ctrl->flags, DEVERR_TIMEOUT);
+          sm.abort = 1;
+          return 0;
+        }
+      }
+    };
     read_offsets(0);
     fetch_quads(0);
     read_offsets(1);
@@ -973,10 +993,13 @@ __global__ void __launch_bounds__(kBatchThreads, 1) k_batch_window(const __grid_
       const uint32_t tb = j % a.tb, lbuf = j % a.lb;
       uint32_t rows, tab_a;  // rows of the list, and its first entry of this warp's ads
       constexpr uint32_t kRowEntries = FWD ? kWarpAds : 32;
+      const uint32_t go = __shfl_sync(0xffffffffu, lane == 0 ? may_start(j) : 0u, 0);
+      if (go == 2) break;  // a meeting comes first
+      if (go == 0) {
+        j = my_wins;
+        break;
+      }
       if (FWD) {
-        if (*((volatile uint32_t *)&sm.abort)) j = my_wins;
-        j = __shfl_sync(0xffffffffu, j, 0);
-        if (j >= my_wins) break;
         rows = make_list();
         tab_a = list_a;
         fetch_quads(j + 1);

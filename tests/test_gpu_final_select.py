@@ -73,7 +73,7 @@ def test_noalloc_selects_what_a_sort_does(kind, n, k, d):
 
 
 @pytest.mark.parametrize("kind", ["normal", "equal", "few", "outlier", "rising"])
-@pytest.mark.parametrize("n,k", [(9_000, 8192), (300, 8192), (150_000, 8191), (150_000, 2049)])
+@pytest.mark.parametrize("n,k", [(9_000, 8192), (300, 8192), (150_000, 8191), (150_000, 2049), (800_000, 20)])
 def test_request_selects_what_a_sort_does(kind, n, k):
     rng = np.random.default_rng(n + k)
     s = _scores(kind, n, rng)
@@ -117,7 +117,7 @@ def test_noalloc_inner_products(n, d):
 
 
 @pytest.mark.parametrize("kind", ["normal", "equal", "few", "outlier", "rising"])
-@pytest.mark.parametrize("n,k,B", [(5_000, 100, 3), (40, 64, 2), (9_000, 2000, 160)])
+@pytest.mark.parametrize("n,k,B", [(5_000, 100, 3), (40, 64, 2), (9_000, 2000, 160), (200_000, 50, 64)])
 def test_batch_selects_what_a_sort_does(kind, n, k, B):
     rng = np.random.default_rng(n + k)
     s = torch.from_numpy(_scores(kind, n, rng)).bfloat16().float().numpy()  # exact in the table
