@@ -172,6 +172,7 @@ struct FwdSmem {
   uint32_t hist[256], misc[8], wtot[2][kMaxConsWarps];
   unsigned long long thr;
   uint32_t n, n_seen, abort, stop, top_bin;
+  uint32_t issued;  // stages whose copies the producer has issued
   uint32_t trim, meet, finished;  // trim asked for; what a meeting of the warps is for; all done
 };
 
@@ -214,15 +215,26 @@ struct TermSum {
   }
 };
 
-// Wait for the stage in ring slot s, turn `turn` of the ring.  A warp does not
-// visit every slot in every turn, so it may get here before the turn before has
-// even arrived, where the parity of the full barrier alone would pass for this
-// turn's.  It waits for the slot to be handed back first: at most S * runs
-// warps work, so the turn before is issued by now and that wait's parity is not
-// ambiguous, and once it is over the turn before has arrived.
-__device__ __forceinline__ bool wait_stage(FwdSmem &sm, uint32_t s, uint32_t turn) {
-  if (turn && !mbar_wait_bounded(&sm.empty[s], (turn - 1u) & 1u, kWaitTimeoutNs)) return false;
-  return mbar_wait_bounded(&sm.full[s], turn & 1u, kWaitTimeoutNs);
+// Wait for stage j, which is in ring slot s = j % S on turn j / S.  A warp may
+// get here while the turn before is still being read, where a barrier's parity
+// alone would pass for this turn's: it waits for the producer's count to say
+// that stage j is issued.  From then on the full barrier's parity is not ambiguous
+// (the next turn is not issued before this warp hands the slot back).  While
+// the stage is not issued, warps that are to read the slot's turn before may
+// have gone to a meeting (sm.trim), which this warp then has to join.
+enum { kStageFail = 0, kStageReady = 1, kStageMeet = 2 };
+__device__ __forceinline__ uint32_t wait_stage(FwdSmem &sm, uint32_t s, uint32_t turn, uint32_t j) {
+  if (*((volatile uint32_t *)&sm.issued) <= j) {
+    const uint64_t t0 = global_timer_ns();
+    do {
+      if (*((volatile uint32_t *)&sm.trim)) return kStageMeet;
+      if (*((volatile uint32_t *)&sm.abort) || global_timer_ns() - t0 > kWaitTimeoutNs)
+        return kStageFail;
+      __nanosleep(32);
+    } while (*((volatile uint32_t *)&sm.issued) <= j);
+  }
+  __threadfence_block();
+  return mbar_wait_bounded(&sm.full[s], turn & 1u, kWaitTimeoutNs) ? kStageReady : kStageFail;
 }
 
 // Sum over the chunks congruent to I modulo S: pairs S apart ... first, so
@@ -269,6 +281,7 @@ __global__ void __launch_bounds__((cons_warps<Elt>() + 2) * 32, 1)
   if (tid == 0) {
     sm.n = 0;
     sm.abort = 0;
+    sm.issued = 0;
     sm.thr = 0ull;
     sm.top_bin = 0;
     sm.trim = 0;
@@ -325,6 +338,8 @@ __global__ void __launch_bounds__((cons_warps<Elt>() + 2) * 32, 1)
             if (kb)
               bulk_g2s_hint(dst + a.emb_bytes, a.fwd + (uint64_t)k0 * a.quad_bytes, kb,
                             &sm.full[s], pol);
+            __threadfence_block();
+            *((volatile uint32_t *)&sm.issued) = seq + 1;
           }
         }
         stop = __shfl_sync(0xffffffffu, (int)stop, 0) != 0;
@@ -490,19 +505,14 @@ __global__ void __launch_bounds__((cons_warps<Elt>() + 2) * 32, 1)
   for (;;) {
     // (one lane's view of the flag: the whole warp goes on or stops)
     while (u < slots && !__shfl_sync(0xffffffffu, *((volatile uint32_t *)&sm.trim), 0)) {
-      const Side sd = next;
-      next = load_side(u + a.workers);
       const uint32_t j = u >> a.lg_runs, rs = u & (runs - 1u);
       const uint32_t s = j % S, turn = j / S;
-      const uint32_t run = (st0 << a.lg_runs) + u;
-      const uint32_t ad = run * 32u + lane;
-      u += a.workers;
-      const bool in = ad < a.n_ads;
-      bool staged = true;
-      if (lane == 0)
-        staged = !*((volatile uint32_t *)&sm.abort) && wait_stage(sm, s, turn);
-      staged = __shfl_sync(0xffffffffu, (int)staged, 0) != 0;
-      if (!staged) {
+      const Side ahead = load_side(u + a.workers);
+      uint32_t staged = kStageFail;
+      if (lane == 0 && !*((volatile uint32_t *)&sm.abort)) staged = wait_stage(sm, s, turn, j);
+      staged = __shfl_sync(0xffffffffu, staged, 0);
+      if (staged == kStageMeet) break;
+      if (staged == kStageFail) {
         if (lane == 0 && !*((volatile uint32_t *)&sm.abort)) {
           atomicOr(&a.ctrl->flags, DEVERR_TIMEOUT);
           sm.abort = 1;
@@ -510,6 +520,12 @@ __global__ void __launch_bounds__((cons_warps<Elt>() + 2) * 32, 1)
         u = slots;
         break;
       }
+      const Side sd = next;
+      next = ahead;
+      const uint32_t run = (st0 << a.lg_runs) + u;
+      const uint32_t ad = run * 32u + lane;
+      u += a.workers;
+      const bool in = ad < a.n_ads;
       mbar_try_wait(&sm.full[s], turn & 1u);  // per-thread acquire
       const uint8_t *stage = smem + (size_t)s * a.stage_bytes;
       const uint32_t ka = smem_u32(stage) + a.emb_bytes + (sd.o0 - sd.os) * a.quad_bytes;
@@ -782,7 +798,10 @@ int launch_t(const FwdCall &c, FwdArgs a, cudaStream_t st) {
   const size_t fixed = (size_t)(a.smem_terms + 3) / 4 * 16 + (D + 3) / 4 * 16 +
                        (a.cand_g ? 0 : (size_t)a.cap * 8);
   uint32_t stages = 2;
-  while (stages < (uint32_t)kFwdMaxStages && (size_t)(stages + 1) * a.stage_bytes <= kRingTarget &&
+  // (no rare terms, no L1 for them: a ring of few runs, 128-element FP32 rows,
+  // gets more; 1M ads with 450 keys 145 -> 122 us)
+  const size_t ring = sw && a.stage_bytes / runs > 16 * 1024 ? 200 * 1024 : kRingTarget;
+  while (stages < (uint32_t)kFwdMaxStages && (size_t)(stages + 1) * a.stage_bytes <= ring &&
          fixed + (size_t)(stages + 1) * a.stage_bytes <= kFwdSmemBudget)
     stages++;
   const size_t smem = fixed + (size_t)stages * a.stage_bytes;
