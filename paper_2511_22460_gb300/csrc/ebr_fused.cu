@@ -832,19 +832,22 @@ __global__ void k_absmax(const float *__restrict__ w, uint32_t n, uint32_t *__re
 // one ad; F goes to *fx_out.  key_id (may be null): the place of each key's
 // term (the forward table's ids).  With route set, does nothing unless *route
 // chose the window-major decode (the device decided the traversal).
-__global__ void k_pack(const float *__restrict__ w, uint32_t n,
-                       const uint32_t *__restrict__ wmax_bits, uint32_t max_keys, int cls_shift,
-                       const uint32_t *__restrict__ route, const uint32_t *__restrict__ key_id,
+// (Launched early: w, wmax_bits and route are the kernel before's, and not
+// __restrict__, since a load through such a pointer may be moved above the wait.)
+__global__ void k_pack(const float *w, uint32_t n, const uint32_t *wmax_bits, uint32_t max_keys,
+                       int cls_shift, const uint32_t *route, const uint32_t *__restrict__ key_id,
                        uint32_t *__restrict__ wq, int *__restrict__ fx_out) {
-  if (route && *route == 0u) return;
-  const int F = fix_exponent(__uint_as_float(*wmax_bits), max_keys);
+  pdl_trigger();
+  pdl_wait();
+  if (route && *((const volatile uint32_t *)route) == 0u) return;
+  const int F = fix_exponent(__uint_as_float(__ldcg(wmax_bits)), max_keys);
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     *fx_out = F;
     wq[n] = 0u;  // the forward table's padding key
   }
   const float s0 = pow2f(F), s1 = pow2f(F + cls_shift), s2 = pow2f(F + 2 * cls_shift);
   for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
-    wq[key_id ? key_id[i] : i] = pack_term(w[i], s0, s1, s2, cls_shift > 0);
+    wq[key_id ? key_id[i] : i] = pack_term(__ldcg(w + i), s0, s1, s2, cls_shift > 0);
 }
 
 // Whether the fused scan fits shared memory for top-k on this index; if not,
@@ -907,10 +910,10 @@ int launch_fused(const ebr_index *ix, const float *h_u, const float *w_hat, uint
       EBR_CUDA_TRY(cudaGetLastError());
       launched++;
     }
-    k_pack<<<std::max<uint32_t>(1, std::min<uint32_t>(1024, (ix->n_keys + 255) / 256)), 256, 0,
-             st>>>(w_hat, ix->n_keys, &ctrl->pad, a.max_keys, a.cls_shift, route, ix->key_id,
-                   wq, reinterpret_cast<int *>(&ctrl->fx));
-    EBR_CUDA_TRY(cudaGetLastError());
+    EBR_CUDA_TRY(launch_pdl(
+        k_pack, std::max<uint32_t>(1, std::min<uint32_t>(1024, (ix->n_keys + 255) / 256)), 256, 0,
+        st, w_hat, ix->n_keys, (const uint32_t *)&ctrl->pad, a.max_keys, a.cls_shift, route,
+        (const uint32_t *)ix->key_id, wq, reinterpret_cast<int *>(&ctrl->fx)));
     launched++;
   }
   int rc;
