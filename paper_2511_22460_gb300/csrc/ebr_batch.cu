@@ -964,19 +964,23 @@ __global__ void __launch_bounds__(kBatchThreads, 1) k_batch_window(const __grid_
     // 0: abort.
     auto may_start = [&](uint32_t w) -> uint32_t {
       const uint32_t tb = w % a.tb, lbuf = w % a.lb;
+      auto ready = [&]() {
+        return (w < a.tb || mbar_try_wait(&sm.t_empty[tb], ((w / a.tb) - 1) & 1u)) &&
+               (FWD || w < a.lb || mbar_try_wait(&sm.l_empty[lbuf], ((w / a.lb) - 1) & 1u));
+      };
+      if (*((volatile uint32_t *)&sm.abort)) return 0;
+      if (ready()) return 1;
       const uint64_t t0 = global_timer_ns();
-      for (;;) {
+      while (!*((volatile uint32_t *)&sm.trim)) {
+        if (ready()) return 1;
         if (*((volatile uint32_t *)&sm.abort)) return 0;
-        if ((w < a.tb || mbar_try_wait(&sm.t_empty[tb], ((w / a.tb) - 1) & 1u)) &&
-            (FWD || w < a.lb || mbar_try_wait(&sm.l_empty[lbuf], ((w / a.lb) - 1) & 1u)))
-          return 1;
-        if (*((volatile uint32_t *)&sm.trim)) return 2;
         if (global_timer_ns() - t0 > kWaitTimeoutNs) {
           atomicOr(&a.ctrl->flags, DEVERR_TIMEOUT);
           sm.abort = 1;
           return 0;
         }
       }
+      return 2;
     };
     read_offsets(0);
     fetch_quads(0);

@@ -88,6 +88,7 @@ struct FwdArgs {
   uint64_t *cand_g;          // if set: the CTAs' candidate buffers, else they are in shared memory
   Ctrl *ctrl;
   float *all_out;            // if set: every score is written here and nothing selected
+  uint32_t direct;           // every ad's key to cand_out[ad] (0: filtered out)
   float *wide_out;           // if set: the per-ad wide term is written here
   uint32_t *hist;            // [kCandBins + 1] candidate-score histogram + top bin
   const int *fx_word;        // F of the packed terms
@@ -355,7 +356,7 @@ __global__ void __launch_bounds__((cons_warps<Elt>() + 2) * 32, 1)
 
   if (warp == kThrWarp) {
     // ----------------------------------------------------------- threshold
-    if (a.all_out) return;
+    if (a.all_out || a.direct) return;
     pdl_wait();  // the histogram and the control block are zeroed before this kernel
     while (!*((volatile uint32_t *)&sm.finished) && !*((volatile uint32_t *)&sm.abort)) {
       // counts below the known bound cannot raise it
@@ -507,7 +508,10 @@ __global__ void __launch_bounds__((cons_warps<Elt>() + 2) * 32, 1)
     while (u < slots && !__shfl_sync(0xffffffffu, *((volatile uint32_t *)&sm.trim), 0)) {
       const uint32_t j = u >> a.lg_runs, rs = u & (runs - 1u);
       const uint32_t s = j % S, turn = j / S;
-      const Side ahead = load_side(u + a.workers);
+      // (FP32: before the wait, 118 -> 114 us for 1M ads of 128 elements; the others
+      // have no registers to hold it meanwhile, 10M FP8 ads 301 -> 330 us)
+      Side ahead;
+      if (!kMma) ahead = load_side(u + a.workers);
       uint32_t staged = kStageFail;
       if (lane == 0 && !*((volatile uint32_t *)&sm.abort)) staged = wait_stage(sm, s, turn, j);
       staged = __shfl_sync(0xffffffffu, staged, 0);
@@ -521,7 +525,7 @@ __global__ void __launch_bounds__((cons_warps<Elt>() + 2) * 32, 1)
         break;
       }
       const Side sd = next;
-      next = ahead;
+      next = kMma ? load_side(u + a.workers) : ahead;
       const uint32_t run = (st0 << a.lg_runs) + u;
       const uint32_t ad = run * 32u + lane;
       u += a.workers;
@@ -648,6 +652,10 @@ __global__ void __launch_bounds__((cons_warps<Elt>() + 2) * 32, 1)
         continue;
       }
       bool keep = in && ((sd.fword >> lane) & 1u);
+      if (a.direct) {
+        if (in) a.cand_out[ad] = keep ? make_key(score, ad) : 0ull;
+        continue;
+      }
       uint64_t kk = 0;
       if (keep) {
         kk = make_key(score, ad);
@@ -665,7 +673,7 @@ __global__ void __launch_bounds__((cons_warps<Elt>() + 2) * 32, 1)
         __syncwarp();
       }
     }
-    if (a.all_out) return;
+    if (a.all_out || a.direct) return;
     // The warps meet: to trim the buffer, or because every warp is done (a
     // warp without runs waits here and takes part in the trims of the others).
     gsync();
@@ -785,7 +793,7 @@ int launch_t(const FwdCall &c, FwdArgs a, cudaStream_t st) {
   a.n_stages = (a.n_ads + a.stage_ads - 1) / a.stage_ads;
   const int grid = (int)std::min<uint32_t>((uint32_t)c.sms, a.n_stages);
   a.trim_at = a.k + kTrimSlack;
-  a.cap = a.all_out ? 0 : (a.trim_at + 64 * cons_warps<Elt>() + 255) / 256 * 256;
+  a.cap = a.all_out || a.direct ? 0 : (a.trim_at + 64 * cons_warps<Elt>() + 255) / 256 * 256;
   a.cand_g = nullptr;
   if (a.cap > kSmemCandMax && (size_t)grid * a.cap <= c.cta_cand_entries) a.cand_g = c.cta_cand;
   // Terms in shared memory: the copy is worth its read where the CTA gathers
@@ -852,6 +860,7 @@ int launch_forward(const FwdCall &c, cudaStream_t st) {
   a.cand_out = c.cand_out;
   a.ctrl = c.ctrl;
   a.all_out = c.all_out;
+  a.direct = c.direct;
   a.wide_out = c.wide_out;
   a.hist = c.hist;
   a.fx_word = reinterpret_cast<const int *>(&c.ctrl->fx);

@@ -873,7 +873,7 @@ int launch_fused(const ebr_index *ix, const float *h_u, const float *w_hat, uint
                  bool packed, const uint64_t *filter, uint32_t k, uint64_t *cand_out,
                  Ctrl *ctrl, float *all_out, float *wide_out, uint32_t *hist, int max_grid,
                  cudaStream_t st, bool wmax_ready, const float *wide_in, const uint32_t *route,
-                 int *n_launched, uint64_t *cta_cand, size_t cta_cand_entries) {
+                 int *n_launched, uint64_t *cta_cand, size_t cta_cand_entries, bool direct) {
   FusedArgs a;
   memset(&a, 0, sizeof(a));
   int launched = 0;
@@ -952,6 +952,7 @@ int launch_fused(const ebr_index *ix, const float *h_u, const float *w_hat, uint
     c.wide_in = wide_in;
     c.route = route;
     c.cls_shift = a.cls_shift;
+    c.direct = direct;
     c.sms = max_grid > 0 ? std::min(ix->num_sms, max_grid) : ix->num_sms;
     rc = launch_forward(c, st);
   } else if (all_out) {

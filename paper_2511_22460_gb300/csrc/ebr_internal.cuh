@@ -236,12 +236,19 @@ int launch_fused(const ebr_index *ix, const float *h_u, const float *w_hat, uint
                  Ctrl *ctrl, float *all_out, float *wide_out, uint32_t *hist, int max_grid,
                  cudaStream_t st, bool wmax_ready = false, const float *wide_in = nullptr,
                  const uint32_t *route = nullptr, int *n_launched = nullptr,
-                 uint64_t *cta_cand = nullptr, size_t cta_cand_entries = 0);
+                 uint64_t *cta_cand = nullptr, size_t cta_cand_entries = 0, bool direct = false);
 bool fused_fits(const ebr_index *ix, uint32_t k);
+// Inventories of up to kDirectAds ads: the forward scan writes every ad's key
+// and the last selection reads them all, so the scan ends without candidate
+// buffers, counts and bounds.  Request times, us, with and without: 10k FP32
+// ads, K = 100, 27.1 and 27.6; 10k FP8, K = 500, 39 and 49; 16k FP32 28.1 and 27.4, K =
+// 1000 32.0 and 27.6 (one CTA reads all the keys), so the line is in between.
+constexpr uint32_t kDirectAds = 12 * 1024;
 // One launch of the scan over the forward key table (ebr_forward.cu): the
 // counterpart of the block-wise fused scan, with the same results.
 struct FwdCall {
   ebr_dtype dtype;
+  bool direct;               // every ad's key to cand_out[ad] (0: filtered out), no selection
   bool tree;                 // FP32: add the inner product's 4-element chunks as a tree
   uint32_t d, n_ads, n_keys, k;
   const void *emb;

@@ -1031,7 +1031,9 @@ int ws_prepare_one(ebr_index *ix, uint32_t n_q, uint32_t kcap) {
   EBR_TRY(dev_reserve(w.scan, entries * sizeof(LenPair)));
   EBR_TRY(dev_reserve(w.work, entries * sizeof(WorkEntry)));
   EBR_TRY(dev_reserve(w.scan_tmp, prims::scan_scratch(entries) * sizeof(LenPair) + 256));
-  EBR_TRY(dev_reserve(w.cand, ((size_t)ix->num_sms * kMaxCtasPerSm + 1) * kcap * 8 +
+  const size_t direct = std::min(ix->n_ads, kDirectAds);
+  EBR_TRY(dev_reserve(w.cand, std::max<size_t>(direct + 2 * (size_t)kcap,
+                                               ((size_t)ix->num_sms * kMaxCtasPerSm + 1) * kcap) * 8 +
                                   2 * (size_t)kcap * 8));
   EBR_TRY(dev_reserve(w.ctrl, kCtrlBytes + kHistWords * 4));
   if (!w.route_stats.p) {  // lifetime counters, zeroed once
@@ -1334,6 +1336,12 @@ int query_one(const ebr_index *cix, const ebr_cross *cross, const ebr_query &q, 
   const size_t cand_used = (size_t)ix->num_sms * kscan +
                            2 * (size_t)pow2_at_least(std::max<uint32_t>(kscan, 1));
   const size_t cta_entries = w.cand.bytes / 8 > cand_used ? w.cand.bytes / 8 - cand_used : 0;
+  // a small inventory's keys are all selected from (n_sel, instead of ctrl's count)
+  const bool direct = ix->fwd && ix->n_ads <= kDirectAds && fused_fits(ix, kscan) &&
+                      ix->n_ads + 2 * (size_t)pow2_at_least(std::max<uint32_t>(kscan, 1)) <=
+                          w.cand.bytes / 8;
+  const Ctrl *n_from = direct ? nullptr : ctrl;
+  const uint32_t n_sel = direct ? ix->n_ads : 0u;
   // a sparse list with no traversal forced: chosen on the device by its work
   const bool auto_route = q_key != nullptr && n_q > 0 &&
                           !(q.flags & (EBR_QF_KEY_MAJOR | EBR_QF_WINDOW_MAJOR)) &&
@@ -1346,7 +1354,7 @@ int query_one(const ebr_index *cix, const ebr_cross *cross, const ebr_query &q, 
     EBR_TRY(launch_fused(ix, q.h_u, q_w, (uint32_t *)w.wq.p, packed, q.filter, kscan,
                          (uint64_t *)w.cand.p, ctrl, nullptr, quant ? (float *)w.wide.p : nullptr,
                          ws_hist(w), ix->num_sms * kMaxCtasPerSm, st, wmax_ready,
-                         nullptr, nullptr, &nl, cta_cand, cta_entries));
+                         nullptr, nullptr, &nl, cta_cand, cta_entries, direct));
     ix->launches += nl;  // (k_absmax, k_pack) k_fused_window
   } else {
     float *w_dense = auto_route ? (float *)w.w_dense.p : nullptr;
@@ -1369,7 +1377,8 @@ int query_one(const ebr_index *cix, const ebr_cross *cross, const ebr_query &q, 
                            auto_route && quant ? (float *)w.wide.p : nullptr,
                            ws_hist(w), ix->num_sms * kMaxCtasPerSm, st,
                            !auto_route || planned, (const float *)w.wide.p,
-                           auto_route ? &ctrl->route : nullptr, &nl, cta_cand, cta_entries));
+                           auto_route ? &ctrl->route : nullptr, &nl, cta_cand, cta_entries,
+                           direct));
       ix->launches += nl;  // (k_absmax, k_pack) k_fused_window
 
     } else {
@@ -1392,7 +1401,7 @@ int query_one(const ebr_index *cix, const ebr_cross *cross, const ebr_query &q, 
   const uint32_t p2 = pow2_at_least(std::max<uint32_t>(kscan, 1));
   if (!quant) {
     EBR_CUDA_TRY(launch_pdl(k_final_select, 1, kFinalThreads, final_smem(k), st,
-                            (const uint64_t *)w.cand.p, (const Ctrl *)ctrl, 0u, k, kmax, ids,
+                            (const uint64_t *)w.cand.p, n_from, n_sel, k, kmax, ids,
                             scores, (uint64_t *)nullptr));
     ix->launches += 1;
   } else {
@@ -1401,7 +1410,7 @@ int query_one(const ebr_index *cix, const ebr_cross *cross, const ebr_query &q, 
     uint64_t *sel = (uint64_t *)w.cand.p + (w.cand.bytes / 8 - 2 * (size_t)p2);
     uint64_t *res = sel + p2;
     EBR_CUDA_TRY(launch_pdl(k_final_select, 1, kFinalThreads, final_smem(kscan), st, ck,
-                            (const Ctrl *)ctrl, 0u, kscan, kscan, (uint32_t *)nullptr,
+                            n_from, n_sel, kscan, kscan, (uint32_t *)nullptr,
                             (float *)nullptr, sel));
     k_rescore<<<launch_grid((uint64_t)kscan * 32, 256, 4096), 256, 0, st>>>(
         sel, kscan, (const float *)ix->emb_f32.p, ix->d, q.h_u, (const float *)w.wide.p, res);
@@ -1985,6 +1994,7 @@ constexpr uint32_t kNoAllocMaxGrid = 160;   // CTAs of the scan (>= SM count of 
 constexpr uint32_t kNoAllocCtrlWords = (kCtrlBytes + kHistWords * 4) / 8;
 constexpr size_t kNoAllocWords = kNoAllocCtrlWords + (size_t)kNoAllocMaxGrid * kNoAllocMaxK;
 // 256 + 16384 + 8 * 160 * 1024 bytes = 1.27 MiB.
+static_assert(kDirectAds <= (size_t)kNoAllocMaxGrid * kNoAllocMaxK, "a key per ad");
 static __device__ __align__(256) unsigned long long g_noalloc_scratch[kNoAllocWords];
 
 constexpr int kNoAllocMaxDevices = 64;
@@ -2104,11 +2114,13 @@ extern "C" int ebr_scan_topk_noalloc(const float *emb, uint32_t n_ads, uint32_t 
     c.hist = reinterpret_cast<uint32_t *>(reinterpret_cast<char *>(base) + kCtrlBytes);
     c.wide_in = wide;
     c.sms = std::min<int>(sms, kNoAllocMaxGrid);
+    c.direct = n_ads <= kDirectAds;
     rc = launch_forward(c, st);
   }
   if (rc == EBR_OK) {
     e = launch_pdl(k_final_select, 1, kFinalThreads, final_smem(k), st, (const uint64_t *)cand,
-                   (const Ctrl *)ctrl, 0u, k, k, out_ids, out_scores, (uint64_t *)nullptr);
+                   n_ads <= kDirectAds ? (const Ctrl *)nullptr : (const Ctrl *)ctrl,
+                   n_ads <= kDirectAds ? n_ads : 0u, k, k, out_ids, out_scores, (uint64_t *)nullptr);
     if (e != cudaSuccess) {
       set_error("ebr_scan_topk_noalloc: %s", cudaGetErrorString(e));
       rc = EBR_ECUDA;

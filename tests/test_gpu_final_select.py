@@ -62,7 +62,8 @@ def _noalloc(s, k, d, mask=None):
 
 @pytest.mark.parametrize("kind", ["normal", "equal", "few", "inf", "outlier", "subnormal", "rising"])
 @pytest.mark.parametrize("n,k,d", [(1, 1, 4), (1, 5, 128), (31, 64, 8), (700, 700, 16),
-                                   (1025, 1024, 32), (70_001, 1000, 4), (200_033, 1024, 64)])
+                                   (1025, 1024, 32), (12_288, 1000, 8), (12_289, 7, 8),
+                                   (70_001, 1000, 4), (200_033, 1024, 64)])
 def test_noalloc_selects_what_a_sort_does(kind, n, k, d):
     rng = np.random.default_rng(n + k)
     s = _scores(kind, n, rng)
@@ -73,7 +74,7 @@ def test_noalloc_selects_what_a_sort_does(kind, n, k, d):
 
 
 @pytest.mark.parametrize("kind", ["normal", "equal", "few", "outlier", "rising"])
-@pytest.mark.parametrize("n,k", [(9_000, 8192), (300, 8192), (150_000, 8191), (150_000, 2049), (800_000, 20)])
+@pytest.mark.parametrize("n,k", [(9_000, 8192), (300, 8192), (12_288, 8192), (12_289, 50), (150_000, 8191), (150_000, 2049), (800_000, 20)])
 def test_request_selects_what_a_sort_does(kind, n, k):
     rng = np.random.default_rng(n + k)
     s = _scores(kind, n, rng)
