@@ -263,18 +263,19 @@ def run_single(args, w, rank, world, local_rank, workload, steps=None, n_req=16,
     peak, peak_kind = _peaks()
     scan_ms = prof.ms_scan / max(prof.calls, 1)
     emb_bytes = info.emb_bytes
-    # the fused scan must read the embedding table and the window-major view of
-    # the compressed lists (keys + value bytes + window offsets)
-    kern_bytes = emb_bytes + info.window_view_bytes
+    # the scan must read the embedding table and the forward key table: every
+    # posting's key id (16 or 24 bits) and the offsets of its runs of 32 ads
+    key_id_bytes = 2 if w.n_keys < 65536 else 3
+    kern_bytes = emb_bytes + key_id_bytes * info.nnz_unique + 4 * (w.n_ads // 32 + 1)
     if w.recipe.emb_dtype != "f32":
         kern_bytes += 4 * w.n_ads  # the FP32 wide term, written for the rescoring
-    kernel = "k_fused_window"
-    bytes_note = ("embedding table (+ FP8 row scales) + window-major view of the compressed "
-                  "lists (+ FP32 wide term out when the table is quantised), per launch")
+    kernel = "k_forward"
+    bytes_note = ("embedding table (+ FP8 row scales) + forward key table (a key id per posting, "
+                  "run offsets) (+ FP32 wide term out when the table is quantised), per launch")
     routes = None
     if sparse:
-        # per launch, the fused scan either reads the wide term Algorithm 2
-        # scattered (no window decoded) or decodes the window-major view
+        # per launch, the scan either reads the wide term Algorithm 2 scattered
+        # or the forward key table
         if args.sparse_route == "auto":
             n_win_r = int(prof.window_routed)
             n_key_r = int(prof.auto_routed - prof.window_routed)
@@ -286,7 +287,7 @@ def run_single(args, w, rank, world, local_rank, workload, steps=None, n_req=16,
         kern_bytes = ((n_win_r * kern_bytes + n_key_r * key_bytes) /
                       max(n_win_r + n_key_r, 1))
         bytes_note = ("embedding table (+ FP8 row scales) + per launch either the FP32 wide "
-                      "term read (Algorithm 2 scattered it) or the window-major view (+ FP32 "
+                      "term read (Algorithm 2 scattered it) or the forward key table (+ FP32 "
                       "wide term out when the table is quantised), averaged over the routes "
                       "the requests took")
     achieved = kern_bytes / (scan_ms / 1e3) / 1e9
@@ -338,7 +339,7 @@ def run_single(args, w, rank, world, local_rank, workload, steps=None, n_req=16,
     return out
 
 
-KERNEL_REV = "fused-v6"
+KERNEL_REV = "forward-v2"
 
 # FP32 add throughput of the CUDA cores: 152 SMs x 128 FP32 lanes x 2.07 GHz
 ALU_ADD_PEAK_T = 152 * 128 * 2.07e9 / 1e12

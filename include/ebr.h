@@ -83,10 +83,13 @@ typedef struct {
 /*
  * Besides the paper's key-major arrays, the index keeps a window-major view
  * of the same blocks (per group, ordered by (window h = ad >> 8, key k), each
- * with its key and its 2^g value bytes, plus per-window offsets).  Requests
- * whose query covers the whole key space (dense w^ or raw user features) walk
- * that view window by window inside the scan; sparse key lists walk the
- * key-major arrays with Algorithm 2.
+ * with its key and its 2^g value bytes, plus per-window offsets), and, decoded
+ * from it, a forward key table: per run of 32 ads their keys, four at a time,
+ * 16 or 24 bits each.  Requests whose query covers the whole key space (dense w^
+ * or raw user features) read the forward table beside the embeddings (an index
+ * whose key counts differ too much within runs, or with 2^24 keys, has none and
+ * they walk the window-major view instead); sparse key lists walk the key-major
+ * arrays with Algorithm 2.
  *
  * Build the compressed inverted list of Algorithm 1 (Block Grouping by
  * ad >> 8, Logarithmic Categorization into groups g = ceil(log2 n) = 0..8,
