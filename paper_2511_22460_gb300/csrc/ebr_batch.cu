@@ -596,6 +596,7 @@ enum { kWalk = 0, kForward = 1, kForwardSw = 2 };
 // 128, so that two windows' accumulators (2 x 128 columns each) fit TMEM and
 // the MMAs of one run while the other's are read.
 constexpr uint32_t kFwdWin = 128;
+constexpr uint32_t accum_bufs(bool fwd) { return fwd ? 2 : 1; }
 
 // cp.async: 16 bytes global -> shared, asynchronously, and the wait for all of
 // the calling thread's.
@@ -611,6 +612,7 @@ __global__ void __launch_bounds__(kBatchThreads, 1) k_batch_window(const __grid_
   constexpr bool FWD = MODE != kWalk, SW = MODE == kForwardSw;
   constexpr uint32_t kWin = FWD ? kFwdWin : kBWin;      // ads of a window
   constexpr uint32_t kWarpAds = kWin / kEpiWarps;       // of them per epilogue warp
+  constexpr uint32_t kTb = accum_bufs(FWD);             // accumulator buffers
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   __shared__ BatchSmem sm;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -963,10 +965,9 @@ __global__ void __launch_bounds__(kBatchThreads, 1) k_batch_window(const __grid_
     // epilogue warps.  (They may be in a meeting, which this warp has to join: 2.)
     // 0: abort.
     auto may_start = [&](uint32_t w) -> uint32_t {
-      const uint32_t tb = w % a.tb, lbuf = w % a.lb;
       auto ready = [&]() {
-        return (w < a.tb || mbar_try_wait(&sm.t_empty[tb], ((w / a.tb) - 1) & 1u)) &&
-               (FWD || w < a.lb || mbar_try_wait(&sm.l_empty[lbuf], ((w / a.lb) - 1) & 1u));
+        return (w < kTb || mbar_try_wait(&sm.t_empty[w % kTb], ((w / kTb) - 1) & 1u)) &&
+               (FWD || w < a.lb || mbar_try_wait(&sm.l_empty[w % a.lb], ((w / a.lb) - 1) & 1u));
       };
       if (*((volatile uint32_t *)&sm.abort)) return 0;
       if (ready()) return 1;
@@ -994,7 +995,7 @@ __global__ void __launch_bounds__(kBatchThreads, 1) k_batch_window(const __grid_
     }
     for (;;) {
     while (j < my_wins && !__shfl_sync(0xffffffffu, *((volatile uint32_t *)&sm.trim), 0)) {
-      const uint32_t tb = j % a.tb, lbuf = j % a.lb;
+      const uint32_t tb = j % kTb, lbuf = FWD ? 0u : j % a.lb;
       uint32_t rows, tab_a;  // rows of the list, and its first entry of this warp's ads
       constexpr uint32_t kRowEntries = FWD ? kWarpAds : 32;
       const uint32_t go = __shfl_sync(0xffffffffu, lane == 0 ? may_start(j) : 0u, 0);
@@ -1097,7 +1098,7 @@ __global__ void __launch_bounds__(kBatchThreads, 1) k_batch_window(const __grid_
         if (kFly > 3 && r + 2 < rows) add_row(v2);
         if (!t_ok) {
           // the deep scores are waited for only now: the MMAs ran behind the gathers
-          t_ok = mbar_wait_bounded(&sm.t_full[tb], (j / a.tb) & 1u, kWaitTimeoutNs);
+          t_ok = mbar_wait_bounded(&sm.t_full[tb], (j / kTb) & 1u, kWaitTimeoutNs);
           t_ok = __all_sync(0xffffffffu, t_ok);
           if (!t_ok) {
             if (lane == 0) {
@@ -1519,7 +1520,7 @@ static bool plan_smem(const ebr_index *ix, uint32_t B, BatchPlan *p) {
   p->list_cap = kBWin * ix->max_keys_per_ad;  // 8 runs x 32 ads x rows
   const uint32_t n_mt = 2;  // even and odd users
   const uint32_t win = ix->fwd ? kFwdWin : kBWin;
-  p->tb = ix->fwd ? 2 : 1;
+  p->tb = accum_bufs(ix->fwd != nullptr);
   p->sa = ix->fwd ? 2 : 1;
   const uint32_t row_bytes = ix->d * (ix->dtype == EBR_FP8E4M3 ? 1u : 2u);
   p->tile_row = row_bytes >= 128 ? 128u : 64u;
