@@ -173,6 +173,7 @@ struct FwdSmem {
   uint32_t hist[256], misc[8], wtot[2][kMaxConsWarps];
   unsigned long long thr;
   uint32_t n, n_seen, abort, stop, top_bin;
+  uint32_t above;   // candidates of the CTA at or above the last bound
   uint32_t issued;  // stages whose copies the producer has issued
   uint32_t trim, meet, finished;  // trim asked for; what a meeting of the warps is for; all done
 };
@@ -724,7 +725,7 @@ __global__ void __launch_bounds__((cons_warps<Elt>() + 2) * 32, 1)
     if (sm.chist[i]) atomicAdd(a.hist + i, atomicExch(&sm.chist[i], 0u));
   if (tid == 0) {
     atomicMax(a.hist + kCandBins, sm.top_bin);
-    sm.n_seen = 0;
+    sm.above = 0;  // (not n_seen: no barrier lies between the other warps' read of it and here)
   }
   gsync();
   if (warp == 0) {
@@ -737,10 +738,10 @@ __global__ void __launch_bounds__((cons_warps<Elt>() + 2) * 32, 1)
     uint32_t above = 0;
     for (uint32_t i = tid; i < n; i += kConsThreads) above += cand[i] >= thr ? 1u : 0u;
     above = __reduce_add_sync(0xffffffffu, above);
-    if (lane == 0 && above) atomicAdd(&sm.n_seen, above);
+    if (lane == 0 && above) atomicAdd(&sm.above, above);
   }
   gsync();
-  if (sm.n_seen > a.k) {
+  if (sm.above > a.k) {
     const uint64_t cut =
         group_radix_select<kConsThreads>(cand, n, a.k, sm.hist, sm.misc, tid, gsync);
     if (tid == 0) {
