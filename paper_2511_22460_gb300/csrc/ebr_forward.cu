@@ -450,10 +450,13 @@ __global__ void __launch_bounds__((cons_warps<Elt>() + 2) * 32, 1)
   const uint32_t hot = a.smem_terms;
   auto term = [&](uint32_t id) -> uint32_t {
     if (ALL) return lds_1(s_terms_a + 4u * id);
-    uint32_t v;  // no branch: lanes read their term from one place or the other
+    // No branch: lanes read their term from one place or the other.  (Not .nc:
+    // the kernel before writes wq while this one already runs, and that path is
+    // for memory that nothing writes as long as the kernel lives.)
+    uint32_t v;
     asm volatile(
         "{\n .reg .pred p;\n setp.lt.u32 p, %1, %2;\n @p ld.shared.u32 %0, [%3];\n"
-        " @!p ld.global.nc.u32 %0, [%4];\n}"
+        " @!p ld.global.u32 %0, [%4];\n}"
         : "=r"(v)
         : "r"(id), "r"(hot), "r"(s_terms_a + 4u * id), "l"(a.wq + id));
     return v;
@@ -495,7 +498,7 @@ __global__ void __launch_bounds__((cons_warps<Elt>() + 2) * 32, 1)
         d.o1 = __ldg(a.fwd_off + run + 1);
       }
       if (ad < a.n_ads) {
-        if (pre) d.wide = __ldg(a.wide_in + ad);
+        if (pre) d.wide = __ldcg(a.wide_in + ad);  // (the kernel before's; see term)
         if (a.scale) d.scale = __ldg(a.scale + ad);
         if (a.filter) d.fword = __ldg(a.filter + run);
       }
