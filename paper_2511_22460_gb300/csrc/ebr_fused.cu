@@ -453,7 +453,7 @@ __global__ void __maxnreg__(96) k_fused_window(FusedArgs a) {
         }
         uint32_t p[kChunksInFlight];
 #pragma unroll
-        for (int q = 0; q < kChunksInFlight; q++) p[q] = valid[q] ? __ldg(a.wq + key[q]) : 0u;
+        for (int q = 0; q < kChunksInFlight; q++) p[q] = valid[q] ? __ldca(a.wq + key[q]) : 0u;
         uint32_t fl = 0;  // chunks whose term is FP32 (class 3)
 #pragma unroll
         for (int q = 0; q < kChunksInFlight; q++) {
@@ -562,7 +562,7 @@ __global__ void __maxnreg__(96) k_fused_window(FusedArgs a) {
     for (int ps = 0; ps < Sh::kPasses; ps++) {
       const uint32_t ad = w * kWin + ps * Sh::kRowsPerPass + prow;
       const bool in = ad < a.n_ads && qd == 0;
-      pre_side[ps] = in && pre ? __ldg(a.wide_in + ad) : 0.f;
+      pre_side[ps] = in && pre ? __ldcg(a.wide_in + ad) : 0.f;
       pre_scale[ps] = in && a.scale ? __ldg(a.scale + ad) : 1.f;
       pre_keep[ps] = !(in && a.filter) || ((__ldg(a.filter + (ad >> 6)) >> (ad & 63)) & 1ull);
     }

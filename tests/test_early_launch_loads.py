@@ -28,3 +28,9 @@ def test_early_kernels_take_no_restrict_pointer_to_the_results_before():
         for a in args:
             assert re.search(r"\*\s*%s\b" % a, head), (kern, a)
             assert not re.search(r"__restrict__\s+%s\b" % a, head), (kern, a)
+
+
+def test_block_wise_scan_reads_terms_and_wide_scores_with_ordinary_loads():
+    src = _code("ebr_fused.cu")
+    assert "ld.global.nc" not in src
+    assert not re.search(r"__ldg\(\s*&?a\.(wq|wide_in|route|fx_word|hist|ctrl)\b", src)
