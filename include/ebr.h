@@ -311,6 +311,18 @@ int ebr_debug_gemm_e4m3(const uint8_t *A, uint32_t n, const uint8_t *U, uint32_t
  */
 int ebr_debug_wait_timeout(uint32_t timeout_us, void *stream);
 
+/*
+ * Failure-detection check (no paper counterpart): ebr_build_index with the
+ * failures in `faults` (0: none) made to happen.  EBR_FAULT_SORT_*: every wait
+ * of that radix sort's look-backs (of the pairs, of the keys by popularity, of
+ * the blocks) runs out at once, which has to end in EBR_ETIMEDOUT where that sort has
+ * more than one tile of 4096 entries.
+ */
+#define EBR_FAULT_SORT_PAIRS 1u
+#define EBR_FAULT_SORT_KEYS 2u
+#define EBR_FAULT_SORT_BLOCKS 4u
+int ebr_debug_build_index(const ebr_index_desc *desc, uint32_t faults, ebr_index **out);
+
 /* ------------------------------------------------------- no-allocation form */
 /*
  * Allocation-free scan + top-K.  The paper has no counterpart: this entry

@@ -58,10 +58,13 @@ struct PairLoad {
 };
 
 // win_start[h] = first word of window h (n_win + 1 entries) of the sorted
-// words, and the number of words equal to the one before them.
+// words, and the number of words equal to the one before them.  Nothing when
+// the sort of the words gave up (*flags).
 __global__ void k_window_starts(const uint64_t *__restrict__ x, uint32_t m, int wshift,
                                 uint32_t n_win, uint32_t *__restrict__ win_start,
-                                uint32_t *__restrict__ n_dup) {
+                                uint32_t *__restrict__ n_dup,
+                                const uint32_t *__restrict__ flags) {
+  if (*flags) return;
   uint32_t dup = 0;
   for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < m; i += gridDim.x * blockDim.x) {
     const uint64_t a = __ldg(x + i);
@@ -93,6 +96,7 @@ struct WinArgs {
   const uint64_t *x;            // sorted distinct words
   const uint32_t *win_start;    // [n_win + 1]
   const uint32_t *n_dup;        // repeated words found (then nothing is walked)
+  const uint32_t *flags;        // a sort before gave up (then neither)
   uint32_t n_win, n_ads;
   int kb;
   // counts (first walk)
@@ -136,7 +140,7 @@ __global__ void __launch_bounds__(kWinThreads) k_windows(const __grid_constant__
   __shared__ uint32_t s_ubase[kGroups];
   extern __shared__ __align__(16) uint8_t s_fwd[];  // the window's quads
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  if (*a.n_dup) return;  // blocks are sets; the caller drops the repeated words first
+  if (*a.flags || *a.n_dup) return;  // blocks are sets; the caller drops the repeated words first
   for (uint32_t w = blockIdx.x; w < a.n_win; w += gridDim.x) {
     const uint32_t b0 = a.win_start[w], b1 = a.win_start[w + 1];
     s_adcnt[tid] = 0;
@@ -345,6 +349,7 @@ struct KeyArgs {
   uint8_t *values[kGroups];
   uint32_t gstart[kGroups + 1];
   int kb;
+  const uint32_t *flags;  // the sort of the blocks gave up (then nothing is written)
 };
 
 // p-th block in (g, k, h) order: its header and its 2^g value bytes, from its
@@ -352,6 +357,7 @@ struct KeyArgs {
 template <typename K>
 __global__ void k_key_major(const K *__restrict__ skey, const uint32_t *__restrict__ sval,
                             uint32_t nb, const __grid_constant__ KeyArgs a) {
+  if (*a.flags) return;
   for (uint32_t p = blockIdx.x * blockDim.x + threadIdx.x; p < nb; p += gridDim.x * blockDim.x) {
     const uint32_t g = (uint32_t)(skey[p] >> a.kb), q = sval[p];
     const uint64_t rank = p - a.gstart[g], src = q - a.gstart[g];
@@ -442,7 +448,9 @@ __global__ void k_pop_records(uint32_t *__restrict__ cnt, uint32_t n, uint32_t *
     key[i] = i;
   }
 }
-__global__ void k_pop_ids(const uint32_t *__restrict__ key, uint32_t n, uint32_t *__restrict__ id) {
+__global__ void k_pop_ids(const uint32_t *__restrict__ key, uint32_t n, uint32_t *__restrict__ id,
+                          const uint32_t *__restrict__ flags) {
+  if (*flags) return;  // the sort gave up
   for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
     id[key[i]] = i;
 }
@@ -503,13 +511,14 @@ static bool on_device(const void *p, int device) {
 template <typename K>
 static int build_key_major(ebr_index *ix, uint32_t nb, KeyArgs &ka, void *k0, void *k1, void *k2,
                            uint32_t *v0, uint32_t *v1, uint32_t *v2, void *scratch,
-                           uint32_t *flags, cudaStream_t st) {
+                           uint32_t *flags, uint32_t max_spins, cudaStream_t st) {
   const K *sk = (const K *)k0;
   const uint32_t *sv = v0;
   if (nb) {
     bool in_b = false;
     EBR_TRY((prims::radix_sort<K, true>(prims::ArrayLoad<K>{(const K *)k0}, v0, (K *)k1, (K *)k2,
-                                        v1, v2, nb, ka.kb + 4, scratch, flags, &in_b, st)));
+                                        v1, v2, nb, ka.kb + 4, scratch, flags, &in_b, st,
+                                        max_spins)));
     sk = (const K *)(in_b ? k2 : k1);
     sv = in_b ? v2 : v1;
     k_key_major<K><<<grid_for(nb), 256, 0, st>>>(sk, sv, nb, ka);
@@ -526,7 +535,11 @@ struct BuildCounts {
   uint32_t flags, n_dup, max_keys, gc[kGroups], win_max[3], fwd[5], m_unique;
 };
 
-static int build_impl(const ebr_index_desc *desc, ebr_index *ix, cudaStream_t st) {
+// faults: see ebr_debug_build_index.
+static int build_impl(const ebr_index_desc *desc, ebr_index *ix, uint32_t faults,
+                      cudaStream_t st) {
+  // polls of a look-back in the sorts of the pairs, the keys by popularity, the blocks
+  auto spins = [&](uint32_t fault) { return faults & fault ? 0u : prims::kSortSpins; };
   const uint64_t nnz = desc->nnz;
   const uint32_t n_keys = desc->n_keys, n_ads = desc->n_ads, n_win = (n_ads + 255) / 256;
   const int kb = bits_for(n_keys), hb = bits_for(n_win);
@@ -586,6 +599,7 @@ static int build_impl(const ebr_index_desc *desc, ebr_index *ix, cudaStream_t st
     memset(&w, 0, sizeof(w));
     w.win_start = win_start;
     w.n_dup = &cnt->n_dup;
+    w.flags = &cnt->flags;
     w.n_win = n_win;
     w.n_ads = n_ads;
     w.kb = kb;
@@ -605,7 +619,8 @@ static int build_impl(const ebr_index_desc *desc, ebr_index *ix, cudaStream_t st
       bool in_b = false;
       BTRY((prims::radix_sort<uint64_t, false>(PairLoad{pk, pa, n_keys, n_ads, kb, &cnt->flags},
                                                nullptr, wa, wb, nullptr, nullptr, nnz,
-                                               hb + kb + 8, scratch, &cnt->flags, &in_b, st)));
+                                               hb + kb + 8, scratch, &cnt->flags, &in_b, st,
+                                               spins(EBR_FAULT_SORT_PAIRS))));
       if (in_b) std::swap(wa, wb);  // wa: sorted
     }
     // blocks and keys per window; taken again when repeated words turn up
@@ -613,7 +628,7 @@ static int build_impl(const ebr_index_desc *desc, ebr_index *ix, cudaStream_t st
       w.x = wa;
       if (m) {
         k_window_starts<<<grid_for(m), 256, 0, st>>>(wa, m, kb + 8, n_win, win_start,
-                                                     &cnt->n_dup);
+                                                     &cnt->n_dup, &cnt->flags);
         BCUDA(cudaGetLastError());
       }
       k_windows<false, uint32_t><<<std::min<uint32_t>(n_win, 1u << 20), kWinThreads, 0, st>>>(w);
@@ -656,6 +671,7 @@ static int build_impl(const ebr_index_desc *desc, ebr_index *ix, cudaStream_t st
     KeyArgs ka;
     memset(&ka, 0, sizeof(ka));
     ka.kb = kb;
+    ka.flags = &cnt->flags;
     for (int g = 0; g < kGroups; g++) {
       ix->n_blocks[g] = hc.gc[g];
       hdr_off[g] = hdr_total;
@@ -713,8 +729,10 @@ static int build_impl(const ebr_index_desc *desc, ebr_index *ix, cudaStream_t st
       BCUDA(cudaGetLastError());
       BTRY((prims::radix_sort<uint32_t, true>(prims::ArrayLoad<uint32_t>{pc[0]}, pc[1], pc[2], pc[3],
                                               pc[4], pc[5], n_keys, kPopBits,
-                                              (char *)pop.p + 6 * kn_b, &cnt->flags, &in_b, st)));
-      k_pop_ids<<<grid_for(n_keys), 256, 0, st>>>(in_b ? pc[5] : pc[4], n_keys, ix->key_id);
+                                              (char *)pop.p + 6 * kn_b, &cnt->flags, &in_b, st,
+                                              spins(EBR_FAULT_SORT_KEYS))));
+      k_pop_ids<<<grid_for(n_keys), 256, 0, st>>>(in_b ? pc[5] : pc[4], n_keys, ix->key_id,
+                                                  &cnt->flags);
       BCUDA(cudaGetLastError());
     }
     const size_t fwd_smem = w.fwd ? (size_t)hc.fwd[3] * (w.quad_bytes + 1024) : 0;
@@ -746,10 +764,10 @@ static int build_impl(const ebr_index_desc *desc, ebr_index *ix, cudaStream_t st
     BCUDA(cudaEventRecord(ev[2], st));
     if (k32)
       BTRY(build_key_major<uint32_t>(ix, nb, ka, w.skey, k1, k2, w.sval, v1, v2, bscr, &cnt->flags,
-                                     st));
+                                     spins(EBR_FAULT_SORT_BLOCKS), st));
     else
       BTRY(build_key_major<uint64_t>(ix, nb, ka, w.skey, k1, k2, w.sval, v1, v2, bscr, &cnt->flags,
-                                     st));
+                                     spins(EBR_FAULT_SORT_BLOCKS), st));
     BCUDA(cudaEventRecord(ev[3], st));
     BCUDA(cudaMemcpyAsync(&hc, cnt, sizeof(hc), cudaMemcpyDeviceToHost, st));
     BCUDA(cudaStreamSynchronize(st));
@@ -821,7 +839,7 @@ extern "C" void ebr_index_free(ebr_index *ix) {
   delete ix;
 }
 
-extern "C" int ebr_build_index(const ebr_index_desc *desc, ebr_index **out) {
+static int build_index(const ebr_index_desc *desc, uint32_t faults, ebr_index **out) {
   clear_error();
   if (!desc || !out) {
     set_error("ebr_build_index: null argument");
@@ -850,7 +868,7 @@ extern "C" int ebr_build_index(const ebr_index_desc *desc, ebr_index **out) {
   ix->rescore_mult = desc->rescore_mult ? desc->rescore_mult : 4;
   cudaDeviceGetAttribute(&ix->num_sms, cudaDevAttrMultiProcessorCount, desc->device);
   cudaStream_t st = (cudaStream_t)desc->stream;
-  int rc = build_impl(desc, ix, st);
+  int rc = build_impl(desc, ix, faults, st);
   if (rc == EBR_OK) rc = upload_embeddings(desc, ix, st);
   if (rc != EBR_OK) {
     std::string msg = ebr_last_error();
@@ -862,6 +880,15 @@ extern "C" int ebr_build_index(const ebr_index_desc *desc, ebr_index **out) {
   cudaSetDevice(prev);
   *out = ix;
   return EBR_OK;
+}
+
+extern "C" int ebr_build_index(const ebr_index_desc *desc, ebr_index **out) {
+  return build_index(desc, 0, out);
+}
+
+extern "C" int ebr_debug_build_index(const ebr_index_desc *desc, uint32_t faults,
+                                     ebr_index **out) {
+  return build_index(desc, faults, out);
 }
 
 extern "C" int ebr_index_get_info(const ebr_index *ix, ebr_index_info *out) {

@@ -274,7 +274,8 @@ template <typename K, typename Load, bool VALS>
 __global__ void __launch_bounds__(kSortThreads, 4) k_sort_pass(
     Load load, const uint32_t *__restrict__ vals, uint64_t n, int shift,
     const uint32_t *__restrict__ hist, uint64_t *status, uint32_t epoch, uint32_t *ticket,
-    K *__restrict__ keys_out, uint32_t *__restrict__ vals_out, uint32_t *__restrict__ flags) {
+    K *__restrict__ keys_out, uint32_t *__restrict__ vals_out, uint32_t *__restrict__ flags,
+    uint32_t max_spins) {
   constexpr int kSortKpt = sort_kpt<K, VALS>();
   constexpr uint32_t kSortTile = kSortThreads * kSortKpt;
   __shared__ K s_keys[kSortTile];
@@ -330,6 +331,10 @@ __global__ void __launch_bounds__(kSortThreads, 4) k_sort_pass(
     uint32_t spins = 0;
     bool open = true;
     for (int t = (int)tile - 1; open;) {
+      if (spins >= max_spins) {  // never published: give up, flag it
+        atomicOr(flags, DEVERR_TIMEOUT);
+        break;
+      }
       uint64_t v[kLook];
 #pragma unroll
       for (int q = 0; q < kLook; q++)
@@ -343,10 +348,7 @@ __global__ void __launch_bounds__(kSortThreads, 4) k_sort_pass(
           t--;
           open = e == epoch;
         } else {
-          if (++spins > kSortSpins) {  // never published: give up, flag it
-            atomicOr(flags, DEVERR_TIMEOUT);
-            open = false;
-          }
+          spins++;
           break;
         }
       }
@@ -385,11 +387,14 @@ inline size_t sort_scratch(uint64_t n) {
 // Sorts n keys (with vals, if given) by bits [0, end_bit).  The first pass
 // reads them through `load`; passes write keys_a, keys_b, keys_a, ... (vals:
 // from vals into vals_a, vals_b, ...).  *in_b tells where the result ended.
-// end_bit >= 1.  A bounded wait that ran out sets DEVERR_TIMEOUT in *flags.
+// end_bit >= 1.  A look-back that polled max_spins times in vain sets
+// DEVERR_TIMEOUT in *flags; the output is then not a permutation of the input
+// (words of it may be whatever the memory held), so a kernel that uses it as
+// indices reads *flags first.
 template <typename K, bool VALS, typename Load>
 int radix_sort(Load load, const uint32_t *vals, K *keys_a, K *keys_b, uint32_t *vals_a,
                uint32_t *vals_b, uint64_t n, int end_bit, void *scratch, uint32_t *flags,
-               bool *in_b, cudaStream_t st) {
+               bool *in_b, cudaStream_t st, uint32_t max_spins = kSortSpins) {
   *in_b = false;
   if (n == 0) return EBR_OK;
   const int passes = std::max(1, (end_bit + 7) / 8);
@@ -408,11 +413,11 @@ int radix_sort(Load load, const uint32_t *vals, K *keys_a, K *keys_b, uint32_t *
     uint32_t *vout = (p & 1) ? vals_b : vals_a;
     if (p == 0)
       k_sort_pass<K, Load, VALS><<<(unsigned)tiles, kSortThreads, 0, st>>>(
-          load, vals, n, 0, hist, status, 1u, tickets, out, vout, flags);
+          load, vals, n, 0, hist, status, 1u, tickets, out, vout, flags, max_spins);
     else
       k_sort_pass<K, ArrayLoad<K>, VALS><<<(unsigned)tiles, kSortThreads, 0, st>>>(
           ArrayLoad<K>{(p & 1) ? keys_a : keys_b}, (p & 1) ? vals_a : vals_b, n, 8 * p,
-          hist + 256 * p, status, 2u * p + 1u, tickets + p, out, vout, flags);
+          hist + 256 * p, status, 2u * p + 1u, tickets + p, out, vout, flags, max_spins);
     EBR_CUDA_TRY(cudaGetLastError());
     *in_b = (p & 1) != 0;
   }

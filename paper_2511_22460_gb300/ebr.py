@@ -30,6 +30,7 @@ W_DENSE, W_HASHED = 0, 1
 IO_DEVICE, IO_HOST = 0, 1
 QF_KEY_MAJOR = 1
 QF_WINDOW_MAJOR = 2
+FAULT_SORT_PAIRS, FAULT_SORT_KEYS, FAULT_SORT_BLOCKS = 1, 2, 4
 _DTYPES = {"f32": F32, "bf16": BF16, "fp8e4m3": FP8E4M3}
 
 vp, u32, u64, i32 = C.c_void_p, C.c_uint32, C.c_uint64, C.c_int
@@ -114,6 +115,8 @@ ebr_scan_topk_noalloc = _sig("ebr_scan_topk_noalloc", i32,
 ebr_debug_gemm_bf16 = _sig("ebr_debug_gemm_bf16", i32, [vp, u32, vp, u32, u32, vp, vp])
 ebr_debug_gemm_e4m3 = _sig("ebr_debug_gemm_e4m3", i32, [vp, u32, vp, u32, u32, vp, vp])
 ebr_debug_wait_timeout = _sig("ebr_debug_wait_timeout", i32, [u32, vp])
+ebr_debug_build_index = _sig("ebr_debug_build_index", i32,
+                             [C.POINTER(IndexDesc), u32, C.POINTER(vp)])
 ebr_profile_enable = _sig("ebr_profile_enable", i32, [vp, i32])
 ebr_profile_read = _sig("ebr_profile_read", i32, [vp, C.POINTER(Profile)])
 ebr_server_create = _sig("ebr_server_create", i32, [vp, vp, vp, C.POINTER(vp)])
@@ -211,14 +214,17 @@ class Index:
 
 
 def build_index(n_ads, n_keys, post_key, post_ad, emb, dtype="f32", rescore_mult=0, device=0,
-                stream=None) -> Index:
+                stream=None, debug_faults=0) -> Index:
     emb_dtype = _DTYPES[dtype] if isinstance(dtype, str) else int(dtype)
     d = IndexDesc(n_ads, n_keys, int(post_key.numel() if hasattr(post_key, "numel") else
                                       post_key.size),
                   ptr(post_key), ptr(post_ad), int(emb.shape[1]), emb_dtype, ptr(emb),
                   rescore_mult, device, stream_ptr(stream))
     h = vp()
-    _check(ebr_build_index(C.byref(d), C.byref(h)), "ebr_build_index")
+    if debug_faults:
+        _check(ebr_debug_build_index(C.byref(d), debug_faults, C.byref(h)), "ebr_build_index")
+    else:
+        _check(ebr_build_index(C.byref(d), C.byref(h)), "ebr_build_index")
     return Index(h)
 
 
