@@ -497,8 +497,10 @@ static int bits_for(uint64_t n) {
   return b;
 }
 
-// True where a kernel can read p in place (device memory of this device).
+// True where a kernel can read 32-bit words at p in place (device memory of
+// this device, on a word boundary; a copy takes any address).
 static bool on_device(const void *p, int device) {
+  if (reinterpret_cast<uintptr_t>(p) % 4) return false;
   cudaPointerAttributes at;
   if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
     cudaGetLastError();
@@ -564,7 +566,7 @@ static int build_impl(const ebr_index_desc *desc, ebr_index *ix, uint32_t faults
   {
     const uint32_t *pk = desc->post_key, *pa = desc->post_ad;
     for (auto &e : ev) BCUDA(cudaEventCreate(&e));
-    // Inputs on the host are brought over first (not part of build_ms).
+    // Inputs that cannot be read in place are brought over first (not part of build_ms).
     if (nnz && !(on_device(pk, ix->device) && on_device(pa, ix->device))) {
       BTRY(dev_alloc(in, nnz * 8));
       BCUDA(cudaMemcpyAsync(in.p, pk, nnz * 4, cudaMemcpyDefault, st));
