@@ -316,11 +316,13 @@ int ebr_debug_wait_timeout(uint32_t timeout_us, void *stream);
  * failures in `faults` (0: none) made to happen.  EBR_FAULT_SORT_*: every wait
  * of that radix sort's look-backs (of the pairs, of the keys by popularity, of
  * the blocks) runs out at once, which has to end in EBR_ETIMEDOUT where that sort has
- * more than one tile of 4096 entries.
+ * more than one tile of 4096 entries.  EBR_FAULT_FORWARD_MEM: the device has no
+ * memory for the forward key table; the index is then built without one.
  */
 #define EBR_FAULT_SORT_PAIRS 1u
 #define EBR_FAULT_SORT_KEYS 2u
 #define EBR_FAULT_SORT_BLOCKS 4u
+#define EBR_FAULT_FORWARD_MEM 8u
 int ebr_debug_build_index(const ebr_index_desc *desc, uint32_t faults, ebr_index **out);
 
 /* ------------------------------------------------------- no-allocation form */

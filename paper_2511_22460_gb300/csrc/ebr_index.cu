@@ -537,9 +537,12 @@ struct BuildCounts {
   uint32_t flags, n_dup, max_keys, gc[kGroups], win_max[3], fwd[5], m_unique;
 };
 
-// faults: see ebr_debug_build_index.
-static int build_impl(const ebr_index_desc *desc, ebr_index *ix, uint32_t faults,
+// faults: see ebr_debug_build_index.  *forward: whether a forward table may be
+// built; on return, whether one was begun.
+static int build_impl(const ebr_index_desc *desc, ebr_index *ix, uint32_t faults, bool *forward,
                       cudaStream_t st) {
+  const bool may_forward = *forward;
+  *forward = false;
   // polls of a look-back in the sorts of the pairs, the keys by popularity, the blocks
   auto spins = [&](uint32_t fault) { return faults & fault ? 0u : prims::kSortSpins; };
   const uint64_t nnz = desc->nnz;
@@ -706,9 +709,12 @@ static int build_impl(const ebr_index_desc *desc, ebr_index *ix, uint32_t faults
     ix->fwd_quads = hc.fwd[4];
     ix->fwd_quad_bytes = n_keys < 65536u ? 256u : 384u;
     for (int g = 0; g < 4; g++) ix->fwd_max_quads[g] = hc.fwd[g];
-    if (m && n_keys < (1u << 24) - 1u && hc.fwd[3] <= kFwdMaxWinQuads &&
-        (uint64_t)hc.fwd[4] * 128 <= 2ull * m + 4ull * n_ads) {
-      BTRY(dev_alloc(ix->mem_fwd, (size_t)ix->fwd_quads * ix->fwd_quad_bytes + 256));
+    *forward = may_forward && m && n_keys < (1u << 24) - 1u && hc.fwd[3] <= kFwdMaxWinQuads &&
+               (uint64_t)hc.fwd[4] * 128 <= 2ull * m + 4ull * n_ads;
+    if (*forward) {
+      BTRY(faults & EBR_FAULT_FORWARD_MEM
+               ? EBR_ENOMEM
+               : dev_alloc(ix->mem_fwd, (size_t)ix->fwd_quads * ix->fwd_quad_bytes + 256));
       ix->fwd = w.fwd = (uint8_t *)ix->mem_fwd.p;
       w.quad_bytes = ix->fwd_quad_bytes;
       w.null_key = n_keys;
@@ -861,23 +867,32 @@ static int build_index(const ebr_index_desc *desc, uint32_t faults, ebr_index **
   int prev = 0;
   cudaGetDevice(&prev);
   EBR_CUDA_TRY(cudaSetDevice(desc->device));
-  ebr_index *ix = new ebr_index();
-  ix->device = desc->device;
-  ix->n_ads = desc->n_ads;
-  ix->n_keys = desc->n_keys;
-  ix->d = d;
-  ix->dtype = desc->emb_dtype;
-  ix->rescore_mult = desc->rescore_mult ? desc->rescore_mult : 4;
-  cudaDeviceGetAttribute(&ix->num_sms, cudaDevAttrMultiProcessorCount, desc->device);
   cudaStream_t st = (cudaStream_t)desc->stream;
-  int rc = build_impl(desc, ix, faults, st);
-  if (rc == EBR_OK) rc = upload_embeddings(desc, ix, st);
-  if (rc != EBR_OK) {
-    std::string msg = ebr_last_error();
+  ebr_index *ix = nullptr;
+  int rc = EBR_OK;
+  // A build with a forward table that runs out of device memory, there or later, is done
+  // again without one: the block-wise scan serves such an index.
+  for (bool forward = true;;) {
+    ix = new ebr_index();
+    ix->device = desc->device;
+    ix->n_ads = desc->n_ads;
+    ix->n_keys = desc->n_keys;
+    ix->d = d;
+    ix->dtype = desc->emb_dtype;
+    ix->rescore_mult = desc->rescore_mult ? desc->rescore_mult : 4;
+    cudaDeviceGetAttribute(&ix->num_sms, cudaDevAttrMultiProcessorCount, desc->device);
+    rc = build_impl(desc, ix, faults, &forward, st);
+    if (rc == EBR_OK) rc = upload_embeddings(desc, ix, st);
+    if (rc == EBR_OK) break;
+    const std::string msg = ebr_last_error();
     ebr_index_free(ix);
     set_error("%s", msg.c_str());
-    cudaSetDevice(prev);
-    return rc;
+    if (rc != EBR_ENOMEM || !forward) {
+      cudaSetDevice(prev);
+      return rc;
+    }
+    clear_error();
+    forward = false;
   }
   cudaSetDevice(prev);
   *out = ix;

@@ -30,7 +30,7 @@ W_DENSE, W_HASHED = 0, 1
 IO_DEVICE, IO_HOST = 0, 1
 QF_KEY_MAJOR = 1
 QF_WINDOW_MAJOR = 2
-FAULT_SORT_PAIRS, FAULT_SORT_KEYS, FAULT_SORT_BLOCKS = 1, 2, 4
+FAULT_SORT_PAIRS, FAULT_SORT_KEYS, FAULT_SORT_BLOCKS, FAULT_FORWARD_MEM = 1, 2, 4, 8
 _DTYPES = {"f32": F32, "bf16": BF16, "fp8e4m3": FP8E4M3}
 
 vp, u32, u64, i32 = C.c_void_p, C.c_uint32, C.c_uint64, C.c_int
