@@ -579,6 +579,21 @@ __global__ void __launch_bounds__((cons_warps<Elt>() + 2) * 32, 1)
         const float z0 = (up ? y[2] : y[0]) + r0, z1 = (up ? y[3] : y[1]) + r1;
         const float z = (odd ? z1 : z0) + __shfl_xor_sync(0xffffffffu, odd ? z0 : z1, 1);
         dot = __shfl_sync(0xffffffffu, z, 4 * (lane & 7) + (lane >> 3));
+        // An infinite element times a piece or a column that is zero is NaN,
+        // which a sum with h_u itself need not be: such rows are summed again
+        // by FP32 multiply-adds.  (E4M3 has no infinities.)
+        if (!kF8 && __any_sync(0xffffffffu, in && !(fabsf(dot) < INFINITY))) {
+          const uint8_t *row = stage + (size_t)(rs * 32u + lane) * Sh::kRowBytes;
+          float again = 0.f;
+#pragma unroll 1
+          for (int c = 0; c < Sh::kChunks; c++) {
+            float f[Tr::kVec];
+            Tr::load(*reinterpret_cast<const uint4 *>(row + c * 16), f);
+#pragma unroll
+            for (int e = 0; e < Tr::kVec; e++) again = fmaf(s_h[c * Tr::kVec + e], f[e], again);
+          }
+          if (!(fabsf(dot) < INFINITY)) dot = again;
+        }
       } else {
         // with two threads per row, rows 16 ps .. 16 ps + 15
 #pragma unroll
