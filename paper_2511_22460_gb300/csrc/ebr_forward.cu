@@ -399,12 +399,14 @@ __global__ void __launch_bounds__((cons_warps<Elt>() + 2) * 32, 1)
     }
   } else {
     float sc = 1.f, inv = 1.f;
-    if (kF8) {  // the largest |h_u| to [1, 2)
+    if (kF8) {  // the largest finite |h_u| to [1, 4); both powers of two are normal numbers
       float mx = 0.f;
-      for (int i = lane; i < D; i += 32) mx = fmaxf(mx, fabsf(s_h[i]));
+      for (int i = lane; i < D; i += 32) {
+        const float x = fabsf(s_h[i]);
+        mx = fmaxf(mx, x < INFINITY ? x : 0.f);
+      }
       for (int o = 16; o; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-      int e = (int)(__float_as_uint(mx) >> 23) - 127;
-      e = mx > 0.f && mx < INFINITY ? max(-100, min(100, e)) : 0;
+      const int e = mx > 0.f ? max(-126, min(126, (int)(__float_as_uint(mx) >> 23) - 127)) : 0;
       sc = pow2f(-e);
       inv = pow2f(e);
     }

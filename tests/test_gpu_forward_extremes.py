@@ -80,3 +80,35 @@ def test_ads_of_minus_infinity_take_no_place_in_the_top_k():
     assert np.all(np.abs(sc.cpu().numpy() - ref[got]) <= tol[got])
     kth = np.sort(ref)[::-1][k - 1]
     assert np.all(ref[got] >= kth - 2 * tol[np.isfinite(ref)].max())
+
+
+@pytest.mark.parametrize("d", [16, 64, 128])
+@pytest.mark.parametrize("top", [1e30, 9e34, 1.8e35])
+def test_huge_user_vectors_on_fp8_tables(d, top):
+    # four elements a row: the sum of h x codes (at most 448) stays finite too
+    n = 3_000
+    rng = np.random.default_rng(d)
+    emb = np.zeros((n, d), np.float32)
+    for i in range(4):
+        emb[np.arange(n), rng.integers(0, d, n)] = rng.standard_normal(n) / d
+    ix = _index(emb, "fp8e4m3")
+    table = _table(ix, "fp8e4m3")
+    h = rng.uniform(-1, 1, d).astype(np.float32)
+    h = h / np.abs(h).max() * np.float32(top)
+    ref = (table * h.astype(np.float64)).sum(1)
+    tol = 1e-5 * (np.abs(table) @ np.abs(h).astype(np.float64))
+    assert np.all(np.abs(_scores(ix, h) - ref) <= tol)
+
+
+def test_an_infinite_user_element_on_an_fp8_table():
+    n, d = 3_000, 64
+    rng = np.random.default_rng(1)
+    ix = _index(rng.standard_normal((n, d)).astype(np.float32), "fp8e4m3")
+    table = _table(ix, "fp8e4m3")
+    h = (rng.standard_normal(d) * 1e6).astype(np.float32)  # beyond FP16 unless scaled
+    h[5] = INF
+    with np.errstate(invalid="ignore"):
+        ref = (table * h.astype(np.float64)).sum(1)  # infinite, or NaN where the element is 0
+    got = _scores(ix, h)
+    assert np.array_equal(np.isnan(got), np.isnan(ref))
+    assert np.array_equal(got[~np.isnan(ref)].astype(np.float64), ref[~np.isnan(ref)])
