@@ -112,11 +112,15 @@ struct FwdShape {
 };
 
 // The inner products of BF16 and FP8 rows on the tensor pipe: 16 rows x 16
-// elements per mma.sync, FP32 accumulators.  h_u is split exactly into three
-// 16-bit pieces, which are three of the eight columns: BF16 pieces of 8 bits
-// each for BF16 rows, FP16 pieces (h_u scaled by a power of two, the pieces by
-// 2^11) for FP8 rows, whose elements are FP16 values.  Every product is exact
-// in FP32, so the result is an FP32 sum like the one of FP32 multiply-adds.
+// elements per mma.sync, FP32 accumulators.  h_u is split into 16-bit pieces,
+// one to a column: three BF16 pieces of 8 bits each for BF16 rows (exact for
+// |h_u| of 2^-109 and more, below which the last one loses bits); for FP8 rows,
+// whose elements are FP16 values, FP16 pieces of 11 bits, h_u scaled by a power of two
+// so that its largest element is near 1 and piece n by 2^11n.  Three of those hold
+// 24 bits of an element down to 2^-22 of the largest (an element of 2^-32 of it
+// would keep 15, of 2^-40 seven); the other five columns, which the instruction
+// multiplies anyway, carry it on to 2^-77.  Every product is exact
+// in FP32; how the tensor pipe rounds their sum is its own.
 // A thread's 16-byte chunk supplies the elements of its own k positions (the
 // order of the sum over k is free), so rows are read as they lie.
 __device__ __forceinline__ void mma_16816(float *d, uint32_t a0, uint32_t a1, uint32_t a2,
@@ -134,8 +138,8 @@ __device__ __forceinline__ void mma_16816(float *d, uint32_t a0, uint32_t a1, ui
         : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
         : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
 }
-// 16 bits of piece n (0, 1, 2; else 0) of h.  A value that is not finite is
-// its own first piece.
+// 16 bits of piece n of h (BF16: 0, 1, 2, else 0).  A value that is not finite
+// is its own first piece.
 __device__ __forceinline__ uint32_t piece_bf16(float h, int n) {
   float r = h;
   uint32_t bits = 0;
@@ -149,7 +153,7 @@ __device__ __forceinline__ uint32_t piece_bf16(float h, int n) {
 __device__ __forceinline__ uint32_t piece_f16(float h, int n) {
   float r = h;
   uint32_t bits = 0;
-  for (int i = 0; i < 3; i++) {
+  for (int i = 0; i < 8; i++) {
     const __half x = __float2half_rn(r);
     if (i == n) bits = (uint32_t)__half_as_ushort(x);
     r = fabsf(h) < INFINITY ? (r - __half2float(x)) * 2048.f : 0.f;
@@ -385,7 +389,7 @@ __global__ void __launch_bounds__((cons_warps<Elt>() + 2) * 32, 1)
   const int qd = lane % Sh::kTPR;
   const uint32_t rot = (lane / Sh::kRowsPer128) % Sh::kCPT;
   float hreg[kMma ? 1 : Sh::kHPT];
-  // BF16, FP8: this thread's part of the three columns of pieces (column
+  // BF16, FP8: this thread's part of the columns of pieces (column
   // lane / 4, chunk 4 step + lane % 4), and the weights of columns 2 (lane % 4)
   // and 2 (lane % 4) + 1
   uint32_t breg[kMma ? Sh::kSteps * Sh::kMmas * 2 : 1];
@@ -410,10 +414,11 @@ __global__ void __launch_bounds__((cons_warps<Elt>() + 2) * 32, 1)
       sc = pow2f(-e);
       inv = pow2f(e);
     }
-    const float step = kF8 ? pow2f(-11) : 1.f;
     const int t = lane & 3, n = lane >> 2;
-    cw0 = t == 0 ? inv : (t == 1 ? inv * step * step : 0.f);
-    cw1 = t == 0 ? inv * step : 0.f;
+    // FP8: column n weighs inv x 2^-11n, down to 0 where a piece has nothing left
+    cw0 = kF8 ? inv : (t < 2 ? 1.f : 0.f);
+    for (int i = 0; kF8 && i < 2 * t; i++) cw0 *= pow2f(-11);
+    cw1 = kF8 ? cw0 * pow2f(-11) : (t == 0 ? 1.f : 0.f);
 #pragma unroll
     for (int j = 0; j < Sh::kSteps; j++)
 #pragma unroll

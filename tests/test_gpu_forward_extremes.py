@@ -112,3 +112,22 @@ def test_an_infinite_user_element_on_an_fp8_table():
     got = _scores(ix, h)
     assert np.array_equal(np.isnan(got), np.isnan(ref))
     assert np.array_equal(got[~np.isnan(ref)].astype(np.float64), ref[~np.isnan(ref)])
+
+
+@pytest.mark.parametrize("d", [16, 64, 128])
+@pytest.mark.parametrize("dtype", ["bf16", "fp8e4m3"])
+def test_ads_that_only_see_small_user_elements(dtype, d):
+    # each ad is nonzero only where h_u has one of these magnitudes
+    n, ratio = 4_000, [0, -25, -32, -40, -60, -75, -40, -32]
+    rng = np.random.default_rng(d)
+    part = np.arange(n) % len(ratio)
+    own = np.arange(d) % len(ratio)
+    emb = rng.standard_normal((n, d)).astype(np.float32) * (part[:, None] == own[None, :])
+    ix = _index(emb.astype(np.float32), dtype)
+    table = _table(ix, dtype)
+    h = np.ldexp(rng.uniform(1, 2, d), np.array(ratio)[own]).astype(np.float32)
+    for scale in (-30, 0, 50):
+        hs = np.ldexp(h, scale).astype(np.float32)
+        ref = (table * hs.astype(np.float64)).sum(1)
+        tol = 1e-5 * (np.abs(table) @ np.abs(hs).astype(np.float64))
+        assert np.all(np.abs(_scores(ix, hs) - ref) <= tol)
