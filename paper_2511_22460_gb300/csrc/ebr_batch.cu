@@ -1700,11 +1700,15 @@ static int stage(void *dst, const void *src, size_t bytes, int io, cudaStream_t 
   return EBR_OK;
 }
 
-// The last row of every group's slice of w^T: the lists' padding key.
+// The last row of every group's slice of w^T: the lists' padding key.  (One
+// call per group: a slice may be longer than a 2-D memset's pitch, 2^31 - 1.)
 static cudaError_t clear_zero_rows(const ebr_index *ix, BatchWs &w, uint32_t Bq, cudaStream_t st) {
-  const size_t slice = ((size_t)ix->n_keys + 1) * kGroup * 4;
-  return cudaMemset2DAsync((char *)w.wT.p + (size_t)ix->n_keys * kGroup * 4, slice, 0, kGroup * 4,
-                           Bq / kGroup, st);
+  const size_t row = kGroup * 4, slice = ((size_t)ix->n_keys + 1) * row;
+  for (uint32_t g = 0; g < Bq / kGroup; g++) {
+    const cudaError_t e = cudaMemsetAsync((char *)w.wT.p + (g + 1) * slice - row, 0, row, st);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
 }
 
 static void (*window_kernel(bool f8, int mode))(BatchArgs) {
@@ -2308,9 +2312,9 @@ int loop_build(ebr_index *ix, const ebr_cross *cross, uint32_t max_user_vals, Ba
       rc = expand_transposed(cross, (const uint32_t *)w.user_vals.p, d_uptr, d_base,
                              std::min(Bmax, Bp), Bp, (float *)w.wT.p, &L.ctrl->flags, st, B_dev,
                              ix->key_id);
-    if (rc == EBR_OK) {
-      clear_zero_rows(ix, w, Bp, st);
-      cudaMemsetAsync(w.uhist.p, 0, user_hist_bytes(Bmax), st);
+    if (rc == EBR_OK) e = clear_zero_rows(ix, w, Bp, st);
+    if (rc == EBR_OK && e == cudaSuccess) e = cudaMemsetAsync(w.uhist.p, 0, user_hist_bytes(Bmax), st);
+    if (rc == EBR_OK && e == cudaSuccess) {
       kern<<<dim3(grid, Bp / kGroup), kBatchThreads, pl.smem, st>>>(ba);
       k_batch_merge<<<std::min(Bmax, Bp), kMergeThreads, msm, st>>>(
           (const CandEntry *)w.cand.p, (const uint32_t *)w.cand_n.p,
