@@ -1551,13 +1551,15 @@ static bool plan_smem(const ebr_index *ix, uint32_t B, BatchPlan *p) {
   return false;
 }
 
+// (The last but one condition bounds w^T, 17 GB: a batch over a larger key space is served
+// by single requests, whose scratch does not grow with the users.)
 bool batch_index_ok(const ebr_index *ix, const ebr_cross *cross, uint32_t batch) {
   BatchPlan p;
   return (ix->dtype == EBR_BF16 || ix->dtype == EBR_FP8E4M3) && (ix->d == 64 || ix->d == 128) &&
          batch >= 2 && batch <= (uint32_t)kMaxUsers && cross && cross->n_keys == ix->n_keys &&
          ix->n_win > 0 && ix->ad_nkeys.p && ix->max_keys_per_ad > 0 &&
          ix->max_keys_per_ad <= kMaxBatchKeysPerAd &&
-         ((uint64_t)ix->n_keys + 1) * kGroup < (1ull << 32) &&
+         ((uint64_t)ix->n_keys + 1) * users_padded(batch) < (1ull << 32) &&
          plan_smem(ix, batch, &p);
 }
 

@@ -65,3 +65,9 @@ def _batch(fields, vocab, B, n_ads=3_000, d=64, k=40):
 @pytest.mark.parametrize("vocab", [932_000, 1_000_000])  # 2.15e9 and 2.3e9 bytes a slice
 def test_slices_longer_than_a_2d_memsets_pitch(vocab):
     assert _batch(9, vocab, 70) == 70
+
+
+@pytest.mark.parametrize("B,batched", [(70, 70), (256, 0)])
+def test_the_largest_weights_of_a_batch(B, batched):
+    # 17 M keys (no forward table): 128 users' weights are 8.7 GB, 256 users' over the bound
+    assert _batch(17, 1_000_000, B) == batched
