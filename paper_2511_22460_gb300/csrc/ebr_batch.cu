@@ -163,7 +163,7 @@ static int debug_gemm(bool f8, const void *A, uint32_t n, const void *U, uint32_
   EBR_CUDA_TRY(cudaMemsetAsync(flags, 0, 4, st));
   const size_t smem = 1024 + (size_t)d * eb * (128 + B);
   auto kern = f8 ? k_gemm_tc<true> : k_gemm_tc<false>;
-  EBR_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  EBR_CUDA_TRY(allow_smem(kern, 1024 + 128 * 2 * (128 + 256)));  // (d = 128, B = 256)
   kern<<<(n + 127) / 128, 128, smem, st>>>(ma, mu, n, B, d, out, flags);
   EBR_CUDA_TRY(cudaGetLastError());
   uint32_t hf = 0;
@@ -1515,6 +1515,7 @@ static uint32_t users_padded(uint32_t B) { return (B + kGroup - 1) / kGroup * kG
 // group's slice of w^T.  One 256-ad stage (or two of 128) is enough, since the next window's MMAs
 // wait for this window's accumulators to be read anyway, and what is left is
 // L1 for the gathers.
+constexpr size_t kBatchSmemBudget = 220 * 1024;
 static bool plan_smem(const ebr_index *ix, uint32_t B, BatchPlan *p) {
   p->Bq = users_padded(B);
   p->list_cap = kBWin * ix->max_keys_per_ad;  // 8 runs x 32 ads x rows
@@ -1529,7 +1530,6 @@ static bool plan_smem(const ebr_index *ix, uint32_t B, BatchPlan *p) {
   const size_t a_stage = (size_t)p->kb_n * win * p->tile_row;
   const size_t hist = (size_t)kTrimWarps * 256 * 4;
   const size_t fixed = 1024 + u_bytes + p->sa * a_stage + hist;
-  const size_t budget = 220 * 1024;
   const uint32_t mq = ix->fwd_max_quads[0];
   const size_t raw = (size_t)mq * win * (ix->fwd_quad_bytes > 256u ? 12 : 8);
   if (ix->fwd) {
@@ -1537,16 +1537,16 @@ static bool plan_smem(const ebr_index *ix, uint32_t B, BatchPlan *p) {
     p->lb = 1;
     p->mode = kForwardSw;
     p->smem = fixed + raw + (size_t)mq * 4 * win * 2 + wt;
-    if (ix->n_keys < 4096 && p->smem <= budget) return true;
+    if (ix->n_keys < 4096 && p->smem <= kBatchSmemBudget) return true;
     p->mode = kForward;
     p->smem = fixed + raw + (size_t)mq * 4 * win * 4;
-    if (p->smem <= budget) return true;
+    if (p->smem <= kBatchSmemBudget) return true;
     return false;
   }
   p->mode = kWalk;
   for (p->lb = 2; p->lb >= 1; p->lb--) {
     p->smem = fixed + p->lb * ((size_t)kListHdr + p->list_cap) * 4;
-    if (p->smem <= budget) return true;
+    if (p->smem <= kBatchSmemBudget) return true;
   }
   return false;
 }
@@ -1901,15 +1901,13 @@ int batch_launch(ebr_index *ix, const ebr_cross *cross, const ebr_query *q, uint
   BatchArgs a;
   EBR_TRY(fill_batch_args(ix, B, pl, w, kk, has_filter, ctrl, nullptr, &a));
   auto kern = window_kernel(f8, pl.mode);
-  EBR_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    (int)pl.smem));
+  EBR_CUDA_TRY(allow_smem(kern, kBatchSmemBudget));
   if (prof) EBR_CUDA_TRY(cudaEventRecord(ev[1], st));
   kern<<<dim3(grid, Bp / kGroup), kBatchThreads, pl.smem, st>>>(a);
   EBR_CUDA_TRY(cudaGetLastError());
   if (prof) EBR_CUDA_TRY(cudaEventRecord(ev[2], st));
   const size_t msm = merge_smem(kscan_max, kmax);
-  EBR_CUDA_TRY(cudaFuncSetAttribute(k_batch_merge, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    (int)msm));
+  EBR_CUDA_TRY(allow_smem(k_batch_merge, merge_smem(8192, 8192)));
   k_batch_merge<<<B, kMergeThreads, msm, st>>>(
       (const CandEntry *)w.cand.p, (const uint32_t *)w.cand_n.p,
       (const unsigned long long *)w.cand_thr.p, (uint32_t)grid, B, pl.cap_u, kk, kk + B, kmax,
@@ -2220,11 +2218,9 @@ int loop_build(ebr_index *ix, const ebr_cross *cross, uint32_t max_user_vals, Ba
   uint32_t *d_uptr = (uint32_t *)w.user_ptr.p;
   uint32_t *d_base = d_uptr + (size_t)Bmax * (fu + 1);
   auto kern = window_kernel(f8, pl.mode);
-  EBR_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    (int)pl.smem));
+  EBR_CUDA_TRY(allow_smem(kern, kBatchSmemBudget));
   const size_t msm = merge_smem(kscan_max, L.kmax);
-  EBR_CUDA_TRY(cudaFuncSetAttribute(k_batch_merge, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    (int)msm));
+  EBR_CUDA_TRY(allow_smem(k_batch_merge, merge_smem(8192, 8192)));
   LoopArgs la;
   memset(&la, 0, sizeof(la));
   la.nsw = 0;  // 64, 128, ... and, last, the table's own width

@@ -849,7 +849,7 @@ int launch_t(const FwdCall &c, FwdArgs a, cudaStream_t st) {
   if constexpr (std::is_same<Elt, float>::value) {
     if (c.tree) kern = k_forward<float, D, false, true>;
   }
-  EBR_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  EBR_CUDA_TRY(allow_smem(kern, kFwdSmemBudget));
   EBR_CUDA_TRY(launch_pdl(kern, grid, (cons_warps<Elt>() + 2) * 32, smem, st, a));
   return EBR_OK;
 }

@@ -786,7 +786,7 @@ static int launch_fused_t(const ebr_index *ix, FusedArgs a, int max_grid, cudaSt
   if constexpr (!ALL) {
     if (a.cand_g) kern = k_fused_window<Elt, D, false, true>;
   }
-  EBR_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  EBR_CUDA_TRY(allow_smem(kern, kFusedSmemBudget));
   int occ = 0;
   EBR_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, kFusedThreads, smem));
   if (occ < 1) {

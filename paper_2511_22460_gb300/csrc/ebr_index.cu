@@ -91,6 +91,10 @@ constexpr int kWinThreads = 256, kWinWarps = kWinThreads / 32;
 constexpr uint32_t kWinChunk = 4096;  // words walked at a time; a block has at most 256
 constexpr uint32_t kWinRows = kWinChunk / kWinThreads;
 constexpr uint32_t kFwdMaxWinQuads = 128;  // most forward quads of one window (176 KB to build)
+// Shared memory a window of `quads` is put together in: the quads and their entries.
+constexpr size_t fwd_win_smem(uint32_t quads, uint32_t quad_bytes) {
+  return (size_t)quads * (quad_bytes + 1024);
+}
 
 struct WinArgs {
   const uint64_t *x;            // sorted distinct words
@@ -743,7 +747,7 @@ static int build_impl(const ebr_index_desc *desc, ebr_index *ix, uint32_t faults
                                                   &cnt->flags);
       BCUDA(cudaGetLastError());
     }
-    const size_t fwd_smem = w.fwd ? (size_t)hc.fwd[3] * (w.quad_bytes + 1024) : 0;
+    const size_t fwd_smem = w.fwd ? fwd_win_smem(hc.fwd[3], w.quad_bytes) : 0;
     // blocks: window of each, then (key, place) records three times over (the
     // sort's input and its two buffers); the sort's scratch is the words'
     const bool k32 = kb + 4 <= 32;
@@ -764,8 +768,7 @@ static int build_impl(const ebr_index_desc *desc, ebr_index *ix, uint32_t faults
     if (nb) {
       const uint32_t grid = std::min<uint32_t>(n_win, 1u << 20);
       auto kern = k32 ? k_windows<true, uint32_t> : k_windows<true, uint64_t>;
-      BCUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)std::max<size_t>(fwd_smem, 16)));
+      BCUDA(allow_smem(kern, fwd_win_smem(kFwdMaxWinQuads, 384)));
       kern<<<grid, kWinThreads, fwd_smem, st>>>(w);
       BCUDA(cudaGetLastError());
     }

@@ -273,6 +273,14 @@ constexpr size_t kHistWords = 4096;  // candidate-score histogram of the fused s
 constexpr size_t kCtrlBytes = 256;   // Ctrl block, then the histogram, in one buffer (one memset)
 inline uint32_t *ws_hist(const Workspace &w) { return (uint32_t *)((char *)w.ctrl.p + kCtrlBytes); }
 
+// Lets launches of kern have up to `most` bytes of dynamic shared memory.  The
+// limit is the kernel's and not the launch's: `most` is the same in every call,
+// or a call of another thread could lower it before this one's launch.
+template <typename... KArgs>
+inline cudaError_t allow_smem(void (*kern)(KArgs...), size_t most) {
+  return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
+}
+
 // Launches kern on st with programmatic stream serialization: it may start
 // while the previous kernel of the stream is still running, and its threads
 // that read that kernel's results call pdl_wait first.

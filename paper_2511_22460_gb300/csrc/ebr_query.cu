@@ -921,8 +921,7 @@ static int final_select_init() {
   EBR_CUDA_TRY(cudaGetDevice(&dev));
   const uint64_t bit = dev < 64 ? 1ull << dev : 0ull;
   if (done.load() & bit) return EBR_OK;
-  EBR_CUDA_TRY(cudaFuncSetAttribute(k_final_select, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    (int)final_smem(8192)));
+  EBR_CUDA_TRY(allow_smem(k_final_select, final_smem(8192)));
   done.fetch_or(bit);
   return EBR_OK;
 }
@@ -958,6 +957,8 @@ static uint32_t pow2_at_least(uint32_t x) {
   return p;
 }
 
+constexpr size_t kScanSmemMax = 224 * 1024;  // beside its static shared memory
+
 struct ScanPlan {
   int grid = 0;
   uint32_t stages = 0, cap = 0;
@@ -988,8 +989,7 @@ static int launch_scan_t(const ebr_index *ix, ScanArgs a, cudaStream_t st) {
   a.cap = p.cap;
   a.stages = p.stages;
   auto kern = k_scan_topk<Elt, D, MODE>;
-  EBR_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    (int)p.smem));
+  EBR_CUDA_TRY(allow_smem(kern, kScanSmemMax));
   kern<<<p.grid, kScanThreads, p.smem, st>>>(a);
   EBR_CUDA_TRY(cudaGetLastError());
   return EBR_OK;
@@ -1202,6 +1202,8 @@ __global__ void __launch_bounds__(kExpThreads)
   if (bad) atomicOr(flags, bad);
 }
 
+constexpr size_t kExpandSmemMax = 200 * 1024;  // pair lists a CTA of the expansion stages
+
 int expand_transposed(const ebr_cross *c, const uint32_t *users, const uint32_t *uptr,
                       const uint32_t *base, uint32_t batch, uint32_t Bp, float *wT,
                       uint32_t *flags, cudaStream_t st, const uint32_t *batch_dev,
@@ -1221,8 +1223,7 @@ int expand_transposed(const ebr_cross *c, const uint32_t *users, const uint32_t 
   auto kern = uptr ? (cv.hashed ? pick(yes, yes) : pick(yes, no))
                    : (cv.hashed ? pick(no, yes) : pick(no, no));
   if (smem > 48 * 1024)
-    EBR_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)std::min<size_t>(smem, 200 * 1024)));
+    EBR_CUDA_TRY(allow_smem(kern, kExpandSmemMax));
   kern<<<blocks, kExpThreads, smem, st>>>(cv, users, uptr, base, batch, Bp, wT, flags, batch_dev,
                                           key_id);
   EBR_CUDA_TRY(cudaGetLastError());
@@ -1242,9 +1243,8 @@ static int expand_into(const ebr_cross *c, const uint32_t *users, uint32_t batch
     return EBR_EINVAL;
   }
   if (smem > 48 * 1024)
-    EBR_CUDA_TRY(cudaFuncSetAttribute(k_expand, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)std::min<size_t>(smem, 200 * 1024)));
-  if (smem > 200 * 1024) {
+    EBR_CUDA_TRY(allow_smem(k_expand, kExpandSmemMax));
+  if (smem > kExpandSmemMax) {
     set_error("query expansion: %u cross pairs exceed the staging area", c->n_pairs);
     return EBR_EINVAL;
   }
