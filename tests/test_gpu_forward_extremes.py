@@ -63,21 +63,27 @@ def test_infinite_elements_of_bf16_tables(d, huge):
         assert np.all(np.abs(got[fin] - ref[fin]) <= tol)
 
 
-def test_ads_of_minus_infinity_take_no_place_in_the_top_k():
-    n, d, k = 5_000, 64, 20
+@pytest.mark.parametrize("n", [5_000, 20_000])  # keys of all ads, and running bounds
+@pytest.mark.parametrize("sign", [-1, 1])
+def test_infinite_ads_in_the_top_k(n, sign):
+    # at least 500 infinite ads, more than (R - 1) K: last, or first by their ids
+    d, k = 64, 20
     rng = np.random.default_rng(0)
     emb = rng.standard_normal((n, d)).astype(np.float32)
-    emb[::10, 3] = -INF  # 500 ads, more than (R - 1) K
+    emb[::10, 3] = sign * INF
     h = np.abs(rng.standard_normal(d)).astype(np.float32)
     ix = _index(emb, "bf16")
     ids = torch.empty(k, dtype=torch.int32, device=DEV)
     sc = torch.empty(k, device=DEV)
     ebr.score_topk(ix, None, [_query(h, k=k)], ids, sc)
+    got, sc = ids.cpu().numpy(), sc.cpu().numpy()
+    if sign > 0:
+        assert np.array_equal(got, 10 * np.arange(k)) and np.all(sc == INF)
+        return
     ref = (emb.astype(np.float64) * h).sum(1)
     tol = 1e-5 * (np.abs(emb).astype(np.float64) * h).sum(1)
-    got = ids.cpu().numpy()
     assert np.unique(got).size == k and np.all(np.isfinite(ref[got]))
-    assert np.all(np.abs(sc.cpu().numpy() - ref[got]) <= tol[got])
+    assert np.all(np.abs(sc - ref[got]) <= tol[got])
     kth = np.sort(ref)[::-1][k - 1]
     assert np.all(ref[got] >= kth - 2 * tol[np.isfinite(ref)].max())
 
