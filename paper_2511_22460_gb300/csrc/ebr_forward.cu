@@ -586,21 +586,6 @@ __global__ void __launch_bounds__((cons_warps<Elt>() + 2) * 32, 1)
         const float z0 = (up ? y[2] : y[0]) + r0, z1 = (up ? y[3] : y[1]) + r1;
         const float z = (odd ? z1 : z0) + __shfl_xor_sync(0xffffffffu, odd ? z0 : z1, 1);
         dot = __shfl_sync(0xffffffffu, z, 4 * (lane & 7) + (lane >> 3));
-        // An infinite element times a piece or a column that is zero is NaN,
-        // which a sum with h_u itself need not be: such rows are summed again
-        // by FP32 multiply-adds.  (E4M3 has no infinities.)
-        if (!kF8 && __any_sync(0xffffffffu, in && !(fabsf(dot) < INFINITY))) {
-          const uint8_t *row = stage + (size_t)(rs * 32u + lane) * Sh::kRowBytes;
-          float again = 0.f;
-#pragma unroll 1
-          for (int c = 0; c < Sh::kChunks; c++) {
-            float f[Tr::kVec];
-            Tr::load(*reinterpret_cast<const uint4 *>(row + c * 16), f);
-#pragma unroll
-            for (int e = 0; e < Tr::kVec; e++) again = fmaf(s_h[c * Tr::kVec + e], f[e], again);
-          }
-          if (!(fabsf(dot) < INFINITY)) dot = again;
-        }
       } else {
         // with two threads per row, rows 16 ps .. 16 ps + 15
 #pragma unroll
@@ -669,6 +654,27 @@ __global__ void __launch_bounds__((cons_warps<Elt>() + 2) * 32, 1)
       float wide = sd.wide;
       if (keys)
         wide = ((float)(ts.all - ts.c1) * u0 + (float)ts.c1 * u1) + ((float)ts.c2 * u2 + ts.fp);
+      if constexpr (kMma && !kF8) {
+        // An infinite element times a piece or a column that is zero is NaN,
+        // which a sum with h_u itself need not be: such rows are summed again
+        // by FP32 multiply-adds (E4M3 has no infinities).  Here and from global
+        // memory, so that the stage and the gathers do not wait for the sum (1M ads
+        // of 128 elements from host buffers 201 us with that, 197 us so).
+        if (__any_sync(0xffffffffu, in && !(fabsf(dot) < INFINITY))) {
+          if (in && !(fabsf(dot) < INFINITY)) {
+            const uint4 *row = reinterpret_cast<const uint4 *>(a.emb) + (uint64_t)ad * Sh::kChunks;
+            dot = 0.f;
+#pragma unroll 1
+            for (int c = 0; c < Sh::kChunks; c++) {
+              float f[Tr::kVec];
+              Tr::load(__ldg(row + c), f);
+#pragma unroll
+              for (int e = 0; e < Tr::kVec; e++) dot = fmaf(s_h[c * Tr::kVec + e], f[e], dot);
+            }
+          }
+          __syncwarp();
+        }
+      }
       float score = dot;
       if (a.scale) score *= sd.scale;
       score += wide;
