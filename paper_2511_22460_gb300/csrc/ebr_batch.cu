@@ -245,7 +245,7 @@ extern "C" int ebr_debug_wait_timeout(uint32_t timeout_us, void *stream) {
 //                      users and the odd users (the user table is stored in
 //                      that pair order), each replicated four times down the
 //                      128 TMEM lanes; deep[user][ad] (Eq. 1) lands in TMEM;
-//   list warps (2)  -- (kWalk, indexes without a forward table) lay out, per
+//   list warps (4; 2) -- (kWalk, indexes without a forward table) lay out, per
 //                      run of 32 ads, a key table T[r][i] = r-th key of ad i
 //                      (the window's slice of L, transposed; short ads padded
 //                      with a zero row of w^T) by a walk over the window's
@@ -278,12 +278,17 @@ extern "C" int ebr_debug_wait_timeout(uint32_t timeout_us, void *stream) {
 namespace ebr {
 
 constexpr int kBWin = 256;
-constexpr int kEpiWarps = 16, kListWarps = 2;
-constexpr int kEpiThreads = kEpiWarps * 32, kListThreads = kListWarps * 32;
-constexpr int kMmaWarp = kEpiWarps + kListWarps, kProdWarpB = kMmaWarp + 1;
-constexpr int kBatchThreads = (kProdWarpB + 1) * 32;  // 640
+// MODE: where an ad's keys come from (see above).
+enum { kWalk = 0, kForward = 1, kForwardSw = 2 };
+constexpr int kEpiWarps = 16, kEpiThreads = kEpiWarps * 32;
+// kWalk: a group's lists are built anew for every group of users, which two warps
+// could not do in the time of an epilogue (256 users x 5M BF16 ads of 24 keys
+// 16.8 ms with two, 11.9 with four, 15.4 with one pass of two warps for all users and
+// no groups).  With a forward table one of two warps raises thresholds.
+constexpr int list_warps(int mode) { return mode == kWalk ? 4 : 2; }
+constexpr int batch_threads(int mode) { return (kEpiWarps + list_warps(mode) + 2) * 32; }
 constexpr int kMaxUsers = 256;
-static_assert(kBWin % (kListWarps * 32) == 0, "list threads split the window's ads evenly");
+static_assert(kBWin % (list_warps(kWalk) * 32) == 0, "list threads split the window's ads evenly");
 // List buffer: run_off[8], run_rows[8], fill[256], then the run tables.
 constexpr uint32_t kListHdr = 8 + 8 + kBWin;
 constexpr uint32_t kMaxBatchKeysPerAd = 64;  // longest key list the batched tables hold
@@ -590,8 +595,6 @@ struct Row4 {
   float2 x[4];
 };
 
-// MODE: where an ad's keys come from (see above).
-enum { kWalk = 0, kForward = 1, kForwardSw = 2 };
 // Ads of a window: the block-wise lists are per 256 ads; with the forward table
 // 128, so that two windows' accumulators (2 x 128 columns each) fit TMEM and
 // the MMAs of one run while the other's are read.
@@ -608,8 +611,10 @@ __device__ __forceinline__ void cp_async_wait() {
 }
 
 template <bool F8, int MODE>
-__global__ void __launch_bounds__(kBatchThreads, 1) k_batch_window(const __grid_constant__ BatchArgs a) {
+__global__ void __launch_bounds__(batch_threads(MODE), 1) k_batch_window(const __grid_constant__ BatchArgs a) {
   constexpr bool FWD = MODE != kWalk, SW = MODE == kForwardSw;
+  constexpr int kListThreads = list_warps(MODE) * 32, kBatchThreads = batch_threads(MODE);
+  constexpr int kMmaWarp = kEpiWarps + list_warps(MODE), kProdWarpB = kMmaWarp + 1;
   constexpr uint32_t kWin = FWD ? kFwdWin : kBWin;      // ads of a window
   constexpr uint32_t kWarpAds = kWin / kEpiWarps;       // of them per epilogue warp
   constexpr uint32_t kTb = accum_bufs(FWD);             // accumulator buffers
@@ -1903,7 +1908,7 @@ int batch_launch(ebr_index *ix, const ebr_cross *cross, const ebr_query *q, uint
   auto kern = window_kernel(f8, pl.mode);
   EBR_CUDA_TRY(allow_smem(kern, kBatchSmemBudget));
   if (prof) EBR_CUDA_TRY(cudaEventRecord(ev[1], st));
-  kern<<<dim3(grid, Bp / kGroup), kBatchThreads, pl.smem, st>>>(a);
+  kern<<<dim3(grid, Bp / kGroup), batch_threads(pl.mode), pl.smem, st>>>(a);
   EBR_CUDA_TRY(cudaGetLastError());
   if (prof) EBR_CUDA_TRY(cudaEventRecord(ev[2], st));
   const size_t msm = merge_smem(kscan_max, kmax);
@@ -2313,7 +2318,7 @@ int loop_build(ebr_index *ix, const ebr_cross *cross, uint32_t max_user_vals, Ba
     if (rc == EBR_OK) e = clear_zero_rows(ix, w, Bp, st);
     if (rc == EBR_OK && e == cudaSuccess) e = cudaMemsetAsync(w.uhist.p, 0, user_hist_bytes(Bmax), st);
     if (rc == EBR_OK && e == cudaSuccess) {
-      kern<<<dim3(grid, Bp / kGroup), kBatchThreads, pl.smem, st>>>(ba);
+      kern<<<dim3(grid, Bp / kGroup), batch_threads(pl.mode), pl.smem, st>>>(ba);
       k_batch_merge<<<std::min(Bmax, Bp), kMergeThreads, msm, st>>>(
           (const CandEntry *)w.cand.p, (const uint32_t *)w.cand_n.p,
           (const unsigned long long *)w.cand_thr.p, (uint32_t)grid, Bmax, pc.cap_u, ks, ko,
