@@ -386,75 +386,6 @@ __device__ void bitonic_sort_desc(uint64_t *v, uint32_t n_pow2) {
   __syncthreads();
 }
 
-// ---------------------------------------------- histogram threshold (K-th bound)
-// hist_c[256] counts candidates by the top 8 bits of ord(score), hist_f[65536]
-// by the top 16 bits.  Every counted candidate is a distinct ad, so if at
-// least K counted candidates have ord(score) >= T, the K-th best score
-// overall is >= T and anything below T can be dropped.  Returns the largest
-// such T of the form (coarse, fine) << 16, as a key threshold (T << 32), or 0.
-// Counts only grow, so racy snapshots give a smaller, still valid, bound.
-// Called by one full warp.
-__device__ __forceinline__ uint64_t hist_threshold(const uint32_t *hist_c, const uint32_t *hist_f,
-                                                   uint32_t K) {
-  const int lane = threadIdx.x & 31;
-  uint32_t c[8], tot = 0;
-#pragma unroll
-  for (int e = 0; e < 8; e++) {
-    c[e] = __ldcg(hist_c + 255 - 8 * lane - e);
-    tot += c[e];
-  }
-  uint32_t incl = tot;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const uint32_t v = __shfl_up_sync(0xffffffffu, incl, o);
-    if (lane >= o) incl += v;
-  }
-  int cb = -1;
-  uint32_t above_c = 0;
-  {
-    uint32_t acc = incl - tot;
-    int found = -1;
-    uint32_t fa = 0;
-#pragma unroll
-    for (int e = 0; e < 8; e++) {
-      if (found < 0 && acc < K && K <= acc + c[e]) {
-        found = 255 - 8 * lane - e;
-        fa = acc;
-      }
-      acc += c[e];
-    }
-    const uint32_t bal = __ballot_sync(0xffffffffu, found >= 0);
-    if (!bal) return 0ull;
-    const int src = __ffs(bal) - 1;
-    cb = __shfl_sync(0xffffffffu, found, src);
-    above_c = __shfl_sync(0xffffffffu, fa, src);
-  }
-  const uint32_t *hf = hist_f + (uint32_t)cb * 256u;
-  tot = 0;
-#pragma unroll
-  for (int e = 0; e < 8; e++) {
-    c[e] = __ldcg(hf + 255 - 8 * lane - e);
-    tot += c[e];
-  }
-  incl = tot;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const uint32_t v = __shfl_up_sync(0xffffffffu, incl, o);
-    if (lane >= o) incl += v;
-  }
-  uint32_t acc = above_c + incl - tot;
-  int found = -1;
-#pragma unroll
-  for (int e = 0; e < 8; e++) {
-    if (found < 0 && acc < K && K <= acc + c[e]) found = 255 - 8 * lane - e;
-    acc += c[e];
-  }
-  const uint32_t bal = __ballot_sync(0xffffffffu, found >= 0);
-  if (!bal) return ((uint64_t)((uint32_t)cb << 24)) << 32;  // coarse bound only
-  const int fb = __shfl_sync(0xffffffffu, found, __ffs(bal) - 1);
-  return ((uint64_t)(((uint32_t)cb << 24) | ((uint32_t)fb << 16))) << 32;
-}
-
 // Candidate-score histogram shared by all CTAs (for a global K-th bound):
 // bins are the top 11 bits of the order-preserving score key (sign, 8
 // exponent bits, 2 mantissa bits).  CTAs count in shared memory and add
