@@ -89,7 +89,9 @@ typedef struct {
  * or raw user features) read the forward table beside the embeddings (an index
  * whose key counts differ too much within runs, or with 2^24 keys, has none and
  * they walk the window-major view instead); sparse key lists walk the key-major
- * arrays with Algorithm 2.
+ * arrays with Algorithm 2.  The forward table takes 2 or 3 bytes per posting and up to
+ * about as much again in padding (not part of ebr_index_info's sizes); a build that
+ * finds no memory for it is done without.
  *
  * Build the compressed inverted list of Algorithm 1 (Block Grouping by
  * ad >> 8, Logarithmic Categorization into groups g = ceil(log2 n) = 0..8,

@@ -388,7 +388,8 @@ struct BatchSmem {
 // Only bins that umap says are in use are read: the 8192 bins are spaced by
 // exponent, and where fewer ads than kscan pass a bitmap, the walk from the top
 // through the empty ones around zero took 300 us at the end of every CTA
-// (195 users x 85k BF16 ads, 64 of them with bitmaps: scan 1307 us, now 395).
+// (195 users x 85k BF16 ads, 64 of them with bitmaps: scan 1307 us; 290 with this
+// and the grid of batch_grid).
 __device__ __forceinline__ void raise_threshold(const BatchArgs &a, BatchSmem &sm, uint32_t g0,
                                                 uint32_t b) {
   const uint32_t need = __ldg(a.kscan + g0 + b);
@@ -1901,7 +1902,8 @@ int batch_launch(ebr_index *ix, const ebr_cross *cross, const ebr_query *q, uint
     EBR_TRY(launch_quantize((const float *)w.users_f32.p, (uint64_t)Bp * d, EBR_BF16,
                             w.users_bf16.p, st));
   EBR_TRY(expand_transposed(cross, (const uint32_t *)w.user_vals.p, d_uptr, d_base, B, Bp,
-                            (float *)w.wT.p, &ctrl->flags, st, nullptr, ix->key_id));
+                            (float *)w.wT.p, &ctrl->flags, ix->num_sms, st, nullptr,
+                            ix->key_id));
   EBR_CUDA_TRY(clear_zero_rows(ix, w, Bp, st));
   BatchArgs a;
   EBR_TRY(fill_batch_args(ix, B, pl, w, kk, has_filter, ctrl, nullptr, &a));
@@ -2313,8 +2315,8 @@ int loop_build(ebr_index *ix, const ebr_cross *cross, uint32_t max_user_vals, Ba
                            w.users_bf16.p, st);
     if (rc == EBR_OK)
       rc = expand_transposed(cross, (const uint32_t *)w.user_vals.p, d_uptr, d_base,
-                             std::min(Bmax, Bp), Bp, (float *)w.wT.p, &L.ctrl->flags, st, B_dev,
-                             ix->key_id);
+                             std::min(Bmax, Bp), Bp, (float *)w.wT.p, &L.ctrl->flags,
+                             ix->num_sms, st, B_dev, ix->key_id);
     if (rc == EBR_OK) e = clear_zero_rows(ix, w, Bp, st);
     if (rc == EBR_OK && e == cudaSuccess) e = cudaMemsetAsync(w.uhist.p, 0, user_hist_bytes(Bmax), st);
     if (rc == EBR_OK && e == cudaSuccess) {

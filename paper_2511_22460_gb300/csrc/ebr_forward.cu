@@ -12,9 +12,10 @@
 // block is decoded, nothing is added in shared memory and no warp waits for
 // another one's part, which is what bounded the block-wise decode
 // (k_fused_window, ebr_fused.cu: 10.2 k warp instructions per 256 ads of 16
-// keys, 5.1 k here, waits included).  The integer sums and the order of the
-// inner product's additions are the block-wise scan's, so the scores are the
-// same bits.
+// keys, 5.1 k here, waits included).  The integer sums are the block-wise scan's
+// bits, and so are the whole scores of FP32 rows (their additions are in its
+// order, but for the TREE form); BF16 and FP8 rows are summed on the tensor
+// pipe, no further off than by its FP32 multiply-adds (kChain).
 //
 // One persistent CTA per SM over a contiguous range of ads:
 //   producer (1 warp): stages of 32 to 256 ads -- their embedding rows and
@@ -29,10 +30,11 @@
 //   threshold (1 warp): adds the CTA's candidate counts to the histogram all
 //       CTAs share and raises the CTA's running threshold from it.
 // The table names keys by popularity rank, and the terms of the first 8 k ranks
-// (0.90 of the gathers of the 2M-ad inventory) are copied to shared memory: gathers of hot terms from global memory all went to the same few L2
-// slices (ncu, 2M ads: the busiest slice at 82 % of its tag rate, the average
-// at 38 %; 39 and 30 % now), and a shared-memory gather of 32 random words
-// takes about four cycles.
+// (0.90 of the gathers of the 2M-ad inventory) are copied to shared memory:
+// gathers of hot terms from global memory all went to the same few L2 slices
+// (ncu, 2M ads: the busiest slice at 82 % of its tag rate, the average at 38 %;
+// 39 and 30 % now), and a shared-memory gather of 32 random words takes about
+// four cycles.
 // What bounds it: 2M FP32 ads (512 MB of rows, 97 MB of keys) the stream, 111 us
 // = 5.5 TB/s (the block-wise scan: 152 us); 10M FP8 ads with 32 keys each (1.32
 // GB) instruction issue, 72 % of the slots, 298 us (block-wise: 814 us).
@@ -52,8 +54,9 @@ namespace ebr {
 namespace {
 
 // Consumer warps, and the quads of a run whose keys are read into registers at
-// once.  FP32 rows keep 64 registers of h_u per thread, BF16 and FP8 rows (on
-// mma.sync) 8 or 16.  Measured scans: 2M FP32 ads (d = 64, 16 keys) 8 warps 111
+// once.  FP32 rows of 64 and 128 elements keep 64 registers of h_u per thread
+// (narrower ones d of them; they have the same eight warps, not tuned apart), BF16
+// and FP8 rows (on mma.sync) 8 or 16.  Measured scans: 2M FP32 ads (d = 64, 16 keys) 8 warps 111
 // us, 10 warps 113-134 us, 14 warps 183 us (they spill); 1M BF16 ads (d = 128,
 // 24 keys) 14 warps keeping 8 quads 70 us, 18 keeping 4 77 us; 10M FP8 ads (d =
 // 64, 32 keys) 22 warps 302 us, 18 313 us, 14 345 us.

@@ -245,7 +245,8 @@ bool fused_fits(const ebr_index *ix, uint32_t k);
 // 1000 32.0 and 27.6 (one CTA reads all the keys), so the line is in between.
 constexpr uint32_t kDirectAds = 12 * 1024;
 // One launch of the scan over the forward key table (ebr_forward.cu): the
-// counterpart of the block-wise fused scan, with the same results.
+// counterpart of the block-wise fused scan (the same wide terms, and with FP32
+// tables the same scores, bit for bit).
 struct FwdCall {
   ebr_dtype dtype;
   bool direct;               // every ad's key to cand_out[ad] (0: filtered out), no selection
@@ -311,11 +312,12 @@ int launch_quantize_rows_fp8(const float *x, uint64_t n, uint32_t d, uint8_t *q,
 // uptr/base null: users[b * f_u + i]; else user b's field i holds
 // users[base[b] + uptr[b][i] .. base[b] + uptr[b][i + 1]) (checked offsets).
 // batch_dev (optional): the users of this wave, read on the device (<= batch).
-// key_id (optional): the row of each key (the forward table's ids).
+// key_id (optional): the row of each key (the forward table's ids).  sms: SMs
+// of the device.
 int expand_transposed(const ebr_cross *c, const uint32_t *users, const uint32_t *uptr,
                       const uint32_t *base, uint32_t batch, uint32_t Bp, float *wT,
-                      uint32_t *flags, cudaStream_t st, const uint32_t *batch_dev = nullptr,
-                      const uint32_t *key_id = nullptr);
+                      uint32_t *flags, int sms, cudaStream_t st,
+                      const uint32_t *batch_dev = nullptr, const uint32_t *key_id = nullptr);
 // Batched tensor-core path; returns EBR_EINVAL (nothing launched) when the
 // batch does not qualify, so the caller can fall back to per-request scans.
 bool batch_qualifies(const ebr_index *ix, const ebr_cross *cross, const ebr_query *q,

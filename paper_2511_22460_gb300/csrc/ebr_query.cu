@@ -327,7 +327,14 @@ constexpr int kWideTile = kWideThreads * kWideUPT;  // units per tile
 // [seg_e, seg_e + units_e) of the whole query.  route_units != 0: choose the
 // traversal of a sparse list on the device (ctrl->route): the window-major
 // decode when the list's work units reach 1/kRouteRatio of the whole
-// index's, where Algorithm 2's scatter costs more than decoding every window.
+// index's, where Algorithm 2's scatter costs more than reading every ad's keys.
+// The ratio was set for the block-wise scan.  With the forward table, requests on
+// FP32 ads of 16 keys (K = 100, keys drawn by list length), in us by scatter, by
+// reading every ad's keys, by this rule: 2M ads, 30 keys 129, 134, 135; 60 keys 149,
+// 135, 156; 100 keys 159, 136, 138; 300 keys 192, 134, 141; 10M ads, 30 keys 488,
+// 495, 493; 60 keys 526, 494, 532; 100 keys 623, 494, 506; 200k ads, 3 keys 56, 52,
+// 63.  The two cross between 30 and 60 keys and the rule turns by 100, so a
+// larger ratio would serve the lists in between better.
 constexpr unsigned long long kRouteRatio = 8;
 
 __global__ void k_wide_compact(IndexView ix, const uint32_t *__restrict__ q_key,
@@ -1102,10 +1109,14 @@ static int run_wide(ebr_index *ix, const uint32_t *q_key, const float *q_w, uint
 // every field holds one value, users[b * f_u + i].  Pairs are summed in pair
 // order and a field's values in their order, as in the single-request
 // expansion, so both give the same FP32 w^.
-// A CTA takes 32 keys of one field for a group of 64 users, a thread eight of
-// them for one user: a pair and its user value are read once for eight hashes
-// and gathers, which do not wait for one another.  With a thread per (key,
-// user) the instructions around each gather bounded it.  Measured, REPLACE_EXP
+// A CTA takes 4 kExpKeys keys of one field for a group of 64 users, a thread
+// kExpKeys of them for one user: with eight, a pair and its user value are read
+// once for eight hashes and gathers, which do not wait for one another.  With a
+// thread per (key, user) the instructions around each gather bounded it.
+// Measured with the staging, one key a thread and eight: 128 users, 32 fields 833
+// and 472 us; 256 users, 24 fields 833 and 660.  Key spaces too small to fill the
+// device with eight keys a thread take one (staging of such a batch 75 us, with
+// eight 125).
 constexpr int kExpThreads = 256;
 constexpr uint32_t exp_tile(uint32_t keys) { return kExpThreads / 64 * keys; }
 template <bool MULTI, bool HASHED, uint32_t kExpKeys>
@@ -1206,13 +1217,14 @@ constexpr size_t kExpandSmemMax = 200 * 1024;  // pair lists a CTA of the expans
 
 int expand_transposed(const ebr_cross *c, const uint32_t *users, const uint32_t *uptr,
                       const uint32_t *base, uint32_t batch, uint32_t Bp, float *wT,
-                      uint32_t *flags, cudaStream_t st, const uint32_t *batch_dev,
+                      uint32_t *flags, int sms, cudaStream_t st, const uint32_t *batch_dev,
                       const uint32_t *key_id) {
   const CrossView cv = cross_view(c);
   const uint64_t groups = Bp / 64;
-  const bool few = (cv.n_keys / exp_tile(8) + cv.f_a) * groups < 152 * 8;
+  const uint64_t fill = (uint64_t)sms * 8;  // CTAs that fill the device
+  const bool few = (cv.n_keys / exp_tile(8) + cv.f_a) * groups < fill;
   const uint64_t tiles = (cv.n_keys / exp_tile(few ? 1 : 8) + cv.f_a) * groups;  // or fewer
-  const uint32_t blocks = (uint32_t)std::min<uint64_t>(tiles, 152 * 8);
+  const uint32_t blocks = (uint32_t)std::min<uint64_t>(tiles, fill);
   const size_t smem = (size_t)2 * (c->f_a + 1) * 4;
   auto pick = [&](auto multi, auto hashed) {
     constexpr bool M = decltype(multi)::value, H = decltype(hashed)::value;
@@ -1355,7 +1367,7 @@ int query_one(const ebr_index *cix, const ebr_cross *cross, const ebr_query &q, 
                          (uint64_t *)w.cand.p, ctrl, nullptr, quant ? (float *)w.wide.p : nullptr,
                          ws_hist(w), ix->num_sms * kMaxCtasPerSm, st, wmax_ready,
                          nullptr, nullptr, &nl, cta_cand, cta_entries, direct));
-    ix->launches += nl;  // (k_absmax, k_pack) k_fused_window
+    ix->launches += nl;  // (k_absmax, k_pack) and the scan
   } else {
     float *w_dense = auto_route ? (float *)w.w_dense.p : nullptr;
     if (auto_route) EBR_CUDA_TRY(cudaMemsetAsync(w_dense, 0, (size_t)ix->n_keys * 4, st));
@@ -1379,7 +1391,7 @@ int query_one(const ebr_index *cix, const ebr_cross *cross, const ebr_query &q, 
                            !auto_route || planned, (const float *)w.wide.p,
                            auto_route ? &ctrl->route : nullptr, &nl, cta_cand, cta_entries,
                            direct));
-      ix->launches += nl;  // (k_absmax, k_pack) k_fused_window
+      ix->launches += nl;  // (k_absmax, k_pack) and the scan
 
     } else {
       ScanArgs a;
