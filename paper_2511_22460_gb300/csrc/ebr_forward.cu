@@ -163,10 +163,12 @@ __device__ __forceinline__ uint32_t piece_bf16(float h, int n) {
   }
   return bits;
 }
+template <int PIECES>
 __device__ __forceinline__ uint32_t piece_f16(float h, int n) {
   float r = h;
   uint32_t bits = 0;
-  for (int i = 0; i < 8; i++) {
+#pragma unroll
+  for (int i = 0; i < PIECES; i++) {
     const __half x = __float2half_rn(r);
     if (i == n) bits = (uint32_t)__half_as_ushort(x);
     r = fabsf(h) < INFINITY ? (r - __half2float(x)) * 2048.f : 0.f;
@@ -416,35 +418,49 @@ __global__ void __launch_bounds__((cons_warps<Elt>() + 2) * 32, 1)
     }
   } else {
     float sc = 1.f, inv = 1.f;
+    bool spread = false;  // elements that three FP16 pieces do not hold
     if (kF8) {  // the largest finite |h_u| to [1, 4); both powers of two are normal numbers
-      float mx = 0.f;
+      float mx = 0.f, mn = INFINITY;
       for (int i = lane; i < D; i += 32) {
         const float x = fabsf(s_h[i]);
         mx = fmaxf(mx, x < INFINITY ? x : 0.f);
+        mn = fminf(mn, x > 0.f ? x : INFINITY);
       }
-      for (int o = 16; o; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+      for (int o = 16; o; o >>= 1) {
+        mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+        mn = fminf(mn, __shfl_xor_sync(0xffffffffu, mn, o));
+      }
       const int e = mx > 0.f ? max(-126, min(126, (int)(__float_as_uint(mx) >> 23) - 127)) : 0;
       sc = pow2f(-e);
       inv = pow2f(e);
+      spread = mn * sc < pow2f(-22);
     }
     const int t = lane & 3, n = lane >> 2;
     // FP8: column n weighs inv x 2^-11n, down to 0 where a piece has nothing left
     cw0 = kF8 ? inv : (t < 2 ? 1.f : 0.f);
     for (int i = 0; kF8 && i < 2 * t; i++) cw0 *= pow2f(-11);
     cw1 = kF8 ? cw0 * pow2f(-11) : (t == 0 ? 1.f : 0.f);
+    auto split = [&](auto pieces) {
+      constexpr int P = decltype(pieces)::value;
 #pragma unroll
-    for (int j = 0; j < Sh::kSteps; j++)
+      for (int j = 0; j < Sh::kSteps; j++)
 #pragma unroll
-      for (int i = 0; i < Sh::kMmas * 2; i++) {
-        const int c = 4 * j + t;
-        uint32_t w = 0;
-        if (c < Sh::kChunks) {
-          const float x = s_h[c * Tr::kVec + 2 * i] * sc, y = s_h[c * Tr::kVec + 2 * i + 1] * sc;
-          w = kF8 ? piece_f16(x, n) | (piece_f16(y, n) << 16)
-                  : piece_bf16(x, n) | (piece_bf16(y, n) << 16);
+        for (int i = 0; i < Sh::kMmas * 2; i++) {
+          const int c = 4 * j + t;
+          uint32_t w = 0;
+          if (c < Sh::kChunks) {
+            const float x = s_h[c * Tr::kVec + 2 * i] * sc, y = s_h[c * Tr::kVec + 2 * i + 1] * sc;
+            w = kF8 ? piece_f16<P>(x, n) | (piece_f16<P>(y, n) << 16)
+                    : piece_bf16(x, n) | (piece_bf16(y, n) << 16);
+          }
+          breg[j * Sh::kMmas * 2 + i] = w;
         }
-        breg[j * Sh::kMmas * 2 + i] = w;
-      }
+    };
+    // (all eight for every vector: 827k FP8 ads of 128 elements 72.2 -> 75.8 us)
+    if (kF8 && spread)
+      split(std::integral_constant<int, 8>());
+    else
+      split(std::integral_constant<int, 3>());
   }
   pdl_wait();  // the packed terms, their exponent and the route are visible from here on
   const bool pre = a.wide_in != nullptr && !(a.route && *a.route);
