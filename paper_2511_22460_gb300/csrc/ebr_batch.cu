@@ -1708,15 +1708,12 @@ static int stage(void *dst, const void *src, size_t bytes, int io, cudaStream_t 
   return EBR_OK;
 }
 
-// The last row of every group's slice of w^T: the lists' padding key.  (One
-// call per group: a slice may be longer than a 2-D memset's pitch, 2^31 - 1.)
+// The last row of every group's slice of w^T: the lists' padding key.  (The pitch
+// may pass 2^31 bytes, 8.4 M keys: unlike a 2-D copy's it is not limited.)
 static cudaError_t clear_zero_rows(const ebr_index *ix, BatchWs &w, uint32_t Bq, cudaStream_t st) {
-  const size_t row = kGroup * 4, slice = ((size_t)ix->n_keys + 1) * row;
-  for (uint32_t g = 0; g < Bq / kGroup; g++) {
-    const cudaError_t e = cudaMemsetAsync((char *)w.wT.p + (g + 1) * slice - row, 0, row, st);
-    if (e != cudaSuccess) return e;
-  }
-  return cudaSuccess;
+  const size_t slice = ((size_t)ix->n_keys + 1) * kGroup * 4;
+  return cudaMemset2DAsync((char *)w.wT.p + (size_t)ix->n_keys * kGroup * 4, slice, 0, kGroup * 4,
+                           Bq / kGroup, st);
 }
 
 static void (*window_kernel(bool f8, int mode))(BatchArgs) {
